@@ -135,6 +135,7 @@ template <int G>
 __global__ void k_mf_vertex64(int N, const int32_t *vorder, const int64_t *vptr,
                               const int32_t *vrow, const double *ginc, const double *w,
                               const double *x, double *u, const PcgScalars *sc) {
+  chain_wait();
   if (sc && is_done(sc)) return;
   mf_vertex64_rows<G>(HW_WARPS, N, vorder, vptr, vrow, ginc, w, x, u);
 }
@@ -182,6 +183,7 @@ template <int G>
 __global__ void __launch_bounds__(256, 8)
     k_mf_vertex32(int N, const int32_t *vorder, const int64_t *vptr, const float4 *ginc,
                   const float *w, const float *x, float *u, const PcgScalars *sc) {
+  chain_wait();
   if (sc && is_done(sc)) return;
   mf_vertex32_rows<G>(HW_WARPS, N, vorder, vptr, ginc, w, x, u);
 }
@@ -333,6 +335,7 @@ __global__ void k_mf_vertex_df(int N, const int32_t *vorder, const int64_t *vptr
                                const float4 *ginc, const float *glo, const float *wh,
                                const float *wl, const float2 *x, float *uh, float *ul,
                                const PcgScalars *sc) {
+  chain_wait();
   if (sc && is_done(sc)) return;
   mf_vertex_df_rows<G>(HW_WARPS, N, vorder, vptr, ginc, glo, wh, wl, x, uh, ul);
 }
@@ -344,6 +347,7 @@ __global__ void __launch_bounds__(256, 4) k_mf_row_df(int E, int m, const int32_
                             const float *gdh, const float *gdl, const float *gth,
                             const float *gtl, const float *uh, const float *ul, const float *ath,
                             const float *atl, const float2 *p, double *q, DotCtx c) {
+  chain_wait();
   if (is_done(c.sc)) return;
   DF dot{0.f, 0.f};
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < m;
@@ -484,6 +488,7 @@ __global__ void k_mf_row(int E, int m, const int32_t *edge, const int32_t *tet, 
                          const T *gt, const T *u, const T *at, const T *x, const T *b,
                          const T *dinv, T omega, T *out, DotCtx c, double *z = nullptr,
                          const double *rr = nullptr, const int32_t *pos = nullptr) {
+  chain_wait();
   if (is_done(c.sc)) return;
   mf_row_body<T, MODE>(blockIdx.x, gridDim.x, E, m, edge, tet, gd, gt, u, at, x, b, dinv, omega,
                        out, c, z, rr, pos);
@@ -718,18 +723,18 @@ mgpbd_status mf_cohort_step(int which, int sel, const CohortMember *d_mem,
 static mgpbd_status mf_vertex(Handle *h, const double *x, int G = 0, bool check_done = true) {
   if (G == 0) G = h->force_vert64 ? h->force_vert64 : h->mf_g64;
   const PcgScalars *sc = check_done ? h->sc : nullptr;
-  MF_G_DISPATCH(G, (k_mf_vertex64<GG><<<mf_vertex_blocks(h, GG), 256, 0, h->stream>>>(
-                       h->N, h->vorder, h->vptr, h->vrow, h->ginc64, h->w, x, h->u64, sc)));
-  MG_LAUNCH("k_mf_vertex64");
+  MF_G_DISPATCH(G, MG_TRY(chain_launch(h, "k_mf_vertex64", k_mf_vertex64<GG>,
+                                        mf_vertex_blocks(h, GG), 256, h->N, h->vorder, h->vptr,
+                                        h->vrow, h->ginc64, h->w, x, h->u64, sc)));
   return MGPBD_OK;
 }
 
 static mgpbd_status mf_vertex(Handle *h, const float *x, int G = 0, bool check_done = true) {
   if (G == 0) G = h->force_vert32 ? h->force_vert32 : h->mf_g32;
   const PcgScalars *sc = check_done ? h->sc : nullptr;
-  MF_G_DISPATCH(G, (k_mf_vertex32<GG><<<mf_vertex_blocks(h, GG), 256, 0, h->stream>>>(
-                       h->N, h->vorder, h->vptr, h->ginc4, h->w32, x, h->u32, sc)));
-  MG_LAUNCH("k_mf_vertex32");
+  MF_G_DISPATCH(G, MG_TRY(chain_launch(h, "k_mf_vertex32", k_mf_vertex32<GG>,
+                                        mf_vertex_blocks(h, GG), 256, h->N, h->vorder, h->vptr,
+                                        h->ginc4, h->w32, x, h->u32, sc)));
   return MGPBD_OK;
 }
 
@@ -738,10 +743,10 @@ static mgpbd_status mf_vertex(Handle *h, const float *x, int G = 0, bool check_d
 static mgpbd_status mf_vertex(Handle *h, const float2 *x, int G = 0, bool check_done = true) {
   if (G == 0) G = h->force_vert64 ? h->force_vert64 : h->mf_g64;
   const PcgScalars *sc = check_done ? h->sc : nullptr;
-  MF_G_DISPATCH(G, (k_mf_vertex_df<GG><<<mf_vertex_blocks(h, GG), 256, 0, h->stream>>>(
-                       h->N, h->vorder, h->vptr, h->ginc4, h->ginc_lo, h->w32, h->w_lo, x,
-                       h->u_hi, h->u_lo, sc)));
-  MG_LAUNCH("k_mf_vertex_df");
+  MF_G_DISPATCH(G, MG_TRY(chain_launch(h, "k_mf_vertex_df", k_mf_vertex_df<GG>,
+                                        mf_vertex_blocks(h, GG), 256, h->N, h->vorder, h->vptr,
+                                        h->ginc4, h->ginc_lo, h->w32, h->w_lo, x, h->u_hi, h->u_lo,
+                                        sc)));
   return MGPBD_OK;
 }
 
@@ -786,19 +791,17 @@ mgpbd_status mf_apply_pq_form(Handle *h, bool pairs, const double *p, double *q,
     MG_TRY(mf_vertex(h, (const float2 *)h->p_df));
     const int grid =
         std::min(mf_grid(h->m, 256), wave_blocks((const void *)k_mf_row_df, 256));
-    k_mf_row_df<<<grid, 256, 0, h->stream>>>(h->E, h->m, h->edge, h->tet, h->gd32, h->gd_lo,
-                                             h->gt32, h->gt_lo, h->u_hi, h->u_lo, h->at32,
-                                             h->at_lo, h->p_df, q, c);
-    MG_LAUNCH("k_mf_row_df(A.p)");
+    MG_TRY(chain_launch(h, "k_mf_row_df(A.p)", k_mf_row_df, grid, 256, h->E, h->m, h->edge, h->tet,
+                        h->gd32, h->gd_lo, h->gt32, h->gt_lo, h->u_hi, h->u_lo, h->at32, h->at_lo,
+                        h->p_df, q, c));
     return MGPBD_OK;
   }
   MG_TRY(mf_vertex(h, p));
   const int grid = std::min(mf_grid(h->m, 256),
                             wave_blocks((const void *)k_mf_row<double, MF_APPLY_DOT>, 256));
-  k_mf_row<double, MF_APPLY_DOT><<<grid, 256, 0, h->stream>>>(
-      h->E, h->m, h->edge, h->tet, h->gd, h->gt, h->u64, h->alpha_t, p, nullptr, nullptr, 0.0, q,
-      c);
-  MG_LAUNCH("k_mf_row(A.p)");
+  MG_TRY(chain_launch(h, "k_mf_row(A.p)", k_mf_row<double, MF_APPLY_DOT>, grid, 256, h->E, h->m,
+                      h->edge, h->tet, h->gd, h->gt, h->u64, h->alpha_t, p, nullptr, nullptr, 0.0,
+                      q, c, nullptr, nullptr, nullptr));
   return MGPBD_OK;
 }
 
@@ -812,9 +815,9 @@ mgpbd_status mf_residual64(Handle *h, const double *x, const double *b, double *
   MG_TRY(mf_vertex(h, x, 0, false));
   DotCtx c{};
   c.sc = h->sc;
-  k_mf_row<double, MF_RESID><<<mf_grid(h->m, 256), 256, 0, h->stream>>>(
-      h->E, h->m, h->edge, h->tet, h->gd, h->gt, h->u64, h->alpha_t, x, b, nullptr, 0.0, r, c);
-  MG_LAUNCH("k_mf_row(b - A x)");
+  MG_TRY(chain_launch(h, "k_mf_row(b - A x)", k_mf_row<double, MF_RESID>, mf_grid(h->m, 256), 256,
+                      h->E, h->m, h->edge, h->tet, h->gd, h->gt, h->u64, h->alpha_t, x, b, nullptr,
+                      0.0, r, c, nullptr, nullptr, nullptr));
   return MGPBD_OK;
 }
 
@@ -837,19 +840,21 @@ mgpbd_status mf_level0<float>(Handle *h, int mode, const float *x, const float *
   DotCtx c{};
   c.sc = h->sc;
   if (mode == MF_SWEEP)
-    k_mf_row<float, MF_SWEEP><<<mf_grid(h->m, 256), 256, 0, h->stream>>>(
-        h->E, h->m, h->edge, h->tet, h->gd32, h->gt32, h->u32, h->at32, x, b, dinv, omega, out, c);
+    MG_TRY(chain_launch(h, "k_mf_row(f32)", k_mf_row<float, MF_SWEEP>, mf_grid(h->m, 256), 256,
+                        h->E, h->m, h->edge, h->tet, h->gd32, h->gt32, h->u32, h->at32, x, b, dinv,
+                        omega, out, c, nullptr, nullptr, nullptr));
   else if (mode == MF_APPLY)
-    k_mf_row<float, MF_APPLY><<<mf_grid(h->m, 256), 256, 0, h->stream>>>(
-        h->E, h->m, h->edge, h->tet, h->gd32, h->gt32, h->u32, h->at32, x, b, dinv, omega, out, c);
+    MG_TRY(chain_launch(h, "k_mf_row(f32)", k_mf_row<float, MF_APPLY>, mf_grid(h->m, 256), 256,
+                        h->E, h->m, h->edge, h->tet, h->gd32, h->gt32, h->u32, h->at32, x, b, dinv,
+                        omega, out, c, nullptr, nullptr, nullptr));
   else if (mode == MF_RESID_MEMBER)
-    k_mf_row<float, MF_RESID_MEMBER><<<mf_grid(h->m, 256), 256, 0, h->stream>>>(
-        h->E, h->m, h->edge, h->tet, h->gd32, h->gt32, h->u32, h->at32, x, b, dinv, omega, out, c,
-        nullptr, nullptr, h->lev[0].mpos);
+    MG_TRY(chain_launch(h, "k_mf_row(f32)", k_mf_row<float, MF_RESID_MEMBER>, mf_grid(h->m, 256),
+                        256, h->E, h->m, h->edge, h->tet, h->gd32, h->gt32, h->u32, h->at32, x, b,
+                        dinv, omega, out, c, nullptr, nullptr, h->lev[0].mpos));
   else
-    k_mf_row<float, MF_RESID><<<mf_grid(h->m, 256), 256, 0, h->stream>>>(
-        h->E, h->m, h->edge, h->tet, h->gd32, h->gt32, h->u32, h->at32, x, b, dinv, omega, out, c);
-  MG_LAUNCH("k_mf_row(f32)");
+    MG_TRY(chain_launch(h, "k_mf_row(f32)", k_mf_row<float, MF_RESID>, mf_grid(h->m, 256), 256,
+                        h->E, h->m, h->edge, h->tet, h->gd32, h->gt32, h->u32, h->at32, x, b, dinv,
+                        omega, out, c, nullptr, nullptr, nullptr));
   return MGPBD_OK;
 }
 
@@ -860,19 +865,21 @@ mgpbd_status mf_level0<double>(Handle *h, int mode, const double *x, const doubl
   DotCtx c{};
   c.sc = h->sc;
   if (mode == MF_SWEEP)
-    k_mf_row<double, MF_SWEEP><<<mf_grid(h->m, 256), 256, 0, h->stream>>>(
-        h->E, h->m, h->edge, h->tet, h->gd, h->gt, h->u64, h->alpha_t, x, b, dinv, omega, out, c);
+    MG_TRY(chain_launch(h, "k_mf_row(f64)", k_mf_row<double, MF_SWEEP>, mf_grid(h->m, 256), 256,
+                        h->E, h->m, h->edge, h->tet, h->gd, h->gt, h->u64, h->alpha_t, x, b, dinv,
+                        omega, out, c, nullptr, nullptr, nullptr));
   else if (mode == MF_APPLY)
-    k_mf_row<double, MF_APPLY><<<mf_grid(h->m, 256), 256, 0, h->stream>>>(
-        h->E, h->m, h->edge, h->tet, h->gd, h->gt, h->u64, h->alpha_t, x, b, dinv, omega, out, c);
+    MG_TRY(chain_launch(h, "k_mf_row(f64)", k_mf_row<double, MF_APPLY>, mf_grid(h->m, 256), 256,
+                        h->E, h->m, h->edge, h->tet, h->gd, h->gt, h->u64, h->alpha_t, x, b, dinv,
+                        omega, out, c, nullptr, nullptr, nullptr));
   else if (mode == MF_RESID_MEMBER)
-    k_mf_row<double, MF_RESID_MEMBER><<<mf_grid(h->m, 256), 256, 0, h->stream>>>(
-        h->E, h->m, h->edge, h->tet, h->gd, h->gt, h->u64, h->alpha_t, x, b, dinv, omega, out, c,
-        nullptr, nullptr, h->lev[0].mpos);
+    MG_TRY(chain_launch(h, "k_mf_row(f64)", k_mf_row<double, MF_RESID_MEMBER>, mf_grid(h->m, 256),
+                        256, h->E, h->m, h->edge, h->tet, h->gd, h->gt, h->u64, h->alpha_t, x, b,
+                        dinv, omega, out, c, nullptr, nullptr, h->lev[0].mpos));
   else
-    k_mf_row<double, MF_RESID><<<mf_grid(h->m, 256), 256, 0, h->stream>>>(
-        h->E, h->m, h->edge, h->tet, h->gd, h->gt, h->u64, h->alpha_t, x, b, dinv, omega, out, c);
-  MG_LAUNCH("k_mf_row(f64)");
+    MG_TRY(chain_launch(h, "k_mf_row(f64)", k_mf_row<double, MF_RESID>, mf_grid(h->m, 256), 256,
+                        h->E, h->m, h->edge, h->tet, h->gd, h->gt, h->u64, h->alpha_t, x, b, dinv,
+                        omega, out, c, nullptr, nullptr, nullptr));
   return MGPBD_OK;
 }
 
@@ -888,15 +895,15 @@ mgpbd_status mf_level0_final(Handle *h, const T *x, const T *b, const T *dinv, T
   DotCtx c = o.c;
   c.sc = h->sc;
   if (o.dot)
-    k_mf_row<T, MF_SWEEP_ZDOT><<<std::min(mf_grid(h->m, 256),
-                                          wave_blocks((const void *)k_mf_row<T, MF_SWEEP_ZDOT>,
-                                                      256)),
-                                 256, 0, h->stream>>>(
-        h->E, h->m, h->edge, h->tet, gd, gt, u, at, x, b, dinv, omega, nullptr, c, o.z, o.r);
+    MG_TRY(chain_launch(h, "k_mf_row(final sweep)", k_mf_row<T, MF_SWEEP_ZDOT>,
+                        std::min(mf_grid(h->m, 256),
+                                 wave_blocks((const void *)k_mf_row<T, MF_SWEEP_ZDOT>, 256)),
+                        256, h->E, h->m, h->edge, h->tet, gd, gt, u, at, x, b, dinv, omega, nullptr,
+                        c, o.z, o.r, nullptr));
   else
-    k_mf_row<T, MF_SWEEP_Z><<<mf_grid(h->m, 256), 256, 0, h->stream>>>(
-        h->E, h->m, h->edge, h->tet, gd, gt, u, at, x, b, dinv, omega, nullptr, c, o.z, o.r);
-  MG_LAUNCH("k_mf_row(final sweep)");
+    MG_TRY(chain_launch(h, "k_mf_row(final sweep)", k_mf_row<T, MF_SWEEP_Z>, mf_grid(h->m, 256),
+                        256, h->E, h->m, h->edge, h->tet, gd, gt, u, at, x, b, dinv, omega, nullptr,
+                        c, o.z, o.r, nullptr));
   return MGPBD_OK;
 }
 

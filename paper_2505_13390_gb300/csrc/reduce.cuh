@@ -196,6 +196,83 @@ __device__ __forceinline__ AT row_dot(const int64_t *ptr, const int32_t *col, co
   return acc;
 }
 
+// The same sum in two halves: row_pre loads the row's extent and the first
+// four entries of each lane (static during a solve), row_fin gathers x and
+// adds them and the rest in the order of row_dot.  In a launch chain row_pre
+// runs before chain_wait, so that the gathers are the only loads behind it;
+// most rows of the coarse levels have at most four entries per lane.
+template <class VT>
+struct RowPre {
+  int64_t k, e;
+  int32_t c[4];
+  VT v[4];
+};
+
+template <int G, class VT>
+__device__ __forceinline__ RowPre<VT> row_pre(const int64_t *ptr, const int32_t *col,
+                                              const VT *val, int64_t i, int g, bool valid) {
+  RowPre<VT> p;
+  p.k = p.e = 0;
+  if (valid) {
+    p.k = ptr[i] + g;
+    p.e = ptr[i + 1];
+  }
+#pragma unroll
+  for (int j = 0; j < 4; ++j)
+    if (p.k + j * G < p.e) {
+      p.c[j] = col[p.k + j * G];
+      p.v[j] = val[p.k + j * G];
+    }
+  return p;
+}
+
+template <int G, class AT, class VT, class XT>
+__device__ __forceinline__ AT row_fin(const RowPre<VT> &p, const int32_t *col, const VT *val,
+                                      const XT *x) {
+  AT acc = 0;
+  XT xv[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j)
+    if (p.k + j * G < p.e) xv[j] = x[p.c[j]];
+#pragma unroll
+  for (int j = 0; j < 4; ++j)
+    if (p.k + j * G < p.e) acc = fma((AT)p.v[j], (AT)xv[j], acc);
+  int64_t k = p.k + 4 * G;
+  for (; k + 3 * G < p.e; k += 4 * G) {
+    const int32_t c0 = col[k], c1 = col[k + G], c2 = col[k + 2 * G], c3 = col[k + 3 * G];
+    const VT v0 = val[k], v1 = val[k + G], v2 = val[k + 2 * G], v3 = val[k + 3 * G];
+    const XT x0 = x[c0], x1 = x[c1], x2 = x[c2], x3 = x[c3];
+    acc = fma((AT)v0, (AT)x0, acc);
+    acc = fma((AT)v1, (AT)x1, acc);
+    acc = fma((AT)v2, (AT)x2, acc);
+    acc = fma((AT)v3, (AT)x3, acc);
+  }
+  for (; k < p.e; k += G) acc = fma((AT)val[k], (AT)x[col[k]], acc);
+  return acc;
+}
+
+// The gate between the loads a kernel may make early and the rest: `open`
+// waits for the chain's predecessor on its first call and reads the solve's
+// done flag beside the loads that follow it; `closed` tells whether the solve
+// has finished (checked before anything is written).  Outside a chain (the
+// cooperative tail, whose blocks have checked already) NoGate does nothing.
+struct ChainGate {
+  const PcgScalars *sc;
+  int state = -1;
+  __device__ __forceinline__ explicit ChainGate(const PcgScalars *s) : sc(s) {}
+  __device__ __forceinline__ void open() {
+    if (state < 0) {
+      chain_wait();
+      state = sc ? ((volatile const PcgScalars *)sc)->done : 0;
+    }
+  }
+  __device__ __forceinline__ bool closed() const { return state != 0; }
+};
+struct NoGate {
+  __device__ __forceinline__ void open() {}
+  __device__ __forceinline__ bool closed() const { return false; }
+};
+
 // Rows handled by G-lane groups, 32/G rows per warp per trip, over warps
 // w0, w0 + nw, ...  The loop bound is uniform across the warp, so full-mask
 // shuffles inside are safe; `valid` marks groups past the last row.  Which

@@ -48,6 +48,7 @@ static DotCtx make_ctx(Handle *h, int mode, double *out = nullptr) {
 // plain vector kernels
 // ---------------------------------------------------------------------------
 __global__ void k_dot(int64_t n, const double *x, const double *y, DotCtx c, int check_done) {
+  chain_wait();
   if (check_done && is_done(c.sc)) return;
   double acc = 0.0;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
@@ -128,6 +129,7 @@ __device__ __forceinline__ void xr_update_body(int vb, int vn, int64_t n, double
 template <class T>
 __global__ void k_xr_update(int64_t n, double *x, double *r, const double *p, const double *q,
                             DotCtx c, T *bl, const T *dinv, T om, T *x0) {
+  chain_wait();
   if (is_done(c.sc)) return;
   xr_update_body<T>(blockIdx.x, gridDim.x, n, x, r, p, q, c, bl, dinv, om, x0);
 }
@@ -137,6 +139,7 @@ __global__ void k_xr_update(int64_t n, double *x, double *r, const double *p, co
 template <class T>
 __global__ void k_top_prep(int64_t n, const double *r, T *bl, const T *dinv, T om, T *x0,
                            const PcgScalars *sc) {
+  chain_wait();
   if (sc && is_done(sc)) return;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
@@ -190,6 +193,7 @@ __device__ __forceinline__ void p_update_body(int vb, int vn, int64_t n, double 
 
 __global__ void k_p_update(int64_t n, double *p, const double *z, const PcgScalars *sc,
                            float2 *pdf) {
+  chain_wait();
   if (is_done(sc)) return;
   p_update_body(blockIdx.x, gridDim.x, n, p, z, sc, pdf);
 }
@@ -213,6 +217,7 @@ __device__ __forceinline__ D convert_to(double v) { return narrow<D>(v); }
 
 template <class S, class D>
 __global__ void k_convert(int64_t n, const S *a, D *b, const PcgScalars *sc) {
+  chain_wait();
   if (sc && is_done(sc)) return;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x)
@@ -226,17 +231,23 @@ __global__ void k_convert(int64_t n, const S *a, D *b, const PcgScalars *sc) {
 template <int G, class VT, class AT>
 __global__ void k_spmv_pq(int n, const int64_t *ptr, const int32_t *col, const VT *val,
                           const double *p, double *q, DotCtx c) {
-  if (is_done(c.sc)) return;
+  ChainGate gate(c.sc);
   double acc = 0.0;
   GROUP_ROWS(G, n) {
-    AT s = valid ? row_dot<G, VT, AT, double>(ptr, col, val, p, (int)i, g) : (AT)0;
+    const RowPre<VT> pre = row_pre<G>(ptr, col, val, i, g, valid);
+    gate.open();
+    const double pi = valid && g == 0 ? p[i] : 0.0;
+    AT s = row_fin<G, AT>(pre, col, val, p);
     s = group_sum<G>(s);
+    if (gate.closed()) break;
     if (valid && g == 0) {
       double qi = (double)s;
       q[i] = qi;
-      acc = fma(p[i], qi, acc);
+      acc = fma(pi, qi, acc);
     }
   }
+  gate.open();  // warps without a row
+  if (gate.closed()) return;
   block_dot_finish(acc, c);
 }
 
@@ -258,6 +269,7 @@ __global__ void k_true_resid(int n, const int64_t *ptr, const int32_t *col, cons
 // weighted Jacobi, first sweep from x = 0: x = omega D^-1 b
 template <class T>
 __global__ void k_jacobi0(int n, const T *b, const T *dinv, T omega, T *x, const PcgScalars *sc) {
+  chain_wait();
   if (is_done(sc)) return;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
     x[i] = omega * (b[i] * dinv[i]);
@@ -269,6 +281,7 @@ template <int G, class T>
 __global__ void k_gs_colour(int nrows, const int32_t *crow, const int64_t *ptr,
                             const int32_t *col, const T *val, const T *dinv, const T *b, T *x,
                             const PcgScalars *sc) {
+  chain_wait();
   if (is_done(sc)) return;
   GROUP_ROWS(G, nrows) {
     int row = valid ? crow[i] : 0;
@@ -282,6 +295,7 @@ __global__ void k_gs_colour(int nrows, const int32_t *crow, const int64_t *ptr,
 template <int G, class T>
 __global__ void k_spmv_plain(int n, const int64_t *ptr, const int32_t *col, const T *val,
                              const T *v, T *y, const PcgScalars *sc) {
+  chain_wait();
   if (is_done(sc)) return;
   GROUP_ROWS(G, n) {
     T s = valid ? row_dot<G, T, T, T>(ptr, col, val, v, (int)i, g) : (T)0;
@@ -295,6 +309,7 @@ __global__ void k_spmv_plain(int n, const int64_t *ptr, const int32_t *col, cons
 template <class T>
 __global__ void k_cheb_start(int n, const T *b, const T *Ax, const T *dinv, T inv_theta, T *r,
                              T *d, T *x, const PcgScalars *sc) {
+  chain_wait();
   if (is_done(sc)) return;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     T ri = (Ax ? b[i] - Ax[i] : b[i]) * dinv[i];  // no Ax: x = 0 on entry
@@ -308,6 +323,7 @@ __global__ void k_cheb_start(int n, const T *b, const T *Ax, const T *dinv, T in
 template <class T>
 __global__ void k_cheb_step(int n, const T *Ad, const T *dinv, T c1, T c2, T *r, T *d, T *x,
                             const PcgScalars *sc) {
+  chain_wait();
   if (is_done(sc)) return;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     T ri = r[i] - Ad[i] * dinv[i];
@@ -319,28 +335,39 @@ __global__ void k_cheb_step(int n, const T *Ad, const T *dinv, T c1, T c2, T *r,
 }
 
 // Row bodies of the CSR-level V-cycle steps, over the warps w0, w0 + nw, ...
-// (a launch's own warps, or every warp of the cooperative coarse tail).
+// (a launch's own warps, or every warp of the cooperative coarse tail); the
+// row's matrix entries are loaded before `gate` opens (reduce.cuh).
 // weighted Jacobi sweep: xn = x + omega D^-1 (b - A x)
-template <int G, class T>
+template <int G, class T, class Gate>
 __device__ __forceinline__ void jacobi_rows(int64_t w0, int64_t nw, int n, const int64_t *ptr,
                                             const int32_t *col, const T *val, const T *dinv,
-                                            T omega, const T *b, const T *x, T *xn) {
+                                            T omega, const T *b, const T *x, T *xn, Gate gate) {
   GROUP_ROWS_OVER(G, n, w0, nw) {
-    T s = valid ? row_dot<G, T, T, T>(ptr, col, val, x, (int)i, g) : (T)0;
+    const RowPre<T> p = row_pre<G>(ptr, col, val, i, g, valid);
+    const bool head = valid && g == 0;
+    const T di = head ? dinv[i] : (T)0;
+    gate.open();
+    const T bi = head ? b[i] : (T)0, xi = head ? x[i] : (T)0;
+    T s = row_fin<G, T>(p, col, val, x);
     s = group_sum<G>(s);
-    if (valid && g == 0) xn[i] = fma(omega, (b[i] - s) * dinv[i], x[i]);
+    if (gate.closed()) return;
+    if (head) xn[i] = fma(omega, (bi - s) * di, xi);
   }
 }
 
 // r = b - A x
-template <int G, class T>
+template <int G, class T, class Gate>
 __device__ __forceinline__ void resid_rows(int64_t w0, int64_t nw, int n, const int64_t *ptr,
                                            const int32_t *col, const T *val, const T *b,
-                                           const T *x, T *r) {
+                                           const T *x, T *r, Gate gate) {
   GROUP_ROWS_OVER(G, n, w0, nw) {
-    T s = valid ? row_dot<G, T, T, T>(ptr, col, val, x, (int)i, g) : (T)0;
+    const RowPre<T> p = row_pre<G>(ptr, col, val, i, g, valid);
+    gate.open();
+    const T bi = valid && g == 0 ? b[i] : (T)0;
+    T s = row_fin<G, T>(p, col, val, x);
     s = group_sum<G>(s);
-    if (valid && g == 0) r[i] = b[i] - s;
+    if (gate.closed()) return;
+    if (valid && g == 0) r[i] = bi - s;
   }
 }
 
@@ -348,38 +375,48 @@ template <int G, class T>
 __global__ void k_jacobi(int n, const int64_t *ptr, const int32_t *col, const T *val,
                          const T *dinv, T omega, const T *b, const T *x, T *xn,
                          const PcgScalars *sc) {
-  if (is_done(sc)) return;
-  jacobi_rows<G, T>(HW_WARPS, n, ptr, col, val, dinv, omega, b, x, xn);
+  jacobi_rows<G, T>(HW_WARPS, n, ptr, col, val, dinv, omega, b, x, xn, ChainGate(sc));
 }
 
 template <int G, class T>
 __global__ void k_resid(int n, const int64_t *ptr, const int32_t *col, const T *val, const T *b,
                         const T *x, T *r, const PcgScalars *sc) {
-  if (sc && is_done(sc)) return;
-  resid_rows<G, T>(HW_WARPS, n, ptr, col, val, b, x, r);
+  resid_rows<G, T>(HW_WARPS, n, ptr, col, val, b, x, r, ChainGate(sc));
 }
 
 // b_c[a*k+c] = sum_{i in a} P_ic r_i (warp per aggregate, k columns of P per
 // aggregate); with xc given, also the coarse level's first Jacobi sweep from
 // zero, xc = omega_c b_c / A_c,diag
-template <class T>
+template <class T, class Gate>
 __device__ __forceinline__ void restrict_aggs(int64_t w, int64_t nw, int na, int k,
                                               const int64_t *mptr, const int32_t *mrow,
                                               const T *P, const T *r, T *bc, const T *dinv_c,
-                                              T om_c, T *xc) {
+                                              T om_c, T *xc, Gate gate) {
   const int lane = threadIdx.x & 31;
   for (int64_t a = w; a < na; a += nw) {
+    const int64_t q0 = mptr[a] + lane, q1 = mptr[a + 1];
     for (int c = 0; c < k; ++c) {
+      const int64_t ac = a * k + c;
+      // the lane's first member and its weight, before the gate
+      int i = 0;
+      T p = 0;
+      if (q0 < q1) {
+        i = mrow[q0];
+        p = P[(int64_t)i * k + c];
+      }
+      const T di = xc && lane == 0 ? dinv_c[ac] : (T)0;
+      gate.open();
       T acc = 0;
-      for (int64_t q = mptr[a] + lane; q < mptr[a + 1]; q += 32) {
-        int i = mrow[q];
+      if (q0 < q1) acc = fma(p, r[i], acc);
+      for (int64_t q = q0 + 32; q < q1; q += 32) {
+        i = mrow[q];
         acc = fma(P[(int64_t)i * k + c], r[i], acc);
       }
       acc = warp_sum(acc);
+      if (gate.closed()) return;
       if (lane == 0) {
-        const int64_t ac = a * k + c;
         bc[ac] = acc;
-        if (xc) xc[ac] = om_c * (acc * dinv_c[ac]);
+        if (xc) xc[ac] = om_c * (acc * di);
       }
     }
   }
@@ -390,16 +427,32 @@ __device__ __forceinline__ void restrict_aggs(int64_t w, int64_t nw, int na, int
 template <class T>
 __global__ void k_restrict_member(int na, const int64_t *mptr, const T *Pm, const T *rm, T *bc,
                                   const PcgScalars *sc, const T *dinv_c, T om_c, T *xc) {
-  if (is_done(sc)) return;
   const int lane = threadIdx.x & 31;
+  ChainGate gate(sc);
   for (int64_t a = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; a < na;
        a += ((int64_t)gridDim.x * blockDim.x) >> 5) {
-    T acc = 0;
-    for (int64_t q = mptr[a] + lane; q < mptr[a + 1]; q += 32) acc = fma(Pm[q], rm[q], acc);
+    // the first three weights of each lane before the gate (the level-0
+    // aggregates of the tet blocks have about eighty members)
+    const int64_t q0 = mptr[a] + lane, q1 = mptr[a + 1];
+    T p[3];
+#pragma unroll
+    for (int j = 0; j < 3; ++j)
+      if (q0 + 32 * j < q1) p[j] = Pm[q0 + 32 * j];
+    const T di = xc && lane == 0 ? dinv_c[a] : (T)0;
+    gate.open();
+    T rv[3], acc = 0;
+#pragma unroll
+    for (int j = 0; j < 3; ++j)
+      if (q0 + 32 * j < q1) rv[j] = rm[q0 + 32 * j];
+#pragma unroll
+    for (int j = 0; j < 3; ++j)
+      if (q0 + 32 * j < q1) acc = fma(p[j], rv[j], acc);
+    for (int64_t q = q0 + 96; q < q1; q += 32) acc = fma(Pm[q], rm[q], acc);
     acc = warp_sum(acc);
+    if (gate.closed()) return;
     if (lane == 0) {
       bc[a] = acc;
-      if (xc) xc[a] = om_c * (acc * dinv_c[a]);
+      if (xc) xc[a] = om_c * (acc * di);
     }
   }
 }
@@ -408,37 +461,39 @@ template <class T>
 __global__ void k_restrict(int na, int k, const int64_t *mptr, const int32_t *mrow, const T *P,
                            const T *r, T *bc, const PcgScalars *sc, const T *dinv_c = nullptr,
                            T om_c = 0, T *xc = nullptr) {
-  if (is_done(sc)) return;
-  restrict_aggs<T>(HW_WARPS, na, k, mptr, mrow, P, r, bc, dinv_c, om_c, xc);
+  restrict_aggs<T>(HW_WARPS, na, k, mptr, mrow, P, r, bc, dinv_c, om_c, xc, ChainGate(sc));
 }
 
 // x_i += P_i x_c[agg_i] (rows left alone have no aggregate); each thread
 // takes four rows a block-width apart so that its loads are in flight together
 constexpr int kProlongRows = 4;
-template <class T>
+template <class T, class Gate>
 __device__ __forceinline__ void prolong_rows(int64_t blk, int64_t nblk, int n, const int32_t *agg,
-                                             const T *P, const T *xc, T *x) {
+                                             const T *P, const T *xc, T *x, Gate gate) {
   const int64_t tile = (int64_t)blockDim.x * kProlongRows;
   for (int64_t base = blk * tile + threadIdx.x; base < n; base += nblk * tile) {
     int a[kProlongRows];
-    T p[kProlongRows], xv[kProlongRows];
+    T p[kProlongRows], xv[kProlongRows], cv[kProlongRows];
 #pragma unroll
     for (int k = 0; k < kProlongRows; ++k) {
       const int64_t i = base + k * (int64_t)blockDim.x;
       a[k] = i < n ? agg[i] : -1;
+      if (i < n) p[k] = P[i];
     }
+    gate.open();
 #pragma unroll
     for (int k = 0; k < kProlongRows; ++k) {
       const int64_t i = base + k * (int64_t)blockDim.x;
       if (a[k] >= 0) {  // left-alone rows: P_i = 0
-        p[k] = P[i];
+        cv[k] = xc[a[k]];
         xv[k] = x[i];
       }
     }
+    if (gate.closed()) return;
 #pragma unroll
     for (int k = 0; k < kProlongRows; ++k) {
       const int64_t i = base + k * (int64_t)blockDim.x;
-      if (a[k] >= 0) x[i] = fma(p[k], xc[a[k]], xv[k]);
+      if (a[k] >= 0) x[i] = fma(p[k], cv[k], xv[k]);
     }
   }
 }
@@ -446,14 +501,14 @@ __device__ __forceinline__ void prolong_rows(int64_t blk, int64_t nblk, int n, c
 template <class T>
 __global__ void k_prolong(int n, const int32_t *agg, const T *P, const T *xc, T *x,
                           const PcgScalars *sc) {  // one column of P per aggregate
-  if (is_done(sc)) return;
-  prolong_rows<T>(blockIdx.x, gridDim.x, n, agg, P, xc, x);
+  prolong_rows<T>(blockIdx.x, gridDim.x, n, agg, P, xc, x, ChainGate(sc));
 }
 
 // x_i += sum_c P_ic x_c[agg_i*k + c], c ascending (k columns of P per aggregate)
 template <class T>
 __global__ void k_prolong_k(int n, int k, const int32_t *agg, const T *P, const T *xc, T *x,
                             const PcgScalars *sc) {
+  chain_wait();
   if (is_done(sc)) return;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
@@ -465,23 +520,38 @@ __global__ void k_prolong_k(int n, int k, const int32_t *agg, const T *P, const 
   }
 }
 
-// coarsest: x = A_c^-1 b with the explicit FP64 inverse (warp per row)
-template <class T>
+// coarsest: x = A_c^-1 b with the explicit FP64 inverse (warp per row); the
+// row's first 256 entries are loaded before the gate
+template <class T, class Gate>
 __device__ __forceinline__ void coarse_rows(int64_t w, int64_t nw, int n, const double *inv,
-                                            const T *b, T *x) {
+                                            const T *b, T *x, Gate gate) {
+  constexpr int kPre = 8;
   const int lane = threadIdx.x & 31;
   for (int64_t i = w; i < n; i += nw) {
+    const double *row = inv + i * (int64_t)n;
+    double a[kPre];
+    T bv[kPre];
+#pragma unroll
+    for (int j = 0; j < kPre; ++j)
+      if (lane + 32 * j < n) a[j] = row[lane + 32 * j];
+    gate.open();
+#pragma unroll
+    for (int j = 0; j < kPre; ++j)
+      if (lane + 32 * j < n) bv[j] = b[lane + 32 * j];
     double acc = 0.0;
-    for (int j = lane; j < n; j += 32) acc = fma(inv[i * (int64_t)n + j], widen(b[j]), acc);
+#pragma unroll
+    for (int j = 0; j < kPre; ++j)
+      if (lane + 32 * j < n) acc = fma(a[j], widen(bv[j]), acc);
+    for (int j = lane + 32 * kPre; j < n; j += 32) acc = fma(row[j], widen(b[j]), acc);
     acc = warp_sum(acc);
+    if (gate.closed()) return;
     if (lane == 0) x[i] = narrow<T>(acc);
   }
 }
 
 template <class T>
 __global__ void k_coarse_apply(int n, const double *inv, const T *b, T *x, const PcgScalars *sc) {
-  if (sc && is_done(sc)) return;
-  coarse_rows<T>(HW_WARPS, n, inv, b, x);
+  coarse_rows<T>(HW_WARPS, n, inv, b, x, ChainGate(sc));
 }
 
 // ---------------------------------------------------------------------------
@@ -717,6 +787,17 @@ static int row_blocks(int64_t rows, int G, int th = 256) {
   return (int)std::max<int64_t>(1, std::min<int64_t>(b, cap));
 }
 
+// grids of the kernels that end in a dot product: one resident wave at most
+template <int G>
+static int spmv_pq_blocks(int m) {
+  return std::min(row_blocks(m, G),
+                  wave_blocks((const void *)k_spmv_pq<G, double, double>, 256));
+}
+template <class T>
+static int xr_blocks(int m) {
+  return std::min(dot_grid(m), wave_blocks((const void *)k_xr_update<T>, kDotThreads));
+}
+
 #define DISPATCH_G(G, ...)                  \
   switch (G) {                              \
     case 4: { constexpr int GG = 4; __VA_ARGS__; } break;   \
@@ -805,33 +886,34 @@ __global__ void __launch_bounds__(256) k_coarse_tail(TailDesc<T> d, unsigned int
     T *x = L.x, *x2 = L.x2;  // x holds the first sweep from zero
     for (int s = 1; s < d.sweeps; ++s) {
       DISPATCH_G(L.G, (jacobi_rows<GG, T>(w0, nw, L.n, L.ptr, L.col, L.val, L.dinv, L.omega,
-                                          L.b, x, x2)));
+                                          L.b, x, x2, NoGate{})));
       if (!sync()) return;
       T *t = x;
       x = x2;
       x2 = t;
     }
-    DISPATCH_G(L.G, (resid_rows<GG, T>(w0, nw, L.n, L.ptr, L.col, L.val, L.b, x, L.r)));
+    DISPATCH_G(L.G, (resid_rows<GG, T>(w0, nw, L.n, L.ptr, L.col, L.val, L.b, x, L.r,
+                                          NoGate{})));
     if (!sync()) return;
     const TailLevel<T> &Lc = d.lev[l + 1];
     const bool c_jac = l + 1 < d.coarsest;  // the coarse level's first sweep rides along
     restrict_aggs<T>(w0, nw, L.n_agg, 1, L.mptr, L.mrow, L.P, L.r, Lc.b,
-                     c_jac ? Lc.dinv : nullptr, Lc.omega, c_jac ? Lc.x : nullptr);
+                     c_jac ? Lc.dinv : nullptr, Lc.omega, c_jac ? Lc.x : nullptr, NoGate{});
     if (!sync()) return;
     cur[l] = x;
   }
   const TailLevel<T> &C = d.lev[d.coarsest];
-  coarse_rows<T>(w0, nw, C.n, d.cinv, C.b, C.x);
+  coarse_rows<T>(w0, nw, C.n, d.cinv, C.b, C.x, NoGate{});
   const T *xc = C.x;
   for (int l = d.coarsest - 1; l >= d.first; --l) {
     if (!sync()) return;
     const TailLevel<T> &L = d.lev[l];
     T *x = cur[l], *x2 = x == L.x ? L.x2 : L.x;
-    prolong_rows<T>(blockIdx.x, gridDim.x, L.n, L.agg, L.P, xc, x);
+    prolong_rows<T>(blockIdx.x, gridDim.x, L.n, L.agg, L.P, xc, x, NoGate{});
     for (int s = 0; s < d.sweeps; ++s) {
       if (!sync()) return;
       DISPATCH_G(L.G, (jacobi_rows<GG, T>(w0, nw, L.n, L.ptr, L.col, L.val, L.dinv, L.omega,
-                                          L.b, x, x2)));
+                                          L.b, x, x2, NoGate{})));
       T *t = x;
       x = x2;
       x2 = t;
@@ -922,12 +1004,12 @@ __global__ void kb_restrict0(const CohortMember *mem, const CohortBlock *blk) {
   const TailLevel<float> &L1 = M.tail.lev[1];
   const bool c_jac = M.tail.coarsest > 1;  // level 1 smooths: its first sweep rides along
   restrict_aggs<float>(VG_WARPS(vb, vn), M.n_agg0, 1, M.mptr0, M.mrow0, M.P0, M.r0, L1.b,
-                       c_jac ? L1.dinv : nullptr, L1.omega, c_jac ? L1.x : nullptr);
+                       c_jac ? L1.dinv : nullptr, L1.omega, c_jac ? L1.x : nullptr, NoGate{});
 }
 
 __global__ void kb_prolong0(const CohortMember *mem, const CohortBlock *blk) {
   COHORT_BLOCK;
-  prolong_rows<float>(vb, vn, M.m, M.agg0, M.P0, M.xc1, M.x20);
+  prolong_rows<float>(vb, vn, M.m, M.agg0, M.P0, M.xc1, M.x20, NoGate{});
 }
 
 __global__ void kb_pupdate(const CohortMember *mem, const CohortBlock *blk) {
@@ -979,16 +1061,17 @@ __global__ void __launch_bounds__(256) kb_tail(const CohortMember *mem, int K, i
   const TailDesc<float> &Tb = mem[kb].tail;
   auto jacobi = [&](const TailLevel<float> &L, const float *x, float *xn) {
     DISPATCH_G(L.G, (jacobi_rows<GG, float>(lw, nlw, L.n, L.ptr, L.col, L.val, L.dinv, L.omega,
-                                            L.b, x, xn)));
+                                            L.b, x, xn, NoGate{})));
   };
   for (int d = 1; d <= maxc; ++d) {
     if (mine && d < ck) jacobi(T.lev[d], T.lev[d].x, T.lev[d].x2);  // the pre-sweep after the first
     if (!sync()) return;
     if (mine && d < ck) {
       const TailLevel<float> &L = T.lev[d];
-      DISPATCH_G(L.G, (resid_rows<GG, float>(lw, nlw, L.n, L.ptr, L.col, L.val, L.b, L.x2, L.r)));
+      DISPATCH_G(L.G, (resid_rows<GG, float>(lw, nlw, L.n, L.ptr, L.col, L.val, L.b, L.x2, L.r,
+                                              NoGate{})));
     } else if (mine && d == ck) {
-      coarse_rows<float>(lw, nlw, T.lev[d].n, T.cinv, T.lev[d].b, T.lev[d].x);
+      coarse_rows<float>(lw, nlw, T.lev[d].n, T.cinv, T.lev[d].b, T.lev[d].x, NoGate{});
     }
     if (!sync()) return;
     if (d == maxc) break;
@@ -996,7 +1079,8 @@ __global__ void __launch_bounds__(256) kb_tail(const CohortMember *mem, int K, i
       const TailLevel<float> &L = T.lev[d], &Lc = T.lev[d + 1];
       const bool c_jac = d + 1 < ck;
       restrict_aggs<float>(lw, nlw, L.n_agg, 1, L.mptr, L.mrow, L.P, L.r, Lc.b,
-                           c_jac ? Lc.dinv : nullptr, Lc.omega, c_jac ? Lc.x : nullptr);
+                           c_jac ? Lc.dinv : nullptr, Lc.omega, c_jac ? Lc.x : nullptr,
+                           NoGate{});
     }
     if (!sync()) return;
   }
@@ -1004,7 +1088,7 @@ __global__ void __launch_bounds__(256) kb_tail(const CohortMember *mem, int K, i
     if (mine_b && d < Tb.coarsest) {
       const TailLevel<float> &L = Tb.lev[d], &Lc = Tb.lev[d + 1];
       const float *xc = d + 1 == Tb.coarsest ? Lc.x : Lc.x2;  // the coarser level's result
-      prolong_rows<float>(blockIdx.x - b_lo, b_hi - b_lo, L.n, L.agg, L.P, xc, L.x2);
+      prolong_rows<float>(blockIdx.x - b_lo, b_hi - b_lo, L.n, L.agg, L.P, xc, L.x2, NoGate{});
     }
     if (!sync()) return;
     for (int s = 0; s < 2; ++s) {
@@ -1142,7 +1226,7 @@ mgpbd_status cohort_build(Cohort *c) {
     c->maxc = std::max(c->maxc, T.coarsest);
     mf_cohort_grids(h, M.grid);
     const int m = h->m;
-    M.grid[CS_XR] = std::min(dot_grid(m), wave_blocks((const void *)k_xr_update<float>, kDotThreads));
+    M.grid[CS_XR] = xr_blocks<float>(m);
     M.grid[CS_RESTRICT] = blocks_for((int64_t)L0.n_agg * 32, 256);
     M.grid[CS_PROLONG] = blocks_for((m + kProlongRows - 1) / kProlongRows, 256);
     M.grid[CS_PUPD] = blocks_for(std::max(1, (m / 2 + 1) / 2), 256);
@@ -1283,9 +1367,8 @@ static mgpbd_status vcycle_level(Handle *h, int l, const T *b_in, bool x0_ready 
   const int n = L.n;
   T *x = (T *)L.x;
   if (l == h->L - 1) {
-    k_coarse_apply<T><<<blocks_for((int64_t)n * 32, 256), 256, 0, h->stream>>>(n, h->cinv, b_in, x,
-                                                                                sc);
-    MG_LAUNCH("k_coarse_apply");
+    MG_TRY(chain_launch(h, "k_coarse_apply", k_coarse_apply<T>, blocks_for((int64_t)n * 32, 256),
+                        256, n, h->cinv, b_in, x, sc));
     return MGPBD_OK;
   }
   const int G = group_for(h, L, sizeof(T) == 8);
@@ -1304,9 +1387,9 @@ static mgpbd_status vcycle_level(Handle *h, int l, const T *b_in, bool x0_ready 
         int c = reverse ? nc - 1 - k : k;
         int64_t off = L.hcptr[c], cnt = L.hcptr[c + 1] - off;
         if (cnt == 0) continue;
-        DISPATCH_G(G, (k_gs_colour<GG, T><<<row_blocks(cnt, GG), 256, 0, h->stream>>>(
-                          (int)cnt, L.crow + off, L.ptr, L.col, val, dinv, b_in, x, sc)));
-        MG_LAUNCH("k_gs_colour");
+        DISPATCH_G(G, MG_TRY(chain_launch(h, "k_gs_colour", k_gs_colour<GG, T>, row_blocks(cnt, GG),
+                                          256, (int)cnt, L.crow + off, L.ptr, L.col, val, dinv,
+                                          b_in, x, sc)));
       }
     return MGPBD_OK;
   };
@@ -1316,9 +1399,8 @@ static mgpbd_status vcycle_level(Handle *h, int l, const T *b_in, bool x0_ready 
   const bool cheb = h->p.smoother == MGPBD_SMOOTH_CHEBYSHEV;
   auto apply = [&](const T *v, T *y) -> mgpbd_status {
     if (mf) return mf_level0<T>(h, kMfApply, v, b_in, dinv, om, y);
-    DISPATCH_G(G, (k_spmv_plain<GG, T><<<row_blocks(n, GG), 256, 0, h->stream>>>(
-                      n, L.ptr, L.col, val, v, y, sc)));
-    MG_LAUNCH("k_spmv_plain");
+    DISPATCH_G(G, MG_TRY(chain_launch(h, "k_spmv_plain", k_spmv_plain<GG, T>, row_blocks(n, GG),
+                                      256, n, L.ptr, L.col, val, v, y, sc)));
     return MGPBD_OK;
   };
   // (from_zero: x = 0 on entry, so A x = 0 needs no product)
@@ -1328,15 +1410,13 @@ static mgpbd_status vcycle_level(Handle *h, int l, const T *b_in, bool x0_ready 
     double rho = 1.0 / sigma;
     T *t = (T *)L.t, *d = x2;
     if (!from_zero) MG_TRY(apply(x, t));
-    k_cheb_start<T><<<blocks_for(n, 256), 256, 0, h->stream>>>(
-        n, b_in, from_zero ? nullptr : t, dinv, (T)(1.0 / theta), r, d, x, sc);
-    MG_LAUNCH("k_cheb_start");
+    MG_TRY(chain_launch(h, "k_cheb_start", k_cheb_start<T>, blocks_for(n, 256), 256, n, b_in,
+                        from_zero ? nullptr : t, dinv, (T)(1.0 / theta), r, d, x, sc));
     for (int k = 1; k < h->p.smooth_sweeps; ++k) {
       MG_TRY(apply(d, t));
       double rho2 = 1.0 / (2.0 * sigma - rho);
-      k_cheb_step<T><<<blocks_for(n, 256), 256, 0, h->stream>>>(
-          n, t, dinv, (T)(rho2 * rho), (T)(2.0 * rho2 / delta), r, d, x, sc);
-      MG_LAUNCH("k_cheb_step");
+      MG_TRY(chain_launch(h, "k_cheb_step", k_cheb_step<T>, blocks_for(n, 256), 256, n, t, dinv,
+                          (T)(rho2 * rho), (T)(2.0 * rho2 / delta), r, d, x, sc));
       rho = rho2;
     }
     return MGPBD_OK;
@@ -1347,17 +1427,16 @@ static mgpbd_status vcycle_level(Handle *h, int l, const T *b_in, bool x0_ready 
     MG_CUDA(cudaMemsetAsync(x, 0, sizeof(T) * n, h->stream));
     MG_TRY(gs_sweeps(false));
   } else if (!x0_ready) {
-    k_jacobi0<T><<<blocks_for(n, 256), 256, 0, h->stream>>>(n, b_in, dinv, om, x, sc);
-    MG_LAUNCH("k_jacobi0");
+    MG_TRY(chain_launch(h, "k_jacobi0", k_jacobi0<T>, blocks_for(n, 256), 256, n, b_in, dinv, om, x,
+                        sc));
   }
   for (int s = 1; s < h->p.smooth_sweeps && !gs && !cheb; ++s) {
     if (l == 0) MG_TRY(prof_begin(h));
     if (mf) {
       MG_TRY(mf_level0<T>(h, kMfSweep, x, b_in, dinv, om, x2));
     } else {
-      DISPATCH_G(G, (k_jacobi<GG, T><<<row_blocks(n, GG), 256, 0, h->stream>>>(
-                        n, L.ptr, L.col, val, dinv, om, b_in, x, x2, sc)));
-      MG_LAUNCH("k_jacobi");
+      DISPATCH_G(G, MG_TRY(chain_launch(h, "k_jacobi", k_jacobi<GG, T>, row_blocks(n, GG), 256, n,
+                                        L.ptr, L.col, val, dinv, om, b_in, x, x2, sc)));
     }
     if (l == 0) MG_TRY(prof_end(h));
     std::swap(x, x2);
@@ -1369,24 +1448,21 @@ static mgpbd_status vcycle_level(Handle *h, int l, const T *b_in, bool x0_ready 
   if (mf && L.mpos && nk == 1) {
     // the residual written in member order, the restriction streaming it
     MG_TRY(mf_level0<T>(h, kMfResidMember, x, b_in, dinv, om, r));
-    k_restrict_member<T><<<blocks_for((int64_t)L.n_agg * 32, 256), 256, 0, h->stream>>>(
-        L.n_agg, L.mptr, (const T *)L.Pm, r, (T *)Lc.b, sc, c_jac ? dinvs<T>(Lc) : nullptr,
-        (T)Lc.omega, c_jac ? (T *)Lc.x : nullptr);
-    MG_LAUNCH("k_restrict_member");
+    MG_TRY(chain_launch(h, "k_restrict_member", k_restrict_member<T>,
+                        blocks_for((int64_t)L.n_agg * 32, 256), 256, L.n_agg, L.mptr,
+                        (const T *)L.Pm, r, (T *)Lc.b, sc, c_jac ? dinvs<T>(Lc) : nullptr,
+                        (T)Lc.omega, c_jac ? (T *)Lc.x : nullptr));
   } else if (mf) {
     MG_TRY(mf_level0<T>(h, kMfResid, x, b_in, dinv, om, r));
-    k_restrict<T><<<blocks_for((int64_t)L.n_agg * 32, 256), 256, 0, h->stream>>>(
-        L.n_agg, nk, L.mptr, L.mrow, Ps<T>(L), r, (T *)Lc.b, sc, c_jac ? dinvs<T>(Lc) : nullptr,
-        (T)Lc.omega, c_jac ? (T *)Lc.x : nullptr);
-    MG_LAUNCH("k_restrict");
+    MG_TRY(chain_launch(h, "k_restrict", k_restrict<T>, blocks_for((int64_t)L.n_agg * 32, 256), 256,
+                        L.n_agg, nk, L.mptr, L.mrow, Ps<T>(L), r, (T *)Lc.b, sc,
+                        c_jac ? dinvs<T>(Lc) : nullptr, (T)Lc.omega, c_jac ? (T *)Lc.x : nullptr));
   } else {
-    DISPATCH_G(G, (k_resid<GG, T><<<row_blocks(n, GG), 256, 0, h->stream>>>(n, L.ptr, L.col, val,
-                                                                           b_in, x, r, sc)));
-    MG_LAUNCH("k_resid");
-    k_restrict<T><<<blocks_for((int64_t)L.n_agg * 32, 256), 256, 0, h->stream>>>(
-        L.n_agg, nk, L.mptr, L.mrow, Ps<T>(L), r, (T *)Lc.b, sc, c_jac ? dinvs<T>(Lc) : nullptr,
-        (T)Lc.omega, c_jac ? (T *)Lc.x : nullptr);
-    MG_LAUNCH("k_restrict");
+    DISPATCH_G(G, MG_TRY(chain_launch(h, "k_resid", k_resid<GG, T>, row_blocks(n, GG), 256, n,
+                                      L.ptr, L.col, val, b_in, x, r, sc)));
+    MG_TRY(chain_launch(h, "k_restrict", k_restrict<T>, blocks_for((int64_t)L.n_agg * 32, 256), 256,
+                        L.n_agg, nk, L.mptr, L.mrow, Ps<T>(L), r, (T *)Lc.b, sc,
+                        c_jac ? dinvs<T>(Lc) : nullptr, (T)Lc.omega, c_jac ? (T *)Lc.x : nullptr));
   }
   const T *xc = (const T *)Lc.x;  // where the coarser level leaves its result
   if (tail_applies(h, l + 1)) {
@@ -1396,12 +1472,12 @@ static mgpbd_status vcycle_level(Handle *h, int l, const T *b_in, bool x0_ready 
     MG_TRY(vcycle_level<T>(h, l + 1, (const T *)Lc.b, c_jac));
   }
   if (nk == 1)
-    k_prolong<T><<<blocks_for((n + kProlongRows - 1) / kProlongRows, 256), 256, 0, h->stream>>>(
-        n, L.agg, Ps<T>(L), xc, x, sc);
+    MG_TRY(chain_launch(h, "k_prolong", k_prolong<T>,
+                        blocks_for((n + kProlongRows - 1) / kProlongRows, 256), 256, n, L.agg,
+                        Ps<T>(L), xc, x, sc));
   else
-    k_prolong_k<T><<<blocks_for(n, 256), 256, 0, h->stream>>>(n, nk, L.agg, Ps<T>(L),
-                                                              (const T *)Lc.x, x, sc);
-  MG_LAUNCH("k_prolong");
+    MG_TRY(chain_launch(h, "k_prolong", k_prolong_k<T>, blocks_for(n, 256), 256, n, nk, L.agg,
+                        Ps<T>(L), (const T *)Lc.x, x, sc));
   if (gs) MG_TRY(gs_sweeps(true));
   if (cheb) MG_TRY(cheb_smooth(false));
   bool zw = false;
@@ -1415,9 +1491,8 @@ static mgpbd_status vcycle_level(Handle *h, int l, const T *b_in, bool x0_ready 
     if (mf) {
       MG_TRY(mf_level0<T>(h, kMfSweep, x, b_in, dinv, om, x2));
     } else {
-      DISPATCH_G(G, (k_jacobi<GG, T><<<row_blocks(n, GG), 256, 0, h->stream>>>(
-                        n, L.ptr, L.col, val, dinv, om, b_in, x, x2, sc)));
-      MG_LAUNCH("k_jacobi");
+      DISPATCH_G(G, MG_TRY(chain_launch(h, "k_jacobi", k_jacobi<GG, T>, row_blocks(n, GG), 256, n,
+                                        L.ptr, L.col, val, dinv, om, b_in, x, x2, sc)));
     }
     if (l == 0) MG_TRY(prof_end(h));
     std::swap(x, x2);
@@ -1432,9 +1507,9 @@ static mgpbd_status vcycle_level(Handle *h, int l, const T *b_in, bool x0_ready 
 static mgpbd_status launch_dot(Handle *h, const double *x, const double *y, int64_t n, int mode,
                                int check_done, double *out = nullptr) {
   DotCtx c = make_ctx(h, mode, out);
-  k_dot<<<std::min(dot_grid(n), wave_blocks((const void *)k_dot, kDotThreads)), kDotThreads, 0,
-          h->stream>>>(n, x, y, c, check_done);
-  MG_LAUNCH("k_dot");
+  MG_TRY(chain_launch(h, "k_dot", k_dot,
+                      std::min(dot_grid(n), wave_blocks((const void *)k_dot, kDotThreads)),
+                      kDotThreads, n, x, y, c, check_done));
   return MGPBD_OK;
 }
 
@@ -1460,27 +1535,24 @@ static mgpbd_status vcycle_top(Handle *h, const double *r, double *z, bool prepa
   bool zw = false;
   if (h->p.precision == MGPBD_MIXED) {
     if (!prepared) {
-      k_top_prep<float><<<blocks_for(m, 256), 256, 0, h->stream>>>(
-          m, r, (float *)L.b, L.dinv32, (float)L.omega, jac ? (float *)L.x : nullptr, h->sc);
-      MG_LAUNCH("k_top_prep");
+      MG_TRY(chain_launch(h, "k_top_prep", k_top_prep<float>, blocks_for(m, 256), 256, m, r,
+                          (float *)L.b, L.dinv32, (float)L.omega, jac ? (float *)L.x : nullptr,
+                          h->sc));
     }
     MG_TRY(vcycle_level<float>(h, 0, (const float *)L.b, jac, &o, &zw));
     if (!zw) {
-      k_convert<float, double><<<blocks_for(m, 256), 256, 0, h->stream>>>(m, (const float *)L.x,
-                                                                          z, h->sc);
-      MG_LAUNCH("k_convert");
+      MG_TRY(chain_launch(h, "k_convert", k_convert<float, double>, blocks_for(m, 256), 256, m,
+                          (const float *)L.x, z, h->sc));
     }
   } else {
     if (!prepared && jac) {
-      k_top_prep<double><<<blocks_for(m, 256), 256, 0, h->stream>>>(m, r, nullptr, L.dinv, L.omega,
-                                                                    (double *)L.x, h->sc);
-      MG_LAUNCH("k_top_prep");
+      MG_TRY(chain_launch(h, "k_top_prep", k_top_prep<double>, blocks_for(m, 256), 256, m, r,
+                          nullptr, L.dinv, L.omega, (double *)L.x, h->sc));
     }
     MG_TRY(vcycle_level<double>(h, 0, r, jac, &o, &zw));
     if (!zw) {
-      k_convert<double, double><<<blocks_for(m, 256), 256, 0, h->stream>>>(
-          m, (const double *)L.x, z, h->sc);
-      MG_LAUNCH("k_convert");
+      MG_TRY(chain_launch(h, "k_convert", k_convert<double, double>, blocks_for(m, 256), 256, m,
+                          (const double *)L.x, z, h->sc));
     }
   }
   if (o.dot && !zw) MG_TRY(launch_dot(h, r, z, m, dot_mode, 1));
@@ -1503,11 +1575,9 @@ mgpbd_status apply_level0(Handle *h, int form, const double *x, double *y) {
   DotCtx c = make_ctx(h, DOT_STORE, &h->sc->tr2);  // x.Ax lands in a scratch scalar
   if (form == 0) {
     const int G = group_for(h, L, true);
-    DISPATCH_G(G, (k_spmv_pq<GG, double, double>
-                   <<<std::min(row_blocks(m, GG),
-                               wave_blocks((const void *)k_spmv_pq<GG, double, double>, 256)),
-                      256, 0, h->stream>>>(m, L.ptr, L.col, L.val, x, y, c)));
-    MG_LAUNCH("k_spmv_pq");
+    DISPATCH_G(G, MG_TRY(chain_launch(h, "k_spmv_pq", k_spmv_pq<GG, double, double>,
+                                      spmv_pq_blocks<GG>(m),
+                                      256, m, L.ptr, L.col, L.val, x, y, c)));
     return MGPBD_OK;
   }
   if (form == 2) MG_TRY(mf_split(h, x, h->p_df, m));
@@ -1535,32 +1605,26 @@ static mgpbd_status pcg_iteration(Handle *h, double *x) {
   if (h->p.level0_op == 1) {
     MG_TRY(mf_apply_pq(h, p, q, cpq));
   } else {
-    DISPATCH_G(G, (k_spmv_pq<GG, double, double>
-                   <<<std::min(row_blocks(m, GG),
-                               wave_blocks((const void *)k_spmv_pq<GG, double, double>, 256)),
-                      256, 0, h->stream>>>(m, L.ptr, L.col, L.val, p, q, cpq)));
-    MG_LAUNCH("k_spmv_pq");
+    DISPATCH_G(G, MG_TRY(chain_launch(h, "k_spmv_pq", k_spmv_pq<GG, double, double>,
+                                      spmv_pq_blocks<GG>(m),
+                                      256, m, L.ptr, L.col, L.val, p, q, cpq)));
   }
   MG_TRY(prof_end(h, PROF_AP));
   // the update also starts the V-cycle (right-hand side, first Jacobi sweep)
   const bool jac = top_jacobi(h);
   if (h->p.precision == MGPBD_MIXED)
-    k_xr_update<float><<<std::min(dot_grid(m), wave_blocks((const void *)k_xr_update<float>,
-                                                           kDotThreads)),
-                         kDotThreads, 0, h->stream>>>(
-        m, x, r, p, q, make_ctx(h, DOT_RR), (float *)L.b, L.dinv32, (float)L.omega,
-        jac ? (float *)L.x : nullptr);
+    MG_TRY(chain_launch(h, "k_xr_update", k_xr_update<float>,
+                        xr_blocks<float>(m),
+                        kDotThreads, m, x, r, p, q, make_ctx(h, DOT_RR), (float *)L.b, L.dinv32,
+                        (float)L.omega, jac ? (float *)L.x : nullptr));
   else
-    k_xr_update<double><<<std::min(dot_grid(m), wave_blocks((const void *)k_xr_update<double>,
-                                                            kDotThreads)),
-                          kDotThreads, 0, h->stream>>>(
-        m, x, r, p, q, make_ctx(h, DOT_RR), nullptr, L.dinv, L.omega,
-        jac ? (double *)L.x : nullptr);
-  MG_LAUNCH("k_xr_update");
+    MG_TRY(chain_launch(h, "k_xr_update", k_xr_update<double>,
+                        xr_blocks<double>(m),
+                        kDotThreads, m, x, r, p, q, make_ctx(h, DOT_RR), nullptr, L.dinv, L.omega,
+                        jac ? (double *)L.x : nullptr));
   MG_TRY(vcycle_top(h, r, z, true, DOT_RZ));
-  k_p_update<<<blocks_for(std::max(1, (m / 2 + 1) / 2), 256), 256, 0, h->stream>>>(
-      m, p, z, h->sc, h->p.ap_split ? h->p_df : nullptr);
-  MG_LAUNCH("k_p_update");
+  MG_TRY(chain_launch(h, "k_p_update", k_p_update, blocks_for(std::max(1, (m / 2 + 1) / 2), 256),
+                      256, m, p, z, h->sc, h->p.ap_split ? h->p_df : nullptr));
   return MGPBD_OK;
 }
 
