@@ -39,9 +39,9 @@ extern unsigned long long g_launches;  // updated atomically
     cudaError_t e_ = cudaGetLastError();                                  \
     if (e_ != cudaSuccess) return mg::cuda_fail(e_, what, __FILE__, __LINE__); \
   } while (0)
-#define MG_TRY(expr)                                                      \
+#define MG_TRY(...)                                                       \
   do {                                                                    \
-    mgpbd_status s_ = (expr);                                             \
+    mgpbd_status s_ = (__VA_ARGS__);                                      \
     if (s_ < 0) return s_;                                                \
   } while (0)
 

@@ -34,6 +34,13 @@ constexpr int kMfVertexLanes = 8;
 // 16-byte load each
 constexpr int kUStride = 3, kUStrideDf = 4;
 
+// Up to this many rows the passes run in their early form (k_mf_row_early,
+// k_mf_vertex32_early, k_mf_vertex64_early: one row or vertex per thread
+// group, static loads before the wait): the kernel is a small part of a wave or
+// one, its time is that of its dependent loads, and its 40 to 80 registers
+// cost nothing.  Above it the plain form's occupancy counts.
+constexpr int kEarlyRows = 1 << 17;
+
 // slot of vertex v in each incident row (create time)
 __global__ void k_vslot(int N, int E, const int32_t *edge, const int32_t *tet, const int64_t *vptr,
                         const int32_t *vrow, uint8_t *vslot) {
@@ -186,6 +193,99 @@ __global__ void __launch_bounds__(256, 8)
   chain_wait();
   if (sc && is_done(sc)) return;
   mf_vertex32_rows<G>(HW_WARPS, N, vorder, vptr, ginc, w, x, u);
+}
+
+// The vertex passes for one group of G lanes per vertex, with the vertex's
+// range and the first four incidences of each lane loaded before the wait (an
+// instance of 30,000 rows has four to eight per lane), so that the gather of
+// x is the only load behind it.  The same sums in the same order.
+template <int G>
+__global__ void __launch_bounds__(256)
+    k_mf_vertex64_early(int N, const int32_t *vorder, const int64_t *vptr, const int32_t *vrow,
+                        const double *ginc, const double *w, const double *x, double *u,
+                        const PcgScalars *sc) {
+  const int g = threadIdx.x & (G - 1);
+  const int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / G;
+  const bool valid = i < N;
+  const int v = valid ? vorder[i] : 0;
+  int64_t q = 0, e = 0;
+  if (valid) {
+    q = vptr[v] + g;
+    e = vptr[v + 1];
+  }
+  const int comp = group_sum3_component<G>(g);
+  const bool head = valid && comp < 3 && (g & (G / 4 - 1)) == 0;
+  const double wv = head ? w[v] : 0.0;
+  double a0 = 0, a1 = 0, a2 = 0;
+  ChainGate gate(sc);
+  do {
+    int r[4];
+    double g3[4][3], xv[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      if (q + k * G < e) {
+        r[k] = vrow[q + k * G];
+        const double *gq = ginc + 3 * (q + k * G);
+        g3[k][0] = gq[0];
+        g3[k][1] = gq[1];
+        g3[k][2] = gq[2];
+      }
+    gate.open();
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      if (q + k * G < e) xv[k] = x[r[k]];
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      if (q + k * G < e) {
+        a0 = fma(g3[k][0], xv[k], a0);
+        a1 = fma(g3[k][1], xv[k], a1);
+        a2 = fma(g3[k][2], xv[k], a2);
+      }
+    q += 4 * G;
+  } while (q < e && !gate.closed());
+  const double s = group_sum3<G>(a0, a1, a2, g);
+  if (head && !gate.closed()) u[kUStride * (int64_t)v + comp] = wv * s;
+}
+
+template <int G>
+__global__ void __launch_bounds__(256)
+    k_mf_vertex32_early(int N, const int32_t *vorder, const int64_t *vptr, const float4 *ginc,
+                        const float *w, const float *x, float *u, const PcgScalars *sc) {
+  const int g = threadIdx.x & (G - 1);
+  const int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / G;
+  const bool valid = i < N;
+  const int v = valid ? vorder[i] : 0;
+  int64_t q = 0, e = 0;
+  if (valid) {
+    q = vptr[v] + g;
+    e = vptr[v + 1];
+  }
+  const int comp = group_sum3_component<G>(g);
+  const bool head = valid && comp < 3 && (g & (G / 4 - 1)) == 0;
+  const float wv = head ? w[v] : 0.f;
+  float a0 = 0, a1 = 0, a2 = 0;
+  ChainGate gate(sc);
+  do {
+    float4 ev[4];
+    float xv[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      if (q + k * G < e) ev[k] = ginc[q + k * G];
+    gate.open();
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      if (q + k * G < e) xv[k] = x[__float_as_int(ev[k].w)];
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      if (q + k * G < e) {
+        a0 = fmaf(ev[k].x, xv[k], a0);
+        a1 = fmaf(ev[k].y, xv[k], a1);
+        a2 = fmaf(ev[k].z, xv[k], a2);
+      }
+    q += 4 * G;
+  } while (q < e && !gate.closed());
+  const float s = group_sum3<G>(a0, a1, a2, g);
+  if (head && !gate.closed()) u[kUStride * (int64_t)v + comp] = wv * s;
 }
 
 // 16-byte loads of the pair form's row pass (all arrays 256-byte aligned by
@@ -432,6 +532,31 @@ enum {
 //   MF_SWEEP_ZDOT the same, with r.z folded into the PCG scalars
 //   MF_RESID_MEMBER out[pos_i] = b - y for rows in an aggregate (the
 //                 residual in member order, for the restriction)
+// the row's result from y = J u + alpha~ x (MODE as above); acc collects the
+// row's share of the dot product
+template <class T, int MODE>
+__device__ __forceinline__ void mf_row_out(int64_t i, T y, T xi, T bi, T di, T omega, T *out,
+                                           double *z, double ri, int32_t q, double &acc) {
+  if (MODE == MF_SWEEP) out[i] = fma(omega, (bi - y) * di, xi);
+  else if (MODE == MF_RESID) out[i] = bi - y;
+  else if (MODE == MF_RESID_MEMBER) {
+    if (q >= 0) out[q] = bi - y;
+  } else if (MODE == MF_APPLY) out[i] = y;
+  else if (MODE == MF_APPLY_DOT) {
+    out[i] = y;
+    acc = fma(widen(xi), widen(y), acc);
+  } else {
+    const double zi = widen(fma(omega, (bi - y) * di, xi));
+    z[i] = zi;
+    if (MODE == MF_SWEEP_ZDOT) acc = fma(ri, zi, acc);
+  }
+}
+
+constexpr bool mf_uses_b(int mode) { return mode != MF_APPLY && mode != MF_APPLY_DOT; }
+constexpr bool mf_uses_dinv(int mode) {
+  return mode == MF_SWEEP || mode == MF_SWEEP_Z || mode == MF_SWEEP_ZDOT;
+}
+
 template <class T, int MODE>
 __device__ __forceinline__ void mf_row_body(int vb, int vn, int E, int m, const int32_t *edge,
                                             const int32_t *tet, const T *gd, const T *gt,
@@ -464,21 +589,10 @@ __device__ __forceinline__ void mf_row_body(int vb, int vn, int E, int m, const 
     }
     T xi = x[i];
     y = fma(at[i], xi, y);
-    if (MODE == MF_SWEEP) out[i] = fma(omega, (b[i] - y) * dinv[i], xi);
-    else if (MODE == MF_RESID) out[i] = b[i] - y;
-    else if (MODE == MF_RESID_MEMBER) {
-      const int32_t q = pos[i];
-      if (q >= 0) out[q] = b[i] - y;
-    }
-    else if (MODE == MF_APPLY) out[i] = y;
-    else if (MODE == MF_APPLY_DOT) {
-      out[i] = y;
-      acc = fma(widen(xi), widen(y), acc);
-    } else {
-      double zi = widen(fma(omega, (b[i] - y) * dinv[i], xi));
-      z[i] = zi;
-      if (MODE == MF_SWEEP_ZDOT) acc = fma(rr[i], zi, acc);
-    }
+    mf_row_out<T, MODE>(i, y, xi, mf_uses_b(MODE) ? b[i] : (T)0,
+                        mf_uses_dinv(MODE) ? dinv[i] : (T)0, omega, out, z,
+                        MODE == MF_SWEEP_ZDOT ? rr[i] : 0.0,
+                        MODE == MF_RESID_MEMBER ? pos[i] : 0, acc);
   }
   if (MODE == MF_APPLY_DOT || MODE == MF_SWEEP_ZDOT) block_dot_finish_vg(acc, c, vb, vn);
 }
@@ -492,6 +606,71 @@ __global__ void k_mf_row(int E, int m, const int32_t *edge, const int32_t *tet, 
   if (is_done(c.sc)) return;
   mf_row_body<T, MODE>(blockIdx.x, gridDim.x, E, m, edge, tet, gd, gt, u, at, x, b, dinv, omega,
                        out, c, z, rr, pos);
+}
+
+// k_mf_row for one row per thread, with the row's vertices, gradient, alpha~,
+// 1/A_ii and member position loaded before the wait: what remains behind it is
+// one level of loads (u, x, b) and the store.  The same arithmetic.
+template <class T, int MODE>
+__global__ void __launch_bounds__(256)
+    k_mf_row_early(int E, int m, const int32_t *edge, const int32_t *tet, const T *gd,
+                   const T *gt, const T *u, const T *at, const T *x, const T *b, const T *dinv,
+                   T omega, T *out, DotCtx c, double *z, const double *rr, const int32_t *pos) {
+  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const bool live = i < m, isE = i < E;
+  int t[4] = {0, 0, 0, 0};
+  T gg[12];
+  T ai = 0, di = 0;
+  int32_t q = 0;
+  if (live) {
+    if (isE) {
+      const int2 e = reinterpret_cast<const int2 *>(edge)[i];
+      t[0] = e.x;
+      t[1] = e.y;
+#pragma unroll
+      for (int k = 0; k < 3; ++k) gg[k] = gd[3 * i + k];
+    } else {
+      const int4 e = reinterpret_cast<const int4 *>(tet)[i - E];
+      t[0] = e.x;
+      t[1] = e.y;
+      t[2] = e.z;
+      t[3] = e.w;
+#pragma unroll
+      for (int k = 0; k < 12; ++k) gg[k] = gt[12 * (i - E) + k];
+    }
+    ai = at[i];
+    if (mf_uses_dinv(MODE)) di = dinv[i];
+    if (MODE == MF_RESID_MEMBER) q = pos[i];
+  }
+  ChainGate gate(c.sc);
+  gate.open();
+  double acc = 0.0;
+  if (live) {
+    const T xi = x[i], bi = mf_uses_b(MODE) ? b[i] : (T)0;
+    const double ri = MODE == MF_SWEEP_ZDOT ? rr[i] : 0.0;
+    T y;
+    if (isE) {
+      const T *ua = u + kUStride * (int64_t)t[0], *ub = u + kUStride * (int64_t)t[1];
+      y = gg[0] * (ua[0] - ub[0]);
+      y = fma(gg[1], ua[1] - ub[1], y);
+      y = fma(gg[2], ua[2] - ub[2], y);
+    } else {
+      T uv[12];
+#pragma unroll
+      for (int s = 0; s < 4; ++s)
+#pragma unroll
+        for (int k = 0; k < 3; ++k) uv[3 * s + k] = u[kUStride * (int64_t)t[s] + k];
+      y = 0;
+#pragma unroll
+      for (int k = 0; k < 12; ++k) y = fma(gg[k], uv[k], y);
+    }
+    y = fma(ai, xi, y);
+    if (!gate.closed()) mf_row_out<T, MODE>(i, y, xi, bi, di, omega, out, z, ri, q, acc);
+  }
+  if (MODE == MF_APPLY_DOT || MODE == MF_SWEEP_ZDOT) {
+    if (gate.closed()) return;
+    block_dot_finish(acc, c);
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -564,6 +743,18 @@ mgpbd_status mf_create(Handle *h) {
 // rows.
 static int mf_grid(int64_t rows, int threads) {
   return (int)std::max<int64_t>(1, std::min<int64_t>((rows + threads - 1) / threads, 8192));
+}
+
+template <class T, int MODE>
+static mgpbd_status mf_row_launch(Handle *h, const char *what, int blocks, const T *gd,
+                                  const T *gt, const T *u, const T *at, const T *x, const T *b,
+                                  const T *dinv, T omega, T *out, const DotCtx &c, double *z,
+                                  const double *rr, const int32_t *pos) {
+  if (h->m <= kEarlyRows)
+    return chain_launch(h, what, k_mf_row_early<T, MODE>, blocks_for(h->m, 256), 256, h->E, h->m,
+                        h->edge, h->tet, gd, gt, u, at, x, b, dinv, omega, out, c, z, rr, pos);
+  return chain_launch(h, what, k_mf_row<T, MODE>, blocks, 256, h->E, h->m, h->edge, h->tet, gd,
+                      gt, u, at, x, b, dinv, omega, out, c, z, rr, pos);
 }
 
 mgpbd_status mf_prepare(Handle *h) {
@@ -723,6 +914,13 @@ mgpbd_status mf_cohort_step(int which, int sel, const CohortMember *d_mem,
 static mgpbd_status mf_vertex(Handle *h, const double *x, int G = 0, bool check_done = true) {
   if (G == 0) G = h->force_vert64 ? h->force_vert64 : h->mf_g64;
   const PcgScalars *sc = check_done ? h->sc : nullptr;
+  if (h->m <= kEarlyRows) {
+    MF_G_DISPATCH(G, MG_TRY(chain_launch(h, "k_mf_vertex64", k_mf_vertex64_early<GG>,
+                                          blocks_for((int64_t)h->N * GG, 256), 256, h->N,
+                                          h->vorder, h->vptr, h->vrow, h->ginc64, h->w, x, h->u64,
+                                          sc)));
+    return MGPBD_OK;
+  }
   MF_G_DISPATCH(G, MG_TRY(chain_launch(h, "k_mf_vertex64", k_mf_vertex64<GG>,
                                         mf_vertex_blocks(h, GG), 256, h->N, h->vorder, h->vptr,
                                         h->vrow, h->ginc64, h->w, x, h->u64, sc)));
@@ -732,6 +930,12 @@ static mgpbd_status mf_vertex(Handle *h, const double *x, int G = 0, bool check_
 static mgpbd_status mf_vertex(Handle *h, const float *x, int G = 0, bool check_done = true) {
   if (G == 0) G = h->force_vert32 ? h->force_vert32 : h->mf_g32;
   const PcgScalars *sc = check_done ? h->sc : nullptr;
+  if (h->m <= kEarlyRows) {
+    MF_G_DISPATCH(G, MG_TRY(chain_launch(h, "k_mf_vertex32", k_mf_vertex32_early<GG>,
+                                          blocks_for((int64_t)h->N * GG, 256), 256, h->N,
+                                          h->vorder, h->vptr, h->ginc4, h->w32, x, h->u32, sc)));
+    return MGPBD_OK;
+  }
   MF_G_DISPATCH(G, MG_TRY(chain_launch(h, "k_mf_vertex32", k_mf_vertex32<GG>,
                                         mf_vertex_blocks(h, GG), 256, h->N, h->vorder, h->vptr,
                                         h->ginc4, h->w32, x, h->u32, sc)));
@@ -799,9 +1003,9 @@ mgpbd_status mf_apply_pq_form(Handle *h, bool pairs, const double *p, double *q,
   MG_TRY(mf_vertex(h, p));
   const int grid = std::min(mf_grid(h->m, 256),
                             wave_blocks((const void *)k_mf_row<double, MF_APPLY_DOT>, 256));
-  MG_TRY(chain_launch(h, "k_mf_row(A.p)", k_mf_row<double, MF_APPLY_DOT>, grid, 256, h->E, h->m,
-                      h->edge, h->tet, h->gd, h->gt, h->u64, h->alpha_t, p, nullptr, nullptr, 0.0,
-                      q, c, nullptr, nullptr, nullptr));
+  MG_TRY(mf_row_launch<double, MF_APPLY_DOT>(
+      h, "k_mf_row(A.p)", grid, h->gd, h->gt, h->u64, h->alpha_t, p, nullptr, nullptr, 0.0, q, c,
+      nullptr, nullptr, nullptr));
   return MGPBD_OK;
 }
 
@@ -815,9 +1019,9 @@ mgpbd_status mf_residual64(Handle *h, const double *x, const double *b, double *
   MG_TRY(mf_vertex(h, x, 0, false));
   DotCtx c{};
   c.sc = h->sc;
-  MG_TRY(chain_launch(h, "k_mf_row(b - A x)", k_mf_row<double, MF_RESID>, mf_grid(h->m, 256), 256,
-                      h->E, h->m, h->edge, h->tet, h->gd, h->gt, h->u64, h->alpha_t, x, b, nullptr,
-                      0.0, r, c, nullptr, nullptr, nullptr));
+  MG_TRY(mf_row_launch<double, MF_RESID>(
+      h, "k_mf_row(b - A x)", mf_grid(h->m, 256), h->gd, h->gt, h->u64, h->alpha_t, x, b, nullptr,
+      0.0, r, c, nullptr, nullptr, nullptr));
   return MGPBD_OK;
 }
 
@@ -840,21 +1044,21 @@ mgpbd_status mf_level0<float>(Handle *h, int mode, const float *x, const float *
   DotCtx c{};
   c.sc = h->sc;
   if (mode == MF_SWEEP)
-    MG_TRY(chain_launch(h, "k_mf_row(f32)", k_mf_row<float, MF_SWEEP>, mf_grid(h->m, 256), 256,
-                        h->E, h->m, h->edge, h->tet, h->gd32, h->gt32, h->u32, h->at32, x, b, dinv,
-                        omega, out, c, nullptr, nullptr, nullptr));
+    MG_TRY(mf_row_launch<float, MF_SWEEP>(
+        h, "k_mf_row(f32)", mf_grid(h->m, 256), h->gd32, h->gt32, h->u32, h->at32, x, b, dinv,
+        omega, out, c, nullptr, nullptr, nullptr));
   else if (mode == MF_APPLY)
-    MG_TRY(chain_launch(h, "k_mf_row(f32)", k_mf_row<float, MF_APPLY>, mf_grid(h->m, 256), 256,
-                        h->E, h->m, h->edge, h->tet, h->gd32, h->gt32, h->u32, h->at32, x, b, dinv,
-                        omega, out, c, nullptr, nullptr, nullptr));
+    MG_TRY(mf_row_launch<float, MF_APPLY>(
+        h, "k_mf_row(f32)", mf_grid(h->m, 256), h->gd32, h->gt32, h->u32, h->at32, x, b, dinv,
+        omega, out, c, nullptr, nullptr, nullptr));
   else if (mode == MF_RESID_MEMBER)
-    MG_TRY(chain_launch(h, "k_mf_row(f32)", k_mf_row<float, MF_RESID_MEMBER>, mf_grid(h->m, 256),
-                        256, h->E, h->m, h->edge, h->tet, h->gd32, h->gt32, h->u32, h->at32, x, b,
-                        dinv, omega, out, c, nullptr, nullptr, h->lev[0].mpos));
+    MG_TRY(mf_row_launch<float, MF_RESID_MEMBER>(
+        h, "k_mf_row(f32)", mf_grid(h->m, 256), h->gd32, h->gt32, h->u32, h->at32, x, b, dinv,
+        omega, out, c, nullptr, nullptr, h->lev[0].mpos));
   else
-    MG_TRY(chain_launch(h, "k_mf_row(f32)", k_mf_row<float, MF_RESID>, mf_grid(h->m, 256), 256,
-                        h->E, h->m, h->edge, h->tet, h->gd32, h->gt32, h->u32, h->at32, x, b, dinv,
-                        omega, out, c, nullptr, nullptr, nullptr));
+    MG_TRY(mf_row_launch<float, MF_RESID>(
+        h, "k_mf_row(f32)", mf_grid(h->m, 256), h->gd32, h->gt32, h->u32, h->at32, x, b, dinv,
+        omega, out, c, nullptr, nullptr, nullptr));
   return MGPBD_OK;
 }
 
@@ -865,21 +1069,21 @@ mgpbd_status mf_level0<double>(Handle *h, int mode, const double *x, const doubl
   DotCtx c{};
   c.sc = h->sc;
   if (mode == MF_SWEEP)
-    MG_TRY(chain_launch(h, "k_mf_row(f64)", k_mf_row<double, MF_SWEEP>, mf_grid(h->m, 256), 256,
-                        h->E, h->m, h->edge, h->tet, h->gd, h->gt, h->u64, h->alpha_t, x, b, dinv,
-                        omega, out, c, nullptr, nullptr, nullptr));
+    MG_TRY(mf_row_launch<double, MF_SWEEP>(
+        h, "k_mf_row(f64)", mf_grid(h->m, 256), h->gd, h->gt, h->u64, h->alpha_t, x, b, dinv, omega,
+        out, c, nullptr, nullptr, nullptr));
   else if (mode == MF_APPLY)
-    MG_TRY(chain_launch(h, "k_mf_row(f64)", k_mf_row<double, MF_APPLY>, mf_grid(h->m, 256), 256,
-                        h->E, h->m, h->edge, h->tet, h->gd, h->gt, h->u64, h->alpha_t, x, b, dinv,
-                        omega, out, c, nullptr, nullptr, nullptr));
+    MG_TRY(mf_row_launch<double, MF_APPLY>(
+        h, "k_mf_row(f64)", mf_grid(h->m, 256), h->gd, h->gt, h->u64, h->alpha_t, x, b, dinv, omega,
+        out, c, nullptr, nullptr, nullptr));
   else if (mode == MF_RESID_MEMBER)
-    MG_TRY(chain_launch(h, "k_mf_row(f64)", k_mf_row<double, MF_RESID_MEMBER>, mf_grid(h->m, 256),
-                        256, h->E, h->m, h->edge, h->tet, h->gd, h->gt, h->u64, h->alpha_t, x, b,
-                        dinv, omega, out, c, nullptr, nullptr, h->lev[0].mpos));
+    MG_TRY(mf_row_launch<double, MF_RESID_MEMBER>(
+        h, "k_mf_row(f64)", mf_grid(h->m, 256), h->gd, h->gt, h->u64, h->alpha_t, x, b, dinv, omega,
+        out, c, nullptr, nullptr, h->lev[0].mpos));
   else
-    MG_TRY(chain_launch(h, "k_mf_row(f64)", k_mf_row<double, MF_RESID>, mf_grid(h->m, 256), 256,
-                        h->E, h->m, h->edge, h->tet, h->gd, h->gt, h->u64, h->alpha_t, x, b, dinv,
-                        omega, out, c, nullptr, nullptr, nullptr));
+    MG_TRY(mf_row_launch<double, MF_RESID>(
+        h, "k_mf_row(f64)", mf_grid(h->m, 256), h->gd, h->gt, h->u64, h->alpha_t, x, b, dinv, omega,
+        out, c, nullptr, nullptr, nullptr));
   return MGPBD_OK;
 }
 
@@ -895,15 +1099,14 @@ mgpbd_status mf_level0_final(Handle *h, const T *x, const T *b, const T *dinv, T
   DotCtx c = o.c;
   c.sc = h->sc;
   if (o.dot)
-    MG_TRY(chain_launch(h, "k_mf_row(final sweep)", k_mf_row<T, MF_SWEEP_ZDOT>,
-                        std::min(mf_grid(h->m, 256),
-                                 wave_blocks((const void *)k_mf_row<T, MF_SWEEP_ZDOT>, 256)),
-                        256, h->E, h->m, h->edge, h->tet, gd, gt, u, at, x, b, dinv, omega, nullptr,
-                        c, o.z, o.r, nullptr));
+    MG_TRY(mf_row_launch<T, MF_SWEEP_ZDOT>(
+        h, "k_mf_row(final sweep)",
+        std::min(mf_grid(h->m, 256), wave_blocks((const void *)k_mf_row<T, MF_SWEEP_ZDOT>, 256)),
+        gd, gt, u, at, x, b, dinv, omega, nullptr, c, o.z, o.r, nullptr));
   else
-    MG_TRY(chain_launch(h, "k_mf_row(final sweep)", k_mf_row<T, MF_SWEEP_Z>, mf_grid(h->m, 256),
-                        256, h->E, h->m, h->edge, h->tet, gd, gt, u, at, x, b, dinv, omega, nullptr,
-                        c, o.z, o.r, nullptr));
+    MG_TRY(mf_row_launch<T, MF_SWEEP_Z>(
+        h, "k_mf_row(final sweep)", mf_grid(h->m, 256), gd, gt, u, at, x, b, dinv, omega, nullptr,
+        c, o.z, o.r, nullptr));
   return MGPBD_OK;
 }
 

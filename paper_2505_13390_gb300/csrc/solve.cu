@@ -86,22 +86,26 @@ __device__ __forceinline__ T xr_entry(double al, double &xi, double &ri, double 
   return bi;
 }
 
-template <class T>
+template <class T, class Gate>
 __device__ __forceinline__ void xr_update_body(int vb, int vn, int64_t n, double *x, double *r,
                                                const double *p, const double *q, const DotCtx &c,
-                                               T *bl, const T *dinv, T om, T *x0) {
+                                               T *bl, const T *dinv, T om, T *x0, Gate gate) {
   using V = typename Pair<T>::V;
+  const int64_t n2 = n / 2;
+  const int64_t k0 = vb * (int64_t)blockDim.x + threadIdx.x;
+  V dv = {};
+  if (x0 && k0 < n2) dv = reinterpret_cast<const V *>(dinv)[k0];
+  gate.open();
   const double al = c.sc->alpha;
   T acc = 0;
-  const int64_t n2 = n / 2;
-  for (int64_t k = vb * (int64_t)blockDim.x + threadIdx.x; k < n2;
-       k += (int64_t)vn * blockDim.x) {
+#pragma unroll 1
+  for (int64_t k = k0; k < n2; k += (int64_t)vn * blockDim.x) {
     double2 xv = reinterpret_cast<const double2 *>(x)[k];
     double2 rv = reinterpret_cast<const double2 *>(r)[k];
     const double2 pv = reinterpret_cast<const double2 *>(p)[k];
     const double2 qv = reinterpret_cast<const double2 *>(q)[k];
-    V dv = {};
-    if (x0) dv = reinterpret_cast<const V *>(dinv)[k];
+    if (x0 && k != k0) dv = reinterpret_cast<const V *>(dinv)[k];
+    if (gate.closed()) return;
     V bv, xv0;
     const T b0 = xr_entry<T>(al, xv.x, rv.x, pv.x, qv.x, dv.x, om, &bv.x, &xv0.x);
     const T b1 = xr_entry<T>(al, xv.y, rv.y, pv.y, qv.y, dv.y, om, &bv.y, &xv0.y);
@@ -112,6 +116,7 @@ __device__ __forceinline__ void xr_update_body(int vb, int vn, int64_t n, double
     if (bl) reinterpret_cast<V *>(bl)[k] = bv;
     if (x0) reinterpret_cast<V *>(x0)[k] = xv0;
   }
+  if (gate.closed()) return;
   if ((n & 1) && vb == 0 && threadIdx.x == 0) {
     const int64_t i = n - 1;
     double xi = x[i], ri = r[i];
@@ -129,9 +134,7 @@ __device__ __forceinline__ void xr_update_body(int vb, int vn, int64_t n, double
 template <class T>
 __global__ void k_xr_update(int64_t n, double *x, double *r, const double *p, const double *q,
                             DotCtx c, T *bl, const T *dinv, T om, T *x0) {
-  chain_wait();
-  if (is_done(c.sc)) return;
-  xr_update_body<T>(blockIdx.x, gridDim.x, n, x, r, p, q, c, bl, dinv, om, x0);
+  xr_update_body<T>(blockIdx.x, gridDim.x, n, x, r, p, q, c, bl, dinv, om, x0, ChainGate(c.sc));
 }
 
 // the same start of a V-cycle on its own: bl = r in the V-cycle's precision,
@@ -152,9 +155,11 @@ __global__ void k_top_prep(int64_t n, const double *r, T *bl, const T *dinv, T o
 // p = z + beta p, two entries per thread (16-byte loads; p and z are
 // 256-byte aligned); with pdf, p also as float-float pairs for the pair form
 // of A.p (params.ap_split)
+template <class Gate>
 __device__ __forceinline__ void p_update_body(int vb, int vn, int64_t n, double *p,
-                                              const double *z, const PcgScalars *sc,
-                                              float2 *pdf = nullptr) {
+                                              const double *z, const PcgScalars *sc, float2 *pdf,
+                                              Gate gate) {
+  gate.open();
   const double be = sc->beta;
   const int64_t n2 = n / 2, h2 = (n2 + 1) / 2;  // pairs k and k + h2 per thread
   double2 *p2 = reinterpret_cast<double2 *>(p);
@@ -168,6 +173,7 @@ __device__ __forceinline__ void p_update_body(int vb, int vn, int64_t n, double 
       pb = p2[k2];
       zb = z2[k2];
     }
+    if (gate.closed()) return;
     pa.x = fma(be, pa.x, za.x);
     pa.y = fma(be, pa.y, za.y);
     p2[k] = pa;
@@ -185,7 +191,7 @@ __device__ __forceinline__ void p_update_body(int vb, int vn, int64_t n, double 
       }
     }
   }
-  if ((n & 1) && vb == 0 && threadIdx.x == 0) {
+  if ((n & 1) && vb == 0 && threadIdx.x == 0 && !gate.closed()) {
     p[n - 1] = fma(be, p[n - 1], z[n - 1]);
     if (pdf) pdf[n - 1] = df_split(p[n - 1]);
   }
@@ -193,9 +199,7 @@ __device__ __forceinline__ void p_update_body(int vb, int vn, int64_t n, double 
 
 __global__ void k_p_update(int64_t n, double *p, const double *z, const PcgScalars *sc,
                            float2 *pdf) {
-  chain_wait();
-  if (is_done(sc)) return;
-  p_update_body(blockIdx.x, gridDim.x, n, p, z, sc, pdf);
+  p_update_body(blockIdx.x, gridDim.x, n, p, z, sc, pdf, ChainGate(sc));
 }
 
 __global__ void k_pcg_init(PcgScalars *sc, unsigned int *bar) {
@@ -996,7 +1000,8 @@ static mgpbd_status launch_tail(Handle *h, int first) {
 
 __global__ void kb_xr(const CohortMember *mem, const CohortBlock *blk) {
   COHORT_BLOCK;
-  xr_update_body<float>(vb, vn, M.m, M.x, M.r, M.p, M.q, M.c_rr, M.b0, M.dinv0, M.om0, M.x0);
+  xr_update_body<float>(vb, vn, M.m, M.x, M.r, M.p, M.q, M.c_rr, M.b0, M.dinv0, M.om0, M.x0,
+                        NoGate{});
 }
 
 __global__ void kb_restrict0(const CohortMember *mem, const CohortBlock *blk) {
@@ -1014,7 +1019,7 @@ __global__ void kb_prolong0(const CohortMember *mem, const CohortBlock *blk) {
 
 __global__ void kb_pupdate(const CohortMember *mem, const CohortBlock *blk) {
   COHORT_BLOCK;
-  p_update_body(vb, vn, M.m, M.p, M.z, M.sc);
+  p_update_body(vb, vn, M.m, M.p, M.z, M.sc, nullptr, NoGate{});
 }
 
 // The V-cycle below level 0 of every member in one cooperative launch, depth
