@@ -84,8 +84,7 @@ inline mgpbd_status alloc_n(Arena &a, T **p, size_t n) {
 // ---------------------------------------------------------------------------
 struct PcgScalars {
   double bnorm2;   // |b|^2
-  double rz;       // r.z of the current iteration
-  double rz_new;
+  double rz[2];    // r.z; iteration k's is in rz[k & 1]
   double pq;       // p.q
   double rr;       // r.r
   double alpha, beta;
@@ -204,6 +203,10 @@ struct Handle {
   unsigned int *gbar = nullptr;      // its grid barrier word
   long long wait_limit = 1ll << 24;  // polls a block waits at the barrier
   double *partials = nullptr;     // dot-product block partials
+  // p.q and r.z are left as block partials and folded by the kernel that needs
+  // them (x/r update, p update): the partials and their number
+  double *part_pq = nullptr, *part_rz = nullptr;
+  int n_pq = 0, n_rz = 0;
   unsigned int *counter = nullptr;
   // scratch for setup
   void *tmp = nullptr;

@@ -40,6 +40,8 @@ constexpr int kUStride = 3, kUStrideDf = 4;
 // one, its time is that of its dependent loads, and its 40 to 80 registers
 // cost nothing.  Above it the plain form's occupancy counts.
 constexpr int kEarlyRows = 1 << 17;
+// threads of the early vertex passes: small blocks, for more SMs (reduce.cuh)
+constexpr int kVertexThreads = 64;
 
 // slot of vertex v in each incident row (create time)
 __global__ void k_vslot(int N, int E, const int32_t *edge, const int32_t *tet, const int64_t *vptr,
@@ -527,9 +529,9 @@ enum {
 // row pass: y_i = sum_s g_{i,s}.u_{v_s} + alpha~_i x_i, then
 //   MF_SWEEP      out = x + omega D^-1 (b - y)
 //   MF_RESID      out = b - y
-//   MF_APPLY_DOT  out = y, with x.y folded into the PCG scalars (DOT_PQ)
+//   MF_APPLY_DOT  out = y, with x.y's block partials
 //   MF_SWEEP_Z    z = x + omega D^-1 (b - y) widened to FP64
-//   MF_SWEEP_ZDOT the same, with r.z folded into the PCG scalars
+//   MF_SWEEP_ZDOT the same, with r.z's block partials
 //   MF_RESID_MEMBER out[pos_i] = b - y for rows in an aggregate (the
 //                 residual in member order, for the restriction)
 // the row's result from y = J u + alpha~ x (MODE as above); acc collects the
@@ -741,8 +743,16 @@ mgpbd_status mf_create(Handle *h) {
 // the 3.68M-row block (14,375 blocks of rows) the cap measured 0.7% faster
 // per PCG iteration than 4,096 blocks and 2% faster than one block per 256
 // rows.
+// (the passes that end in a dot product run one resident wave of kDotThreads)
 static int mf_grid(int64_t rows, int threads) {
   return (int)std::max<int64_t>(1, std::min<int64_t>((rows + threads - 1) / threads, 8192));
+}
+
+// blocks of a row pass with a dot product (its partials are one per block)
+template <class T, int MODE>
+static int mf_dot_grid(int m) {
+  return std::min((m + kDotThreads - 1) / kDotThreads,
+                  wave_blocks((const void *)k_mf_row<T, MODE>, kDotThreads));
 }
 
 template <class T, int MODE>
@@ -751,9 +761,11 @@ static mgpbd_status mf_row_launch(Handle *h, const char *what, int blocks, const
                                   const T *dinv, T omega, T *out, const DotCtx &c, double *z,
                                   const double *rr, const int32_t *pos) {
   if (h->m <= kEarlyRows)
-    return chain_launch(h, what, k_mf_row_early<T, MODE>, blocks_for(h->m, 256), 256, h->E, h->m,
-                        h->edge, h->tet, gd, gt, u, at, x, b, dinv, omega, out, c, z, rr, pos);
-  return chain_launch(h, what, k_mf_row<T, MODE>, blocks, 256, h->E, h->m, h->edge, h->tet, gd,
+    return chain_launch(h, what, k_mf_row_early<T, MODE>, blocks_for(h->m, kDotThreads),
+                        kDotThreads, h->E, h->m, h->edge, h->tet, gd, gt, u, at, x, b, dinv,
+                        omega, out, c, z, rr, pos);
+  const bool dot = MODE == MF_APPLY_DOT || MODE == MF_SWEEP_ZDOT;
+  return chain_launch(h, what, k_mf_row<T, MODE>, blocks, dot ? kDotThreads : 256, h->E, h->m, h->edge, h->tet, gd,
                       gt, u, at, x, b, dinv, omega, out, c, z, rr, pos);
 }
 
@@ -876,11 +888,9 @@ void mf_cohort_grids(const Handle *h, int grid[CS_STEPS]) {
   const int g32 = h->force_vert32 ? h->force_vert32 : h->mf_g32;
   MF_G_DISPATCH(g64, (grid[CS_VERT64] = mf_vertex_blocks(h, GG)));
   MF_G_DISPATCH(g32, (grid[CS_VERT32] = mf_vertex_blocks(h, GG)));
-  grid[CS_ROW_PQ] = std::min(mf_grid(h->m, 256),
-                             wave_blocks((const void *)k_mf_row<double, MF_APPLY_DOT>, 256));
+  grid[CS_ROW_PQ] = mf_dot_grid<double, MF_APPLY_DOT>(h->m);
   grid[CS_ROW] = mf_grid(h->m, 256);
-  grid[CS_ROW_FINAL] = std::min(mf_grid(h->m, 256),
-                                wave_blocks((const void *)k_mf_row<float, MF_SWEEP_ZDOT>, 256));
+  grid[CS_ROW_FINAL] = mf_dot_grid<float, MF_SWEEP_ZDOT>(h->m);
 }
 
 mgpbd_status mf_cohort_step(int which, int sel, const CohortMember *d_mem,
@@ -890,7 +900,7 @@ mgpbd_status mf_cohort_step(int which, int sel, const CohortMember *d_mem,
       kb_vertex64<<<blocks, 256, 0, st>>>(d_mem, d_blk);
       break;
     case CS_ROW_PQ:
-      kb_row_pq<<<blocks, 256, 0, st>>>(d_mem, d_blk);
+      kb_row_pq<<<blocks, kDotThreads, 0, st>>>(d_mem, d_blk);
       break;
     case CS_VERT32:
       if (gv32 == 4 || gv32 == 8 || gv32 == 16) {
@@ -903,7 +913,7 @@ mgpbd_status mf_cohort_step(int which, int sel, const CohortMember *d_mem,
       kb_row<<<blocks, 256, 0, st>>>(d_mem, d_blk, sel);
       break;
     default:
-      kb_row_final<<<blocks, 256, 0, st>>>(d_mem, d_blk);
+      kb_row_final<<<blocks, kDotThreads, 0, st>>>(d_mem, d_blk);
       break;
   }
   MG_LAUNCH("kb_mf");
@@ -916,8 +926,8 @@ static mgpbd_status mf_vertex(Handle *h, const double *x, int G = 0, bool check_
   const PcgScalars *sc = check_done ? h->sc : nullptr;
   if (h->m <= kEarlyRows) {
     MF_G_DISPATCH(G, MG_TRY(chain_launch(h, "k_mf_vertex64", k_mf_vertex64_early<GG>,
-                                          blocks_for((int64_t)h->N * GG, 256), 256, h->N,
-                                          h->vorder, h->vptr, h->vrow, h->ginc64, h->w, x, h->u64,
+                                          blocks_for((int64_t)h->N * GG, kVertexThreads),
+                                          kVertexThreads, h->N, h->vorder, h->vptr, h->vrow, h->ginc64, h->w, x, h->u64,
                                           sc)));
     return MGPBD_OK;
   }
@@ -932,8 +942,8 @@ static mgpbd_status mf_vertex(Handle *h, const float *x, int G = 0, bool check_d
   const PcgScalars *sc = check_done ? h->sc : nullptr;
   if (h->m <= kEarlyRows) {
     MF_G_DISPATCH(G, MG_TRY(chain_launch(h, "k_mf_vertex32", k_mf_vertex32_early<GG>,
-                                          blocks_for((int64_t)h->N * GG, 256), 256, h->N,
-                                          h->vorder, h->vptr, h->ginc4, h->w32, x, h->u32, sc)));
+                                          blocks_for((int64_t)h->N * GG, kVertexThreads),
+                                          kVertexThreads, h->N, h->vorder, h->vptr, h->ginc4, h->w32, x, h->u32, sc)));
     return MGPBD_OK;
   }
   MF_G_DISPATCH(G, MG_TRY(chain_launch(h, "k_mf_vertex32", k_mf_vertex32<GG>,
@@ -994,17 +1004,18 @@ mgpbd_status mf_apply_pq_form(Handle *h, bool pairs, const double *p, double *q,
   if (pairs) {
     MG_TRY(mf_vertex(h, (const float2 *)h->p_df));
     const int grid =
-        std::min(mf_grid(h->m, 256), wave_blocks((const void *)k_mf_row_df, 256));
-    MG_TRY(chain_launch(h, "k_mf_row_df(A.p)", k_mf_row_df, grid, 256, h->E, h->m, h->edge, h->tet,
+        std::min((h->m + kDotThreads - 1) / kDotThreads,
+                 wave_blocks((const void *)k_mf_row_df, kDotThreads));
+    h->n_pq = grid;
+    MG_TRY(chain_launch(h, "k_mf_row_df(A.p)", k_mf_row_df, grid, kDotThreads, h->E, h->m, h->edge, h->tet,
                         h->gd32, h->gd_lo, h->gt32, h->gt_lo, h->u_hi, h->u_lo, h->at32, h->at_lo,
                         h->p_df, q, c));
     return MGPBD_OK;
   }
   MG_TRY(mf_vertex(h, p));
-  const int grid = std::min(mf_grid(h->m, 256),
-                            wave_blocks((const void *)k_mf_row<double, MF_APPLY_DOT>, 256));
+  h->n_pq = mf_dot_grid<double, MF_APPLY_DOT>(h->m);
   MG_TRY(mf_row_launch<double, MF_APPLY_DOT>(
-      h, "k_mf_row(A.p)", grid, h->gd, h->gt, h->u64, h->alpha_t, p, nullptr, nullptr, 0.0, q, c,
+      h, "k_mf_row(A.p)", h->n_pq, h->gd, h->gt, h->u64, h->alpha_t, p, nullptr, nullptr, 0.0, q, c,
       nullptr, nullptr, nullptr));
   return MGPBD_OK;
 }
@@ -1098,10 +1109,11 @@ mgpbd_status mf_level0_final(Handle *h, const T *x, const T *b, const T *dinv, T
   const T *at = dbl ? (const T *)h->alpha_t : (const T *)h->at32;
   DotCtx c = o.c;
   c.sc = h->sc;
+  if (o.dot) h->n_rz = mf_dot_grid<T, MF_SWEEP_ZDOT>(h->m);
   if (o.dot)
     MG_TRY(mf_row_launch<T, MF_SWEEP_ZDOT>(
         h, "k_mf_row(final sweep)",
-        std::min(mf_grid(h->m, 256), wave_blocks((const void *)k_mf_row<T, MF_SWEEP_ZDOT>, 256)),
+        h->n_rz,
         gd, gt, u, at, x, b, dinv, omega, nullptr, c, o.z, o.r, nullptr));
   else
     MG_TRY(mf_row_launch<T, MF_SWEEP_Z>(

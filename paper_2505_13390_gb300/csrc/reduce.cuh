@@ -3,22 +3,29 @@
 // Every dot product is a fixed-grid two-stage reduction: each block folds its
 // threads in a fixed order, the last block to finish folds the per-block
 // partials in block order and applies the next PCG recurrence step on the
-// device (dot_finalize).  Results are therefore identical run to run.
+// device (dot_finalize).  Results are therefore identical run to run.  The two
+// dot products whose result one kernel waits for right away, p.q and r.z, leave
+// only their partials (DOT_PART): every block of that kernel folds them itself,
+// in the same order, which costs it less than the fence, counter and re-read of
+// a last block cost the kernel before.
 #pragma once
 
 #include "common.cuh"
 
 namespace mg {
 
-constexpr int kDotThreads = 256;
+// Threads of the kernels that end in a dot product.  FP64 issues at about 1.6
+// lanes per clock and SM, so a warp's FP64 instruction holds its SM for 20
+// clocks: blocks of 128 spread the FP64 work of an instance of 20,000 rows over
+// every SM (256-row blocks left a third of them idle).
+constexpr int kDotThreads = 128;
 
 enum DotMode {
   DOT_STORE = 0,  // *out = s
   DOT_BNORM,      // |b|^2; zero right-hand side finishes at once
   DOT_RZ0,        // initial r.z
-  DOT_PQ,         // p.q and alpha
+  DOT_PART,       // block partials only (p.q, r.z)
   DOT_RR,         // r.r, iteration count and convergence test
-  DOT_RZ,         // new r.z and beta
   DOT_TR          // |b - A x|^2
 };
 
@@ -51,19 +58,10 @@ static __device__ void dot_finalize(const DotCtx &c, double s) {
       }
       break;
     case DOT_RZ0:
-      sc->rz = s;
+      sc->rz[0] = s;
       if (!(s > 0.0)) {
         sc->done = 1;
         sc->status = MGPBD_E_BREAKDOWN;
-      }
-      break;
-    case DOT_PQ:
-      sc->pq = s;
-      if (!(s > 0.0)) {
-        sc->done = 1;
-        sc->status = MGPBD_E_BREAKDOWN;
-      } else {
-        sc->alpha = sc->rz / s;
       }
       break;
     case DOT_RR:
@@ -80,19 +78,49 @@ static __device__ void dot_finalize(const DotCtx &c, double s) {
         sc->status = MGPBD_W_NOT_CONVERGED;
       }
       break;
-    case DOT_RZ:
-      if (!(s > 0.0)) {
-        sc->done = 1;
-        sc->status = MGPBD_E_BREAKDOWN;
-      } else {
-        sc->beta = s / sc->rz;
-        sc->rz = s;
-      }
-      break;
     case DOT_TR:
       sc->tr2 = s;
       break;
+    case DOT_PART:
+      break;
   }
+}
+
+// Sum of one value per thread of a block of kDotThreads: through shared memory
+// and one warp, nine FP64 additions instead of five per warp and a serial tail.
+// The result is in thread 0.
+static __device__ __forceinline__ double block_sum(double v) {
+  __shared__ double sd[kDotThreads];
+  sd[threadIdx.x] = v;
+  __syncthreads();
+  if (threadIdx.x >= 32) return 0.0;
+#pragma unroll
+  for (int k = 32; k < kDotThreads; k += 32) v += sd[threadIdx.x + k];
+  return warp_sum(v);
+}
+
+// sum over the partials of a reduction of vn blocks by one block, in a fixed
+// order whatever block does it; the result is in thread 0
+static __device__ __forceinline__ double fold_partials(const double *partials, int vn) {
+  double s = 0.0;
+  for (int b = threadIdx.x; b < vn; b += 4 * kDotThreads) {
+    double t[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      t[k] = b + k * kDotThreads < vn ? __ldcg(partials + b + k * kDotThreads) : 0.0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) s += t[k];
+  }
+  return block_sum(s);
+}
+
+// fold_partials with the result in every thread
+static __device__ __forceinline__ double fold_partials_all(const double *partials, int vn) {
+  __shared__ double all;
+  const double s = fold_partials(partials, vn);
+  if (threadIdx.x == 0) all = s;
+  __syncthreads();
+  return all;
 }
 
 // block reduce of one value per thread in a fixed order, then the last block
@@ -101,16 +129,11 @@ static __device__ void dot_finalize(const DotCtx &c, double s) {
 // instance's share of a launch that serves several instances (the partition
 // into blocks, and so every rounding, is the instance's own either way).
 static __device__ void block_dot_finish_vg(double v, const DotCtx &c, int vb, int vn) {
-  __shared__ double ws[32];
   __shared__ bool last;
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  v = warp_sum(v);
-  if (lane == 0) ws[wid] = v;
-  __syncthreads();
+  const double s = block_sum(v);
+  if (threadIdx.x == 0) c.partials[vb] = s;
+  if (c.mode == DOT_PART) return;
   if (threadIdx.x == 0) {
-    double s = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += ws[w];
-    c.partials[vb] = s;
     __threadfence();
     unsigned t = atomicAdd(c.counter, 1u);
     last = (t == (unsigned)vn - 1);
@@ -118,15 +141,8 @@ static __device__ void block_dot_finish_vg(double v, const DotCtx &c, int vb, in
   __syncthreads();
   if (!last) return;
   __threadfence();
-  double s = 0.0;
-  for (int b = threadIdx.x; b < vn; b += blockDim.x)
-    s += ((volatile double *)c.partials)[b];
-  s = warp_sum(s);
-  if (lane == 0) ws[wid] = s;
-  __syncthreads();
+  const double t = fold_partials(c.partials, vn);
   if (threadIdx.x == 0) {
-    double t = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += ws[w];
     dot_finalize(c, t);
     *c.counter = 0;
   }

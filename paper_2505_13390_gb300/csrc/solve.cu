@@ -26,10 +26,12 @@
 
 namespace mg {
 
-// blocks of a dot-product kernel over n entries: about 4 entries per thread,
-// at least two blocks per SM, at most the 4096 partials the handle holds
+// blocks of a dot-product kernel over n entries: two entries per thread up to
+// four blocks per SM, then about eight; at most the 4096 partials the handle holds
 static int dot_grid(int64_t n) {
-  return (int)std::min<int64_t>(4096, std::max<int64_t>(2 * num_sms(), (n + 1023) / 1024));
+  const int64_t two = (n + 2 * kDotThreads - 1) / (2 * kDotThreads);
+  const int64_t more = std::max<int64_t>(4 * num_sms(), (n + 1023) / 1024);
+  return (int)std::min<int64_t>(4096, std::max<int64_t>(1, std::min(two, more)));
 }
 
 static DotCtx make_ctx(Handle *h, int mode, double *out = nullptr) {
@@ -41,6 +43,18 @@ static DotCtx make_ctx(Handle *h, int mode, double *out = nullptr) {
   c.mode = mode;
   c.rtol = h->p.pcg_rtol;
   c.maxiter = h->p.pcg_maxiter;
+  return c;
+}
+
+// p.q and r.z, left as partials
+static DotCtx pq_ctx(Handle *h) {
+  DotCtx c = make_ctx(h, DOT_PART);
+  c.partials = h->part_pq;
+  return c;
+}
+static DotCtx rz_ctx(Handle *h) {
+  DotCtx c = make_ctx(h, DOT_PART);
+  c.partials = h->part_rz;
   return c;
 }
 
@@ -57,6 +71,7 @@ __global__ void k_dot(int64_t n, const double *x, const double *y, DotCtx c, int
   block_dot_finish(acc, c);
 }
 
+// alpha = r.z / p.q from p.q's partials (a breakdown p.q <= 0 ends the solve);
 // x += alpha p; r -= alpha q; then r.r (convergence test).  The start of the
 // next V-cycle is folded in: bl = r in the V-cycle's precision (MGPBD_MIXED)
 // and, with the Jacobi smoother, its first sweep from zero x0 = omega D^-1 r.
@@ -89,23 +104,47 @@ __device__ __forceinline__ T xr_entry(double al, double &xi, double &ri, double 
 template <class T, class Gate>
 __device__ __forceinline__ void xr_update_body(int vb, int vn, int64_t n, double *x, double *r,
                                                const double *p, const double *q, const DotCtx &c,
-                                               T *bl, const T *dinv, T om, T *x0, Gate gate) {
+                                               const double *part_pq, int n_pq, T *bl,
+                                               const T *dinv, T om, T *x0, Gate gate) {
   using V = typename Pair<T>::V;
+  PcgScalars *sc = c.sc;
   const int64_t n2 = n / 2;
   const int64_t k0 = vb * (int64_t)blockDim.x + threadIdx.x;
   V dv = {};
   if (x0 && k0 < n2) dv = reinterpret_cast<const V *>(dinv)[k0];
   gate.open();
-  const double al = c.sc->alpha;
+  // the first entries, beside the fold of p.q
+  double2 xv = {}, rv = {}, pv = {}, qv = {};
+  auto load = [&](int64_t k) {
+    xv = reinterpret_cast<const double2 *>(x)[k];
+    rv = reinterpret_cast<const double2 *>(r)[k];
+    pv = reinterpret_cast<const double2 *>(p)[k];
+    qv = reinterpret_cast<const double2 *>(q)[k];
+  };
+  if (k0 < n2) load(k0);
+  const double rz = sc->rz[sc->iters & 1];
+  const double pq = fold_partials_all(part_pq, n_pq);
+  if (gate.closed()) return;
+  if (!(pq > 0.0)) {
+    if (vb == 0 && threadIdx.x == 0) {
+      sc->pq = pq;
+      sc->status = MGPBD_E_BREAKDOWN;
+      sc->done = 1;
+    }
+    return;
+  }
+  const double al = rz / pq;
+  if (vb == 0 && threadIdx.x == 0) {
+    sc->pq = pq;
+    sc->alpha = al;
+  }
   T acc = 0;
 #pragma unroll 1
   for (int64_t k = k0; k < n2; k += (int64_t)vn * blockDim.x) {
-    double2 xv = reinterpret_cast<const double2 *>(x)[k];
-    double2 rv = reinterpret_cast<const double2 *>(r)[k];
-    const double2 pv = reinterpret_cast<const double2 *>(p)[k];
-    const double2 qv = reinterpret_cast<const double2 *>(q)[k];
-    if (x0 && k != k0) dv = reinterpret_cast<const V *>(dinv)[k];
-    if (gate.closed()) return;
+    if (k != k0) {
+      load(k);
+      if (x0) dv = reinterpret_cast<const V *>(dinv)[k];
+    }
     V bv, xv0;
     const T b0 = xr_entry<T>(al, xv.x, rv.x, pv.x, qv.x, dv.x, om, &bv.x, &xv0.x);
     const T b1 = xr_entry<T>(al, xv.y, rv.y, pv.y, qv.y, dv.y, om, &bv.y, &xv0.y);
@@ -116,7 +155,6 @@ __device__ __forceinline__ void xr_update_body(int vb, int vn, int64_t n, double
     if (bl) reinterpret_cast<V *>(bl)[k] = bv;
     if (x0) reinterpret_cast<V *>(x0)[k] = xv0;
   }
-  if (gate.closed()) return;
   if ((n & 1) && vb == 0 && threadIdx.x == 0) {
     const int64_t i = n - 1;
     double xi = x[i], ri = r[i];
@@ -133,8 +171,10 @@ __device__ __forceinline__ void xr_update_body(int vb, int vn, int64_t n, double
 
 template <class T>
 __global__ void k_xr_update(int64_t n, double *x, double *r, const double *p, const double *q,
-                            DotCtx c, T *bl, const T *dinv, T om, T *x0) {
-  xr_update_body<T>(blockIdx.x, gridDim.x, n, x, r, p, q, c, bl, dinv, om, x0, ChainGate(c.sc));
+                            DotCtx c, const double *part_pq, int n_pq, T *bl, const T *dinv,
+                            T om, T *x0) {
+  xr_update_body<T>(blockIdx.x, gridDim.x, n, x, r, p, q, c, part_pq, n_pq, bl, dinv, om, x0,
+                    ChainGate(c.sc));
 }
 
 // the same start of a V-cycle on its own: bl = r in the V-cycle's precision,
@@ -152,28 +192,50 @@ __global__ void k_top_prep(int64_t n, const double *r, T *bl, const T *dinv, T o
   }
 }
 
-// p = z + beta p, two entries per thread (16-byte loads; p and z are
-// 256-byte aligned); with pdf, p also as float-float pairs for the pair form
-// of A.p (params.ap_split)
+// beta = r.z / (r.z of the iteration before) from r.z's partials (a breakdown
+// r.z <= 0 ends the solve); p = z + beta p, two entries per thread (16-byte
+// loads; p and z are 256-byte aligned); with pdf, p also as float-float pairs
+// for the pair form of A.p (params.ap_split)
 template <class Gate>
 __device__ __forceinline__ void p_update_body(int vb, int vn, int64_t n, double *p,
-                                              const double *z, const PcgScalars *sc, float2 *pdf,
+                                              const double *z, PcgScalars *sc,
+                                              const double *part_rz, int n_rz, float2 *pdf,
                                               Gate gate) {
-  gate.open();
-  const double be = sc->beta;
   const int64_t n2 = n / 2, h2 = (n2 + 1) / 2;  // pairs k and k + h2 per thread
   double2 *p2 = reinterpret_cast<double2 *>(p);
   const double2 *z2 = reinterpret_cast<const double2 *>(z);
-  for (int64_t k = vb * (int64_t)blockDim.x + threadIdx.x; k < h2;
-       k += (int64_t)vn * blockDim.x) {
+  const int64_t k0 = vb * (int64_t)blockDim.x + threadIdx.x;
+  double2 pa = {}, za = {}, pb = {}, zb = {};
+  auto load = [&](int64_t k) {
+    pa = p2[k];
+    za = z2[k];
+    if (k + h2 < n2) {
+      pb = p2[k + h2];
+      zb = z2[k + h2];
+    }
+  };
+  gate.open();
+  if (k0 < h2) load(k0);  // beside the fold of r.z
+  const int it = sc->iters;
+  const double rz_old = sc->rz[(it - 1) & 1];
+  const double rz = fold_partials_all(part_rz, n_rz);
+  if (gate.closed()) return;
+  if (!(rz > 0.0)) {
+    if (vb == 0 && threadIdx.x == 0) {
+      sc->status = MGPBD_E_BREAKDOWN;
+      sc->done = 1;
+    }
+    return;
+  }
+  const double be = rz / rz_old;
+  if (vb == 0 && threadIdx.x == 0) {
+    sc->rz[it & 1] = rz;
+    sc->beta = be;
+  }
+  for (int64_t k = k0; k < h2; k += (int64_t)vn * blockDim.x) {
     const int64_t k2 = k + h2;
     const bool two = k2 < n2;
-    double2 pa = p2[k], za = z2[k], pb = {0.0, 0.0}, zb = {0.0, 0.0};
-    if (two) {
-      pb = p2[k2];
-      zb = z2[k2];
-    }
-    if (gate.closed()) return;
+    if (k != k0) load(k);
     pa.x = fma(be, pa.x, za.x);
     pa.y = fma(be, pa.y, za.y);
     p2[k] = pa;
@@ -191,15 +253,15 @@ __device__ __forceinline__ void p_update_body(int vb, int vn, int64_t n, double 
       }
     }
   }
-  if ((n & 1) && vb == 0 && threadIdx.x == 0 && !gate.closed()) {
+  if ((n & 1) && vb == 0 && threadIdx.x == 0) {
     p[n - 1] = fma(be, p[n - 1], z[n - 1]);
     if (pdf) pdf[n - 1] = df_split(p[n - 1]);
   }
 }
 
-__global__ void k_p_update(int64_t n, double *p, const double *z, const PcgScalars *sc,
-                           float2 *pdf) {
-  p_update_body(blockIdx.x, gridDim.x, n, p, z, sc, pdf, ChainGate(sc));
+__global__ void k_p_update(int64_t n, double *p, const double *z, PcgScalars *sc,
+                           const double *part_rz, int n_rz, float2 *pdf) {
+  p_update_body(blockIdx.x, gridDim.x, n, p, z, sc, part_rz, n_rz, pdf, ChainGate(sc));
 }
 
 __global__ void k_pcg_init(PcgScalars *sc, unsigned int *bar) {
@@ -207,7 +269,7 @@ __global__ void k_pcg_init(PcgScalars *sc, unsigned int *bar) {
   sc->done = 0;
   sc->iters = 0;
   sc->status = MGPBD_W_NOT_CONVERGED;
-  sc->rz = sc->pq = sc->rr = sc->alpha = sc->beta = sc->tr2 = 0.0;
+  sc->rz[0] = sc->rz[1] = sc->pq = sc->rr = sc->alpha = sc->beta = sc->tr2 = 0.0;
 }
 
 template <class D>
@@ -784,6 +846,12 @@ int group_for(const Handle *h, const Level &L, bool fp64) {
   return g ? g : group_rule(L, fp64);
 }
 
+// Threads per block of the V-cycle's row kernels for `items` threads' work:
+// 64 while blocks of 256 would leave SMs idle (a level of 1,600 rows with 16
+// lanes each then spreads over every SM, which matters most for the FP64 ones),
+// else 256.
+static int spread(int64_t items) { return items >= 512 * (int64_t)num_sms() ? 256 : 64; }
+
 static int row_blocks(int64_t rows, int G, int th = 256) {
   int64_t groups_per_block = th / G;
   int64_t b = (rows + groups_per_block - 1) / groups_per_block;
@@ -794,8 +862,13 @@ static int row_blocks(int64_t rows, int G, int th = 256) {
 // grids of the kernels that end in a dot product: one resident wave at most
 template <int G>
 static int spmv_pq_blocks(int m) {
-  return std::min(row_blocks(m, G),
-                  wave_blocks((const void *)k_spmv_pq<G, double, double>, 256));
+  return std::min(row_blocks(m, G, kDotThreads),
+                  wave_blocks((const void *)k_spmv_pq<G, double, double>, kDotThreads));
+}
+// p update: four entries per thread, at most sixteen blocks per SM (every block
+// folds r.z's partials)
+static int p_blocks(int m) {
+  return std::min(blocks_for(std::max(1, (m / 2 + 1) / 2), kDotThreads), 16 * num_sms());
 }
 template <class T>
 static int xr_blocks(int m) {
@@ -1000,8 +1073,8 @@ static mgpbd_status launch_tail(Handle *h, int first) {
 
 __global__ void kb_xr(const CohortMember *mem, const CohortBlock *blk) {
   COHORT_BLOCK;
-  xr_update_body<float>(vb, vn, M.m, M.x, M.r, M.p, M.q, M.c_rr, M.b0, M.dinv0, M.om0, M.x0,
-                        NoGate{});
+  xr_update_body<float>(vb, vn, M.m, M.x, M.r, M.p, M.q, M.c_rr,
+                        M.c_pq.partials, M.grid[CS_ROW_PQ], M.b0, M.dinv0, M.om0, M.x0, NoGate{});
 }
 
 __global__ void kb_restrict0(const CohortMember *mem, const CohortBlock *blk) {
@@ -1019,7 +1092,8 @@ __global__ void kb_prolong0(const CohortMember *mem, const CohortBlock *blk) {
 
 __global__ void kb_pupdate(const CohortMember *mem, const CohortBlock *blk) {
   COHORT_BLOCK;
-  p_update_body(vb, vn, M.m, M.p, M.z, M.sc, nullptr, NoGate{});
+  p_update_body(vb, vn, M.m, M.p, M.z, M.sc, M.c_rz.partials, M.grid[CS_ROW_FINAL], nullptr,
+                NoGate{});
 }
 
 // The V-cycle below level 0 of every member in one cooperative launch, depth
@@ -1188,9 +1262,9 @@ mgpbd_status cohort_build(Cohort *c) {
     M.p = h->pp;
     M.q = h->pq;
     M.sc = h->sc;
-    M.c_pq = make_ctx(h, DOT_PQ);
+    M.c_pq = pq_ctx(h);
     M.c_rr = make_ctx(h, DOT_RR);
-    M.c_rz = make_ctx(h, DOT_RZ);
+    M.c_rz = rz_ctx(h);
     M.b0 = (float *)L0.b;
     M.x0 = (float *)L0.x;
     M.x20 = (float *)L0.x2;
@@ -1234,7 +1308,7 @@ mgpbd_status cohort_build(Cohort *c) {
     M.grid[CS_XR] = xr_blocks<float>(m);
     M.grid[CS_RESTRICT] = blocks_for((int64_t)L0.n_agg * 32, 256);
     M.grid[CS_PROLONG] = blocks_for((m + kProlongRows - 1) / kProlongRows, 256);
-    M.grid[CS_PUPD] = blocks_for(std::max(1, (m / 2 + 1) / 2), 256);
+    M.grid[CS_PUPD] = p_blocks(m);
     c->gens[k] = h->gen;
   }
   c->gv32 = mem.empty() ? 0 : mem[0].gv32;
@@ -1317,7 +1391,7 @@ static mgpbd_status cohort_iteration(Cohort *c) {
   MG_TRY(mf(CS_ROW, 2));
   MG_TRY(mf(CS_VERT32, 0));
   MG_TRY(mf(CS_ROW_FINAL, 0));
-  kb_pupdate<<<c->blocks[CS_PUPD], 256, 0, st>>>(m, blk(CS_PUPD));
+  kb_pupdate<<<c->blocks[CS_PUPD], kDotThreads, 0, st>>>(m, blk(CS_PUPD));
   MG_LAUNCH("kb_pupdate");
   return MGPBD_OK;
 }
@@ -1372,8 +1446,8 @@ static mgpbd_status vcycle_level(Handle *h, int l, const T *b_in, bool x0_ready 
   const int n = L.n;
   T *x = (T *)L.x;
   if (l == h->L - 1) {
-    MG_TRY(chain_launch(h, "k_coarse_apply", k_coarse_apply<T>, blocks_for((int64_t)n * 32, 256),
-                        256, n, h->cinv, b_in, x, sc));
+    MG_TRY(chain_launch(h, "k_coarse_apply", k_coarse_apply<T>,
+                        blocks_for((int64_t)n * 32, spread(32ll * n)), spread(32ll * n), n, h->cinv, b_in, x, sc));
     return MGPBD_OK;
   }
   const int G = group_for(h, L, sizeof(T) == 8);
@@ -1404,8 +1478,9 @@ static mgpbd_status vcycle_level(Handle *h, int l, const T *b_in, bool x0_ready 
   const bool cheb = h->p.smoother == MGPBD_SMOOTH_CHEBYSHEV;
   auto apply = [&](const T *v, T *y) -> mgpbd_status {
     if (mf) return mf_level0<T>(h, kMfApply, v, b_in, dinv, om, y);
-    DISPATCH_G(G, MG_TRY(chain_launch(h, "k_spmv_plain", k_spmv_plain<GG, T>, row_blocks(n, GG),
-                                      256, n, L.ptr, L.col, val, v, y, sc)));
+    DISPATCH_G(G, MG_TRY(chain_launch(h, "k_spmv_plain", k_spmv_plain<GG, T>,
+                                      row_blocks(n, GG, spread(n * (int64_t)GG)),
+                                      spread(n * (int64_t)GG), n, L.ptr, L.col, val, v, y, sc)));
     return MGPBD_OK;
   };
   // (from_zero: x = 0 on entry, so A x = 0 needs no product)
@@ -1415,12 +1490,12 @@ static mgpbd_status vcycle_level(Handle *h, int l, const T *b_in, bool x0_ready 
     double rho = 1.0 / sigma;
     T *t = (T *)L.t, *d = x2;
     if (!from_zero) MG_TRY(apply(x, t));
-    MG_TRY(chain_launch(h, "k_cheb_start", k_cheb_start<T>, blocks_for(n, 256), 256, n, b_in,
+    MG_TRY(chain_launch(h, "k_cheb_start", k_cheb_start<T>, blocks_for(n, spread(n)), spread(n), n, b_in,
                         from_zero ? nullptr : t, dinv, (T)(1.0 / theta), r, d, x, sc));
     for (int k = 1; k < h->p.smooth_sweeps; ++k) {
       MG_TRY(apply(d, t));
       double rho2 = 1.0 / (2.0 * sigma - rho);
-      MG_TRY(chain_launch(h, "k_cheb_step", k_cheb_step<T>, blocks_for(n, 256), 256, n, t, dinv,
+      MG_TRY(chain_launch(h, "k_cheb_step", k_cheb_step<T>, blocks_for(n, spread(n)), spread(n), n, t, dinv,
                           (T)(rho2 * rho), (T)(2.0 * rho2 / delta), r, d, x, sc));
       rho = rho2;
     }
@@ -1432,15 +1507,17 @@ static mgpbd_status vcycle_level(Handle *h, int l, const T *b_in, bool x0_ready 
     MG_CUDA(cudaMemsetAsync(x, 0, sizeof(T) * n, h->stream));
     MG_TRY(gs_sweeps(false));
   } else if (!x0_ready) {
-    MG_TRY(chain_launch(h, "k_jacobi0", k_jacobi0<T>, blocks_for(n, 256), 256, n, b_in, dinv, om, x,
-                        sc));
+    MG_TRY(chain_launch(h, "k_jacobi0", k_jacobi0<T>, blocks_for(n, spread(n)), spread(n), n, b_in,
+                        dinv, om, x, sc));
   }
   for (int s = 1; s < h->p.smooth_sweeps && !gs && !cheb; ++s) {
     if (l == 0) MG_TRY(prof_begin(h));
     if (mf) {
       MG_TRY(mf_level0<T>(h, kMfSweep, x, b_in, dinv, om, x2));
     } else {
-      DISPATCH_G(G, MG_TRY(chain_launch(h, "k_jacobi", k_jacobi<GG, T>, row_blocks(n, GG), 256, n,
+      DISPATCH_G(G, MG_TRY(chain_launch(h, "k_jacobi", k_jacobi<GG, T>,
+                                        row_blocks(n, GG, spread(n * (int64_t)GG)),
+                                        spread(n * (int64_t)GG), n,
                                         L.ptr, L.col, val, dinv, om, b_in, x, x2, sc)));
     }
     if (l == 0) MG_TRY(prof_end(h));
@@ -1454,19 +1531,24 @@ static mgpbd_status vcycle_level(Handle *h, int l, const T *b_in, bool x0_ready 
     // the residual written in member order, the restriction streaming it
     MG_TRY(mf_level0<T>(h, kMfResidMember, x, b_in, dinv, om, r));
     MG_TRY(chain_launch(h, "k_restrict_member", k_restrict_member<T>,
-                        blocks_for((int64_t)L.n_agg * 32, 256), 256, L.n_agg, L.mptr,
+                        blocks_for(32ll * L.n_agg, spread(32ll * L.n_agg)),
+                        spread(32ll * L.n_agg), L.n_agg, L.mptr,
                         (const T *)L.Pm, r, (T *)Lc.b, sc, c_jac ? dinvs<T>(Lc) : nullptr,
                         (T)Lc.omega, c_jac ? (T *)Lc.x : nullptr));
   } else if (mf) {
     MG_TRY(mf_level0<T>(h, kMfResid, x, b_in, dinv, om, r));
-    MG_TRY(chain_launch(h, "k_restrict", k_restrict<T>, blocks_for((int64_t)L.n_agg * 32, 256), 256,
-                        L.n_agg, nk, L.mptr, L.mrow, Ps<T>(L), r, (T *)Lc.b, sc,
+    MG_TRY(chain_launch(h, "k_restrict", k_restrict<T>,
+                        blocks_for(32ll * L.n_agg, spread(32ll * L.n_agg)),
+                        spread(32ll * L.n_agg), L.n_agg, nk, L.mptr, L.mrow, Ps<T>(L), r, (T *)Lc.b, sc,
                         c_jac ? dinvs<T>(Lc) : nullptr, (T)Lc.omega, c_jac ? (T *)Lc.x : nullptr));
   } else {
-    DISPATCH_G(G, MG_TRY(chain_launch(h, "k_resid", k_resid<GG, T>, row_blocks(n, GG), 256, n,
+    DISPATCH_G(G, MG_TRY(chain_launch(h, "k_resid", k_resid<GG, T>,
+                                      row_blocks(n, GG, spread(n * (int64_t)GG)),
+                                      spread(n * (int64_t)GG), n,
                                       L.ptr, L.col, val, b_in, x, r, sc)));
-    MG_TRY(chain_launch(h, "k_restrict", k_restrict<T>, blocks_for((int64_t)L.n_agg * 32, 256), 256,
-                        L.n_agg, nk, L.mptr, L.mrow, Ps<T>(L), r, (T *)Lc.b, sc,
+    MG_TRY(chain_launch(h, "k_restrict", k_restrict<T>,
+                        blocks_for(32ll * L.n_agg, spread(32ll * L.n_agg)),
+                        spread(32ll * L.n_agg), L.n_agg, nk, L.mptr, L.mrow, Ps<T>(L), r, (T *)Lc.b, sc,
                         c_jac ? dinvs<T>(Lc) : nullptr, (T)Lc.omega, c_jac ? (T *)Lc.x : nullptr));
   }
   const T *xc = (const T *)Lc.x;  // where the coarser level leaves its result
@@ -1478,8 +1560,8 @@ static mgpbd_status vcycle_level(Handle *h, int l, const T *b_in, bool x0_ready 
   }
   if (nk == 1)
     MG_TRY(chain_launch(h, "k_prolong", k_prolong<T>,
-                        blocks_for((n + kProlongRows - 1) / kProlongRows, 256), 256, n, L.agg,
-                        Ps<T>(L), xc, x, sc));
+                        blocks_for((n + kProlongRows - 1) / kProlongRows, spread(n / kProlongRows)),
+                        spread(n / kProlongRows), n, L.agg, Ps<T>(L), xc, x, sc));
   else
     MG_TRY(chain_launch(h, "k_prolong", k_prolong_k<T>, blocks_for(n, 256), 256, n, nk, L.agg,
                         Ps<T>(L), (const T *)Lc.x, x, sc));
@@ -1496,7 +1578,9 @@ static mgpbd_status vcycle_level(Handle *h, int l, const T *b_in, bool x0_ready 
     if (mf) {
       MG_TRY(mf_level0<T>(h, kMfSweep, x, b_in, dinv, om, x2));
     } else {
-      DISPATCH_G(G, MG_TRY(chain_launch(h, "k_jacobi", k_jacobi<GG, T>, row_blocks(n, GG), 256, n,
+      DISPATCH_G(G, MG_TRY(chain_launch(h, "k_jacobi", k_jacobi<GG, T>,
+                                        row_blocks(n, GG, spread(n * (int64_t)GG)),
+                                        spread(n * (int64_t)GG), n,
                                         L.ptr, L.col, val, dinv, om, b_in, x, x2, sc)));
     }
     if (l == 0) MG_TRY(prof_end(h));
@@ -1511,11 +1595,10 @@ static mgpbd_status vcycle_level(Handle *h, int l, const T *b_in, bool x0_ready 
 
 static mgpbd_status launch_dot(Handle *h, const double *x, const double *y, int64_t n, int mode,
                                int check_done, double *out = nullptr) {
-  DotCtx c = make_ctx(h, mode, out);
-  MG_TRY(chain_launch(h, "k_dot", k_dot,
-                      std::min(dot_grid(n), wave_blocks((const void *)k_dot, kDotThreads)),
-                      kDotThreads, n, x, y, c, check_done));
-  return MGPBD_OK;
+  const DotCtx c = mode == DOT_PART ? rz_ctx(h) : make_ctx(h, mode, out);
+  const int blocks = std::min(dot_grid(n), wave_blocks((const void *)k_dot, kDotThreads));
+  if (mode == DOT_PART) h->n_rz = blocks;
+  return chain_launch(h, "k_dot", k_dot, blocks, kDotThreads, n, x, y, c, check_done);
 }
 
 // level 0 starts its V-cycle with a Jacobi sweep from zero (not the coarsest)
@@ -1536,7 +1619,7 @@ static mgpbd_status vcycle_top(Handle *h, const double *r, double *z, bool prepa
   o.r = r;
   o.z = z;
   o.dot = dot_mode >= 0;
-  o.c = make_ctx(h, o.dot ? dot_mode : DOT_STORE);
+  o.c = dot_mode == DOT_PART ? rz_ctx(h) : make_ctx(h, o.dot ? dot_mode : DOT_STORE);
   bool zw = false;
   if (h->p.precision == MGPBD_MIXED) {
     if (!prepared) {
@@ -1546,7 +1629,7 @@ static mgpbd_status vcycle_top(Handle *h, const double *r, double *z, bool prepa
     }
     MG_TRY(vcycle_level<float>(h, 0, (const float *)L.b, jac, &o, &zw));
     if (!zw) {
-      MG_TRY(chain_launch(h, "k_convert", k_convert<float, double>, blocks_for(m, 256), 256, m,
+      MG_TRY(chain_launch(h, "k_convert", k_convert<float, double>, blocks_for(m, spread(m)), spread(m), m,
                           (const float *)L.x, z, h->sc));
     }
   } else {
@@ -1556,7 +1639,7 @@ static mgpbd_status vcycle_top(Handle *h, const double *r, double *z, bool prepa
     }
     MG_TRY(vcycle_level<double>(h, 0, r, jac, &o, &zw));
     if (!zw) {
-      MG_TRY(chain_launch(h, "k_convert", k_convert<double, double>, blocks_for(m, 256), 256, m,
+      MG_TRY(chain_launch(h, "k_convert", k_convert<double, double>, blocks_for(m, spread(m)), spread(m), m,
                           (const double *)L.x, z, h->sc));
     }
   }
@@ -1581,8 +1664,7 @@ mgpbd_status apply_level0(Handle *h, int form, const double *x, double *y) {
   if (form == 0) {
     const int G = group_for(h, L, true);
     DISPATCH_G(G, MG_TRY(chain_launch(h, "k_spmv_pq", k_spmv_pq<GG, double, double>,
-                                      spmv_pq_blocks<GG>(m),
-                                      256, m, L.ptr, L.col, L.val, x, y, c)));
+                                      spmv_pq_blocks<GG>(m), kDotThreads, m, L.ptr, L.col, L.val, x, y, c)));
     return MGPBD_OK;
   }
   if (form == 2) MG_TRY(mf_split(h, x, h->p_df, m));
@@ -1599,7 +1681,7 @@ static mgpbd_status pcg_iteration(Handle *h, double *x) {
   const int m = h->m;
   double *r = h->pr, *z = h->pz, *p = h->pp, *q = h->pq;
   const int G = group_for(h, L, true);
-  DotCtx cpq = make_ctx(h, DOT_PQ);
+  DotCtx cpq = pq_ctx(h);
   // A.p is part of the Krylov recurrence, not of the preconditioner, and stays
   // FP64 in both modes: rounding A's values to FP32 perturbs entries of size
   // ~1e4 by ~1e-3, far above alpha~ (~1e-7), and the FP32 operator is then
@@ -1611,8 +1693,8 @@ static mgpbd_status pcg_iteration(Handle *h, double *x) {
     MG_TRY(mf_apply_pq(h, p, q, cpq));
   } else {
     DISPATCH_G(G, MG_TRY(chain_launch(h, "k_spmv_pq", k_spmv_pq<GG, double, double>,
-                                      spmv_pq_blocks<GG>(m),
-                                      256, m, L.ptr, L.col, L.val, p, q, cpq)));
+                                      h->n_pq = spmv_pq_blocks<GG>(m), kDotThreads, m, L.ptr,
+                                      L.col, L.val, p, q, cpq)));
   }
   MG_TRY(prof_end(h, PROF_AP));
   // the update also starts the V-cycle (right-hand side, first Jacobi sweep)
@@ -1620,16 +1702,17 @@ static mgpbd_status pcg_iteration(Handle *h, double *x) {
   if (h->p.precision == MGPBD_MIXED)
     MG_TRY(chain_launch(h, "k_xr_update", k_xr_update<float>,
                         xr_blocks<float>(m),
-                        kDotThreads, m, x, r, p, q, make_ctx(h, DOT_RR), (float *)L.b, L.dinv32,
+                        kDotThreads, m, x, r, p, q, make_ctx(h, DOT_RR), h->part_pq, h->n_pq,
+                        (float *)L.b, L.dinv32,
                         (float)L.omega, jac ? (float *)L.x : nullptr));
   else
     MG_TRY(chain_launch(h, "k_xr_update", k_xr_update<double>,
                         xr_blocks<double>(m),
-                        kDotThreads, m, x, r, p, q, make_ctx(h, DOT_RR), nullptr, L.dinv, L.omega,
+                        kDotThreads, m, x, r, p, q, make_ctx(h, DOT_RR), h->part_pq, h->n_pq,
+                        nullptr, L.dinv, L.omega,
                         jac ? (double *)L.x : nullptr));
-  MG_TRY(vcycle_top(h, r, z, true, DOT_RZ));
-  MG_TRY(chain_launch(h, "k_p_update", k_p_update, blocks_for(std::max(1, (m / 2 + 1) / 2), 256),
-                      256, m, p, z, h->sc, h->p.ap_split ? h->p_df : nullptr));
+  MG_TRY(vcycle_top(h, r, z, true, DOT_PART));
+  MG_TRY(chain_launch(h, "k_p_update", k_p_update, p_blocks(m), kDotThreads, m, p, z, h->sc, h->part_rz, h->n_rz, h->p.ap_split ? h->p_df : nullptr));
   return MGPBD_OK;
 }
 
@@ -1747,8 +1830,9 @@ mgpbd_status pcg_solve(Handle *h, const double *b, double *x, mgpbd_solve_info *
 mgpbd_status pcg_finish(Handle *h, const double *b, double *x, mgpbd_solve_info *info) {
   const int m = h->m;
   memset(info, 0, sizeof(*info));
-  k_true_resid<<<std::min(row_blocks(m, 4), wave_blocks((const void *)k_true_resid, 256)), 256, 0,
-                 h->stream>>>(
+  k_true_resid<<<std::min(row_blocks(m, 4, kDotThreads),
+                          wave_blocks((const void *)k_true_resid, kDotThreads)),
+                 kDotThreads, 0, h->stream>>>(
       m, h->lev[0].ptr, h->lev[0].col, h->lev[0].val, x, b, make_ctx(h, DOT_TR));
   MG_LAUNCH("k_true_resid");
   MG_CUDA(cudaMemcpyAsync(h->sc_host, h->sc, sizeof(PcgScalars), cudaMemcpyDeviceToHost,
