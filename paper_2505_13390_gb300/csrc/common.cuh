@@ -89,10 +89,12 @@ struct PcgScalars {
   double rr;       // r.r
   double alpha, beta;
   double tr2;      // |b - A x|^2 (true residual)
+  double thr2;     // (rtol |b|)^2: r.r at or below it has converged
   int done;        // 1 once converged or failed
-  int iters;       // PCG iterations taken
+  // PCG iterations taken: x/r updates, and p updates.  Each kernel reads the
+  // other one's count, so that no block reads what another writes.
+  int iters, p_updates;
   int status;      // MGPBD_OK / MGPBD_W_NOT_CONVERGED / MGPBD_E_BREAKDOWN
-  int pad;
 };
 
 // ---------------------------------------------------------------------------
@@ -203,10 +205,11 @@ struct Handle {
   unsigned int *gbar = nullptr;      // its grid barrier word
   long long wait_limit = 1ll << 24;  // polls a block waits at the barrier
   double *partials = nullptr;     // dot-product block partials
-  // p.q and r.z are left as block partials and folded by the kernel that needs
-  // them (x/r update, p update): the partials and their number
+  // p.q, and r.z beside r.r (in `partials`), are left as block partials and
+  // folded by the kernel that needs them (x/r update, p update): the partials
+  // and their number
   double *part_pq = nullptr, *part_rz = nullptr;
-  int n_pq = 0, n_rz = 0;
+  int n_pq = 0, n_rz = 0, n_rr = 0;
   unsigned int *counter = nullptr;
   // scratch for setup
   void *tmp = nullptr;

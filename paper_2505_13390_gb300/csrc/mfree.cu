@@ -713,6 +713,10 @@ mgpbd_status mf_create(Handle *h) {
   k_vslot<<<blocks_for(h->N, 128), 128, 0, h->stream>>>(h->N, h->E, h->edge, h->tet, h->vptr,
                                                        h->vrow, h->vslot);
   MG_LAUNCH("k_vslot");
+  // FP64 lanes per vertex until the autotuner says otherwise: four (fewest FP64
+  // additions), but on small instances of long incidence lists (tet meshes:
+  // about thirty) eight, so that most lists are one batch of loads
+  if (h->m <= kEarlyRows && ninc > 16 * (int64_t)h->N) h->mf_g64 = 8;
   // Vertex-pass order: within windows of kOrderWindow consecutive vertices,
   // by incidence count (then id).  A G-lane group loops over its vertex's
   // incidences, so a warp costs its longest vertex; neighbouring vertices of
@@ -765,8 +769,8 @@ static mgpbd_status mf_row_launch(Handle *h, const char *what, int blocks, const
                         kDotThreads, h->E, h->m, h->edge, h->tet, gd, gt, u, at, x, b, dinv,
                         omega, out, c, z, rr, pos);
   const bool dot = MODE == MF_APPLY_DOT || MODE == MF_SWEEP_ZDOT;
-  return chain_launch(h, what, k_mf_row<T, MODE>, blocks, dot ? kDotThreads : 256, h->E, h->m, h->edge, h->tet, gd,
-                      gt, u, at, x, b, dinv, omega, out, c, z, rr, pos);
+  return chain_launch(h, what, k_mf_row<T, MODE>, blocks, dot ? kDotThreads : 256, h->E, h->m,
+                      h->edge, h->tet, gd, gt, u, at, x, b, dinv, omega, out, c, z, rr, pos);
 }
 
 mgpbd_status mf_prepare(Handle *h) {
@@ -927,8 +931,8 @@ static mgpbd_status mf_vertex(Handle *h, const double *x, int G = 0, bool check_
   if (h->m <= kEarlyRows) {
     MF_G_DISPATCH(G, MG_TRY(chain_launch(h, "k_mf_vertex64", k_mf_vertex64_early<GG>,
                                           blocks_for((int64_t)h->N * GG, kVertexThreads),
-                                          kVertexThreads, h->N, h->vorder, h->vptr, h->vrow, h->ginc64, h->w, x, h->u64,
-                                          sc)));
+                                          kVertexThreads, h->N, h->vorder, h->vptr, h->vrow,
+                                          h->ginc64, h->w, x, h->u64, sc)));
     return MGPBD_OK;
   }
   MF_G_DISPATCH(G, MG_TRY(chain_launch(h, "k_mf_vertex64", k_mf_vertex64<GG>,
@@ -943,7 +947,8 @@ static mgpbd_status mf_vertex(Handle *h, const float *x, int G = 0, bool check_d
   if (h->m <= kEarlyRows) {
     MF_G_DISPATCH(G, MG_TRY(chain_launch(h, "k_mf_vertex32", k_mf_vertex32_early<GG>,
                                           blocks_for((int64_t)h->N * GG, kVertexThreads),
-                                          kVertexThreads, h->N, h->vorder, h->vptr, h->ginc4, h->w32, x, h->u32, sc)));
+                                          kVertexThreads, h->N, h->vorder, h->vptr, h->ginc4,
+                                          h->w32, x, h->u32, sc)));
     return MGPBD_OK;
   }
   MF_G_DISPATCH(G, MG_TRY(chain_launch(h, "k_mf_vertex32", k_mf_vertex32<GG>,
@@ -964,15 +969,18 @@ static mgpbd_status mf_vertex(Handle *h, const float2 *x, int G = 0, bool check_
   return MGPBD_OK;
 }
 
-// Times the vertex pass with 4, 8 and 16 lanes per vertex in each precision
-// the solve uses and keeps the fastest (params.autotune); with ap_split the
-// A.p's lanes are timed on its pair form.
+// Times the vertex pass with 4, 8 and, in FP32, 16 lanes per vertex in each
+// precision the solve uses and keeps the fastest (params.autotune); with
+// ap_split the A.p's lanes are timed on its pair form.  Sixteen FP64 lanes
+// never pay beyond the timing of one pass: they add as often as they multiply
+// (five additions per lane for two incidences of a tet vertex), which takes
+// FP64 issue slots from every kernel beside it.
 mgpbd_status mf_autotune(Handle *h) {
   if (h->m == 0 || !h->vslot) return MGPBD_OK;
-  auto pick = [&](auto *x, int *out) -> mgpbd_status {
+  auto pick = [&](auto *x, int n_cands, int *out) -> mgpbd_status {
     const int cands[3] = {4, 8, 16};
     float best = 1e30f;
-    for (int c = 0; c < 3; ++c) {
+    for (int c = 0; c < n_cands; ++c) {
       for (int rep = 0; rep < 5; ++rep) {
         MG_TRY(evict_l2(h));
         MG_CUDA(cudaEventRecord(h->ev0, h->stream));
@@ -990,10 +998,10 @@ mgpbd_status mf_autotune(Handle *h) {
     return MGPBD_OK;
   };
   if (h->p.ap_split)
-    MG_TRY(pick((const float2 *)h->p_df, &h->mf_g64));
+    MG_TRY(pick((const float2 *)h->p_df, 2, &h->mf_g64));
   else
-    MG_TRY(pick((const double *)h->pr, &h->mf_g64));
-  if (h->p.precision == MGPBD_MIXED) MG_TRY(pick((const float *)h->lev[0].b, &h->mf_g32));
+    MG_TRY(pick((const double *)h->pr, 2, &h->mf_g64));
+  if (h->p.precision == MGPBD_MIXED) MG_TRY(pick((const float *)h->lev[0].b, 3, &h->mf_g32));
   return MGPBD_OK;
 }
 
@@ -1007,7 +1015,8 @@ mgpbd_status mf_apply_pq_form(Handle *h, bool pairs, const double *p, double *q,
         std::min((h->m + kDotThreads - 1) / kDotThreads,
                  wave_blocks((const void *)k_mf_row_df, kDotThreads));
     h->n_pq = grid;
-    MG_TRY(chain_launch(h, "k_mf_row_df(A.p)", k_mf_row_df, grid, kDotThreads, h->E, h->m, h->edge, h->tet,
+    MG_TRY(chain_launch(h, "k_mf_row_df(A.p)", k_mf_row_df, grid, kDotThreads, h->E, h->m,
+                        h->edge, h->tet,
                         h->gd32, h->gd_lo, h->gt32, h->gt_lo, h->u_hi, h->u_lo, h->at32, h->at_lo,
                         h->p_df, q, c));
     return MGPBD_OK;

@@ -3,11 +3,11 @@
 // Every dot product is a fixed-grid two-stage reduction: each block folds its
 // threads in a fixed order, the last block to finish folds the per-block
 // partials in block order and applies the next PCG recurrence step on the
-// device (dot_finalize).  Results are therefore identical run to run.  The two
-// dot products whose result one kernel waits for right away, p.q and r.z, leave
-// only their partials (DOT_PART): every block of that kernel folds them itself,
-// in the same order, which costs it less than the fence, counter and re-read of
-// a last block cost the kernel before.
+// device (dot_finalize).  Results are therefore identical run to run.  The dot
+// products of the recurrence leave only their partials (DOT_PART): every block
+// of the kernel that needs them (p.q: the x/r update; r.r and r.z: the p
+// update) folds them itself, in the same order, which costs it less than the
+// fence, counter and re-read of a last block cost the kernel before.
 #pragma once
 
 #include "common.cuh"
@@ -24,8 +24,7 @@ enum DotMode {
   DOT_STORE = 0,  // *out = s
   DOT_BNORM,      // |b|^2; zero right-hand side finishes at once
   DOT_RZ0,        // initial r.z
-  DOT_PART,       // block partials only (p.q, r.z)
-  DOT_RR,         // r.r, iteration count and convergence test
+  DOT_PART,       // block partials only (p.q, r.r, r.z)
   DOT_TR          // |b - A x|^2
 };
 
@@ -47,7 +46,7 @@ static __device__ void dot_finalize(const DotCtx &c, double s) {
       break;
     case DOT_BNORM:
       sc->bnorm2 = s;
-      sc->iters = 0;
+      sc->thr2 = c.rtol * c.rtol * s;
       sc->rr = s;
       if (s == 0.0) {
         sc->done = 1;
@@ -62,20 +61,6 @@ static __device__ void dot_finalize(const DotCtx &c, double s) {
       if (!(s > 0.0)) {
         sc->done = 1;
         sc->status = MGPBD_E_BREAKDOWN;
-      }
-      break;
-    case DOT_RR:
-      sc->rr = s;
-      sc->iters += 1;
-      if (!(s == s)) {
-        sc->done = 1;
-        sc->status = MGPBD_E_BREAKDOWN;
-      } else if (sqrt(s) <= c.rtol * sqrt(sc->bnorm2)) {
-        sc->done = 1;
-        sc->status = MGPBD_OK;
-      } else if (sc->iters >= c.maxiter) {
-        sc->done = 1;
-        sc->status = MGPBD_W_NOT_CONVERGED;
       }
       break;
     case DOT_TR:
@@ -112,15 +97,6 @@ static __device__ __forceinline__ double fold_partials(const double *partials, i
     for (int k = 0; k < 4; ++k) s += t[k];
   }
   return block_sum(s);
-}
-
-// fold_partials with the result in every thread
-static __device__ __forceinline__ double fold_partials_all(const double *partials, int vn) {
-  __shared__ double all;
-  const double s = fold_partials(partials, vn);
-  if (threadIdx.x == 0) all = s;
-  __syncthreads();
-  return all;
 }
 
 // block reduce of one value per thread in a fixed order, then the last block

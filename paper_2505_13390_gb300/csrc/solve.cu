@@ -72,7 +72,7 @@ __global__ void k_dot(int64_t n, const double *x, const double *y, DotCtx c, int
 }
 
 // alpha = r.z / p.q from p.q's partials (a breakdown p.q <= 0 ends the solve);
-// x += alpha p; r -= alpha q; then r.r (convergence test).  The start of the
+// x += alpha p; r -= alpha q; then r.r's partials.  The start of the
 // next V-cycle is folded in: bl = r in the V-cycle's precision (MGPBD_MIXED)
 // and, with the Jacobi smoother, its first sweep from zero x0 = omega D^-1 r.
 // In mixed precision each thread sums the squares of its FP32 copies of r in
@@ -122,22 +122,28 @@ __device__ __forceinline__ void xr_update_body(int vb, int vn, int64_t n, double
     qv = reinterpret_cast<const double2 *>(q)[k];
   };
   if (k0 < n2) load(k0);
-  const double rz = sc->rz[sc->iters & 1];
-  const double pq = fold_partials_all(part_pq, n_pq);
-  if (gate.closed()) return;
-  if (!(pq > 0.0)) {
-    if (vb == 0 && threadIdx.x == 0) {
+  const int it = sc->p_updates;
+  const double rz = sc->rz[it & 1];
+  __shared__ double sh_al;
+  __shared__ bool sh_ok;  // false on a breakdown
+  const double pq = fold_partials(part_pq, n_pq);
+  if (threadIdx.x == 0) {  // one division per block: FP64 is scarce
+    sh_ok = pq > 0.0;
+    sh_al = rz / pq;
+    if (vb == 0 && !gate.closed()) {
       sc->pq = pq;
-      sc->status = MGPBD_E_BREAKDOWN;
-      sc->done = 1;
+      if (pq > 0.0) {
+        sc->alpha = sh_al;
+        sc->iters = it + 1;
+      } else {
+        sc->status = MGPBD_E_BREAKDOWN;
+        sc->done = 1;
+      }
     }
-    return;
   }
-  const double al = rz / pq;
-  if (vb == 0 && threadIdx.x == 0) {
-    sc->pq = pq;
-    sc->alpha = al;
-  }
+  __syncthreads();
+  const double al = sh_al;
+  if (gate.closed() || !sh_ok) return;
   T acc = 0;
 #pragma unroll 1
   for (int64_t k = k0; k < n2; k += (int64_t)vn * blockDim.x) {
@@ -192,13 +198,16 @@ __global__ void k_top_prep(int64_t n, const double *r, T *bl, const T *dinv, T o
   }
 }
 
-// beta = r.z / (r.z of the iteration before) from r.z's partials (a breakdown
-// r.z <= 0 ends the solve); p = z + beta p, two entries per thread (16-byte
+// The convergence test on r.r and beta = r.z / (r.z of the iteration before),
+// both from block partials (r.r at the tolerance, the iteration cap and a
+// breakdown r.z <= 0 end the solve; the V-cycle of the last iteration has then
+// run for nothing); p = z + beta p, two entries per thread (16-byte
 // loads; p and z are 256-byte aligned); with pdf, p also as float-float pairs
 // for the pair form of A.p (params.ap_split)
 template <class Gate>
 __device__ __forceinline__ void p_update_body(int vb, int vn, int64_t n, double *p,
-                                              const double *z, PcgScalars *sc,
+                                              const double *z, PcgScalars *sc, int maxiter,
+                                              const double *part_rr, int n_rr,
                                               const double *part_rz, int n_rz, float2 *pdf,
                                               Gate gate) {
   const int64_t n2 = n / 2, h2 = (n2 + 1) / 2;  // pairs k and k + h2 per thread
@@ -217,21 +226,36 @@ __device__ __forceinline__ void p_update_body(int vb, int vn, int64_t n, double 
   gate.open();
   if (k0 < h2) load(k0);  // beside the fold of r.z
   const int it = sc->iters;
-  const double rz_old = sc->rz[(it - 1) & 1];
-  const double rz = fold_partials_all(part_rz, n_rz);
-  if (gate.closed()) return;
-  if (!(rz > 0.0)) {
-    if (vb == 0 && threadIdx.x == 0) {
-      sc->status = MGPBD_E_BREAKDOWN;
-      sc->done = 1;
+  const double rz_old = sc->rz[(it - 1) & 1], thr2 = sc->thr2;
+  __shared__ double sh_be;
+  __shared__ int sh_go;
+  const double rr = fold_partials(part_rr, n_rr);
+  __syncthreads();  // before the buffer of block_sum is used again
+  const double rz = fold_partials(part_rz, n_rz);
+  if (threadIdx.x == 0) {
+    int go = 0, st = MGPBD_OK;
+    if (!(rr == rr)) st = MGPBD_E_BREAKDOWN;
+    else if (rr <= thr2) st = MGPBD_OK;
+    else if (it >= maxiter) st = MGPBD_W_NOT_CONVERGED;
+    else if (!(rz > 0.0)) st = MGPBD_E_BREAKDOWN;
+    else go = 1;
+    sh_be = go ? rz / rz_old : 0.0;
+    sh_go = go;
+    if (vb == 0 && !gate.closed()) {
+      sc->rr = rr;
+      if (go) {
+        sc->rz[it & 1] = rz;
+        sc->beta = sh_be;
+        sc->p_updates = it;
+      } else {
+        sc->status = st;
+        sc->done = 1;
+      }
     }
-    return;
   }
-  const double be = rz / rz_old;
-  if (vb == 0 && threadIdx.x == 0) {
-    sc->rz[it & 1] = rz;
-    sc->beta = be;
-  }
+  __syncthreads();
+  const double be = sh_be;
+  if (gate.closed() || !sh_go) return;
   for (int64_t k = k0; k < h2; k += (int64_t)vn * blockDim.x) {
     const int64_t k2 = k + h2;
     const bool two = k2 < n2;
@@ -259,15 +283,18 @@ __device__ __forceinline__ void p_update_body(int vb, int vn, int64_t n, double 
   }
 }
 
-__global__ void k_p_update(int64_t n, double *p, const double *z, PcgScalars *sc,
-                           const double *part_rz, int n_rz, float2 *pdf) {
-  p_update_body(blockIdx.x, gridDim.x, n, p, z, sc, part_rz, n_rz, pdf, ChainGate(sc));
+__global__ void k_p_update(int64_t n, double *p, const double *z, PcgScalars *sc, int maxiter,
+                           const double *part_rr, int n_rr, const double *part_rz, int n_rz,
+                           float2 *pdf) {
+  p_update_body(blockIdx.x, gridDim.x, n, p, z, sc, maxiter, part_rr, n_rr, part_rz, n_rz, pdf,
+                ChainGate(sc));
 }
 
 __global__ void k_pcg_init(PcgScalars *sc, unsigned int *bar) {
   bar[0] = 0;  // the coarse tail's barrier word starts each solve at zero
   sc->done = 0;
-  sc->iters = 0;
+  sc->iters = sc->p_updates = 0;
+  sc->thr2 = 0.0;
   sc->status = MGPBD_W_NOT_CONVERGED;
   sc->rz[0] = sc->rz[1] = sc->pq = sc->rr = sc->alpha = sc->beta = sc->tr2 = 0.0;
 }
@@ -448,6 +475,85 @@ template <int G, class T>
 __global__ void k_resid(int n, const int64_t *ptr, const int32_t *col, const T *val, const T *b,
                         const T *x, T *r, const PcgScalars *sc) {
   resid_rows<G, T>(HW_WARPS, n, ptr, col, val, b, x, r, ChainGate(sc));
+}
+
+// The first post-smoothing sweep with the prolongation taken along: every x_j
+// it reads is x_j + P_j x_c[agg_j], the value k_prolong would have stored (one
+// launch less per level; on large levels the two gathers more per entry cost
+// more than the launch, see kFuseProlongRows)
+template <int G, class T>
+__global__ void k_jacobi_prolong(int n, const int64_t *ptr, const int32_t *col, const T *val,
+                                 const T *dinv, T omega, const T *b, const int32_t *agg,
+                                 const T *P, const T *xc, const T *x, T *xn,
+                                 const PcgScalars *sc) {
+  ChainGate gate(sc);
+  GROUP_ROWS(G, n) {
+    const RowPre<T> p = row_pre<G>(ptr, col, val, i, g, valid);
+    int a[4];
+    T pj[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      if (p.k + j * G < p.e) {
+        a[j] = agg[p.c[j]];
+        pj[j] = P[p.c[j]];
+      }
+    const bool head = valid && g == 0;
+    const T di = head ? dinv[i] : (T)0, pi = head ? P[i] : (T)0;
+    const int ai = head ? agg[i] : -1;
+    gate.open();
+    T xv[4], cv[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      if (p.k + j * G < p.e) {
+        xv[j] = x[p.c[j]];
+        cv[j] = a[j] >= 0 ? xc[a[j]] : (T)0;
+      }
+    const T bi = head ? b[i] : (T)0;
+    T xi = head ? x[i] : (T)0;
+    if (ai >= 0) xi = fma(pi, xc[ai], xi);  // rows left alone have no aggregate
+    T s = 0;
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      if (p.k + j * G < p.e) s = fma(p.v[j], a[j] >= 0 ? fma(pj[j], cv[j], xv[j]) : xv[j], s);
+    for (int64_t k = p.k + 4 * G; k < p.e; k += G) {
+      const int c = col[k], ac = agg[c];
+      const T xk = x[c];
+      s = fma(val[k], ac >= 0 ? fma(P[c], xc[ac], xk) : xk, s);
+    }
+    s = group_sum<G>(s);
+    if (gate.closed()) return;
+    if (head) xn[i] = fma(omega, (bi - s) * di, xi);
+  }
+}
+constexpr int kFuseProlongRows = 1 << 16;
+
+// The last post-smoothing sweep of level 0: z = the new iterate in FP64, with
+// r.z when `dot` is set
+template <int G, class T>
+__global__ void k_jacobi_final(int n, const int64_t *ptr, const int32_t *col, const T *val,
+                               const T *dinv, T omega, const T *b, const T *x, double *z,
+                               const double *r, bool dot, DotCtx c) {
+  ChainGate gate(c.sc);
+  double acc = 0.0;
+  GROUP_ROWS(G, n) {
+    const RowPre<T> p = row_pre<G>(ptr, col, val, i, g, valid);
+    const bool head = valid && g == 0;
+    const T di = head ? dinv[i] : (T)0;
+    gate.open();
+    const T bi = head ? b[i] : (T)0, xi = head ? x[i] : (T)0;
+    const double ri = head && dot ? r[i] : 0.0;
+    T s = row_fin<G, T>(p, col, val, x);
+    s = group_sum<G>(s);
+    if (gate.closed()) break;
+    if (head) {
+      const double zi = widen(fma(omega, (bi - s) * di, xi));
+      z[i] = zi;
+      acc = fma(ri, zi, acc);
+    }
+  }
+  gate.open();  // warps without a row
+  if (gate.closed()) return;
+  if (dot) block_dot_finish(acc, c);
 }
 
 // b_c[a*k+c] = sum_{i in a} P_ic r_i (warp per aggregate, k columns of P per
@@ -865,6 +971,11 @@ static int spmv_pq_blocks(int m) {
   return std::min(row_blocks(m, G, kDotThreads),
                   wave_blocks((const void *)k_spmv_pq<G, double, double>, kDotThreads));
 }
+template <int G, class T>
+static int jacobi_final_blocks(int n) {
+  return std::min(row_blocks(n, G, kDotThreads),
+                  wave_blocks((const void *)k_jacobi_final<G, T>, kDotThreads));
+}
 // p update: four entries per thread, at most sixteen blocks per SM (every block
 // folds r.z's partials)
 static int p_blocks(int m) {
@@ -1092,8 +1203,8 @@ __global__ void kb_prolong0(const CohortMember *mem, const CohortBlock *blk) {
 
 __global__ void kb_pupdate(const CohortMember *mem, const CohortBlock *blk) {
   COHORT_BLOCK;
-  p_update_body(vb, vn, M.m, M.p, M.z, M.sc, M.c_rz.partials, M.grid[CS_ROW_FINAL], nullptr,
-                NoGate{});
+  p_update_body(vb, vn, M.m, M.p, M.z, M.sc, M.c_rr.maxiter, M.c_rr.partials, M.grid[CS_XR],
+                M.c_rz.partials, M.grid[CS_ROW_FINAL], nullptr, NoGate{});
 }
 
 // The V-cycle below level 0 of every member in one cooperative launch, depth
@@ -1263,7 +1374,7 @@ mgpbd_status cohort_build(Cohort *c) {
     M.q = h->pq;
     M.sc = h->sc;
     M.c_pq = pq_ctx(h);
-    M.c_rr = make_ctx(h, DOT_RR);
+    M.c_rr = make_ctx(h, DOT_PART);
     M.c_rz = rz_ctx(h);
     M.b0 = (float *)L0.b;
     M.x0 = (float *)L0.x;
@@ -1434,22 +1545,37 @@ mgpbd_status cohort_chunk(Cohort *c, int iters) {
   return MGPBD_OK;
 }
 
-// V-cycle on level l in precision T: L.b -> L.x (zero start).  On level 0 of
-// a top V-cycle, `x0_ready` says the first Jacobi sweep is already in L.x,
-// and `top` lets the last matrix-free sweep write z in FP64 (and r.z)
-// instead of L.x; `*z_written` then reports that it did.
+// a kernel of the V-cycle with a thread per item; the row kernels loop beyond
+// 64 blocks per SM
+template <class... P, class... A>
+static mgpbd_status item_launch(Handle *h, const char *what, void (*k)(P...), int64_t items,
+                                A... args) {
+  const int th = spread(items);
+  return chain_launch(h, what, k, blocks_for(items, th), th, args...);
+}
+template <class... P, class... A>
+static mgpbd_status rows_launch(Handle *h, const char *what, void (*k)(P...), int64_t rows, int G,
+                                A... args) {
+  const int th = spread(rows * G);
+  return chain_launch(h, what, k, row_blocks(rows, G, th), th, args...);
+}
+
+// V-cycle on level l in precision T from its right-hand side (zero start);
+// *res is the vector of the level that holds the result.  On level 0 of a top
+// V-cycle, `x0_ready` says the first Jacobi sweep is already in L.x, and `top`
+// lets the last Jacobi sweep write z in FP64 (and r.z) instead; `*z_written`
+// then reports that it did.
 template <class T>
-static mgpbd_status vcycle_level(Handle *h, int l, const T *b_in, bool x0_ready = false,
+static mgpbd_status vcycle_level(Handle *h, int l, const T *b_in, T **res, bool x0_ready = false,
                                  const TopOut *top = nullptr, bool *z_written = nullptr) {
   Level &L = h->lev[l];
   const PcgScalars *sc = h->sc;
   const int n = L.n;
   T *x = (T *)L.x;
-  if (l == h->L - 1) {
-    MG_TRY(chain_launch(h, "k_coarse_apply", k_coarse_apply<T>,
-                        blocks_for((int64_t)n * 32, spread(32ll * n)), spread(32ll * n), n, h->cinv, b_in, x, sc));
-    return MGPBD_OK;
-  }
+  *res = x;
+  if (l == h->L - 1)
+    return item_launch(h, "k_coarse_apply", k_coarse_apply<T>, 32ll * n, n, h->cinv, b_in, x,
+                       sc);
   const int G = group_for(h, L, sizeof(T) == 8);
   const T om = (T)L.omega;
   const T *val = vals<T>(L);
@@ -1466,9 +1592,8 @@ static mgpbd_status vcycle_level(Handle *h, int l, const T *b_in, bool x0_ready 
         int c = reverse ? nc - 1 - k : k;
         int64_t off = L.hcptr[c], cnt = L.hcptr[c + 1] - off;
         if (cnt == 0) continue;
-        DISPATCH_G(G, MG_TRY(chain_launch(h, "k_gs_colour", k_gs_colour<GG, T>, row_blocks(cnt, GG),
-                                          256, (int)cnt, L.crow + off, L.ptr, L.col, val, dinv,
-                                          b_in, x, sc)));
+        DISPATCH_G(G, MG_TRY(rows_launch(h, "k_gs_colour", k_gs_colour<GG, T>, cnt, GG, (int)cnt,
+                                         L.crow + off, L.ptr, L.col, val, dinv, b_in, x, sc)));
       }
     return MGPBD_OK;
   };
@@ -1478,9 +1603,8 @@ static mgpbd_status vcycle_level(Handle *h, int l, const T *b_in, bool x0_ready 
   const bool cheb = h->p.smoother == MGPBD_SMOOTH_CHEBYSHEV;
   auto apply = [&](const T *v, T *y) -> mgpbd_status {
     if (mf) return mf_level0<T>(h, kMfApply, v, b_in, dinv, om, y);
-    DISPATCH_G(G, MG_TRY(chain_launch(h, "k_spmv_plain", k_spmv_plain<GG, T>,
-                                      row_blocks(n, GG, spread(n * (int64_t)GG)),
-                                      spread(n * (int64_t)GG), n, L.ptr, L.col, val, v, y, sc)));
+    DISPATCH_G(G, MG_TRY(rows_launch(h, "k_spmv_plain", k_spmv_plain<GG, T>, n, GG, n, L.ptr, L.col,
+                                     val, v, y, sc)));
     return MGPBD_OK;
   };
   // (from_zero: x = 0 on entry, so A x = 0 needs no product)
@@ -1490,106 +1614,105 @@ static mgpbd_status vcycle_level(Handle *h, int l, const T *b_in, bool x0_ready 
     double rho = 1.0 / sigma;
     T *t = (T *)L.t, *d = x2;
     if (!from_zero) MG_TRY(apply(x, t));
-    MG_TRY(chain_launch(h, "k_cheb_start", k_cheb_start<T>, blocks_for(n, spread(n)), spread(n), n, b_in,
-                        from_zero ? nullptr : t, dinv, (T)(1.0 / theta), r, d, x, sc));
+    MG_TRY(item_launch(h, "k_cheb_start", k_cheb_start<T>, n, n, b_in, from_zero ? nullptr : t,
+                       dinv, (T)(1.0 / theta), r, d, x, sc));
     for (int k = 1; k < h->p.smooth_sweeps; ++k) {
       MG_TRY(apply(d, t));
       double rho2 = 1.0 / (2.0 * sigma - rho);
-      MG_TRY(chain_launch(h, "k_cheb_step", k_cheb_step<T>, blocks_for(n, spread(n)), spread(n), n, t, dinv,
-                          (T)(rho2 * rho), (T)(2.0 * rho2 / delta), r, d, x, sc));
+      MG_TRY(item_launch(h, "k_cheb_step", k_cheb_step<T>, n, n, t, dinv, (T)(rho2 * rho),
+                         (T)(2.0 * rho2 / delta), r, d, x, sc));
       rho = rho2;
     }
     return MGPBD_OK;
   };
+  // one Jacobi sweep x -> x2, then the two swap
+  auto sweep = [&]() -> mgpbd_status {
+    if (l == 0) MG_TRY(prof_begin(h));
+    if (mf) {
+      MG_TRY(mf_level0<T>(h, kMfSweep, x, b_in, dinv, om, x2));
+    } else {
+      DISPATCH_G(G, MG_TRY(rows_launch(h, "k_jacobi", k_jacobi<GG, T>, n, GG, n, L.ptr, L.col, val,
+                                       dinv, om, b_in, x, x2, sc)));
+    }
+    if (l == 0) MG_TRY(prof_end(h));
+    std::swap(x, x2);
+    return MGPBD_OK;
+  };
+  const bool jac = !gs && !cheb;
+  const int sweeps = jac ? h->p.smooth_sweeps : 0;
   if (cheb) {
     MG_TRY(cheb_smooth(true));
   } else if (gs) {
     MG_CUDA(cudaMemsetAsync(x, 0, sizeof(T) * n, h->stream));
     MG_TRY(gs_sweeps(false));
   } else if (!x0_ready) {
-    MG_TRY(chain_launch(h, "k_jacobi0", k_jacobi0<T>, blocks_for(n, spread(n)), spread(n), n, b_in,
-                        dinv, om, x, sc));
+    MG_TRY(item_launch(h, "k_jacobi0", k_jacobi0<T>, n, n, b_in, dinv, om, x, sc));
   }
-  for (int s = 1; s < h->p.smooth_sweeps && !gs && !cheb; ++s) {
-    if (l == 0) MG_TRY(prof_begin(h));
-    if (mf) {
-      MG_TRY(mf_level0<T>(h, kMfSweep, x, b_in, dinv, om, x2));
-    } else {
-      DISPATCH_G(G, MG_TRY(chain_launch(h, "k_jacobi", k_jacobi<GG, T>,
-                                        row_blocks(n, GG, spread(n * (int64_t)GG)),
-                                        spread(n * (int64_t)GG), n,
-                                        L.ptr, L.col, val, dinv, om, b_in, x, x2, sc)));
-    }
-    if (l == 0) MG_TRY(prof_end(h));
-    std::swap(x, x2);
-  }
+  for (int s = 1; s < sweeps; ++s) MG_TRY(sweep());
   Level &Lc = h->lev[l + 1];
   // the coarse level's first Jacobi sweep from zero rides on the restriction
-  const bool c_jac = !gs && !cheb && l + 2 < h->L;
+  const bool c_jac = jac && l + 2 < h->L;
   const int nk = h->p.nk_vectors;
+  const T *dinv_c = c_jac ? dinvs<T>(Lc) : nullptr;
+  T *x_c = c_jac ? (T *)Lc.x : nullptr;
   if (mf && L.mpos && nk == 1) {
     // the residual written in member order, the restriction streaming it
     MG_TRY(mf_level0<T>(h, kMfResidMember, x, b_in, dinv, om, r));
-    MG_TRY(chain_launch(h, "k_restrict_member", k_restrict_member<T>,
-                        blocks_for(32ll * L.n_agg, spread(32ll * L.n_agg)),
-                        spread(32ll * L.n_agg), L.n_agg, L.mptr,
-                        (const T *)L.Pm, r, (T *)Lc.b, sc, c_jac ? dinvs<T>(Lc) : nullptr,
-                        (T)Lc.omega, c_jac ? (T *)Lc.x : nullptr));
-  } else if (mf) {
-    MG_TRY(mf_level0<T>(h, kMfResid, x, b_in, dinv, om, r));
-    MG_TRY(chain_launch(h, "k_restrict", k_restrict<T>,
-                        blocks_for(32ll * L.n_agg, spread(32ll * L.n_agg)),
-                        spread(32ll * L.n_agg), L.n_agg, nk, L.mptr, L.mrow, Ps<T>(L), r, (T *)Lc.b, sc,
-                        c_jac ? dinvs<T>(Lc) : nullptr, (T)Lc.omega, c_jac ? (T *)Lc.x : nullptr));
+    MG_TRY(item_launch(h, "k_restrict_member", k_restrict_member<T>, 32ll * L.n_agg, L.n_agg,
+                       L.mptr, (const T *)L.Pm, r, (T *)Lc.b, sc, dinv_c, (T)Lc.omega, x_c));
   } else {
-    DISPATCH_G(G, MG_TRY(chain_launch(h, "k_resid", k_resid<GG, T>,
-                                      row_blocks(n, GG, spread(n * (int64_t)GG)),
-                                      spread(n * (int64_t)GG), n,
-                                      L.ptr, L.col, val, b_in, x, r, sc)));
-    MG_TRY(chain_launch(h, "k_restrict", k_restrict<T>,
-                        blocks_for(32ll * L.n_agg, spread(32ll * L.n_agg)),
-                        spread(32ll * L.n_agg), L.n_agg, nk, L.mptr, L.mrow, Ps<T>(L), r, (T *)Lc.b, sc,
-                        c_jac ? dinvs<T>(Lc) : nullptr, (T)Lc.omega, c_jac ? (T *)Lc.x : nullptr));
+    if (mf)
+      MG_TRY(mf_level0<T>(h, kMfResid, x, b_in, dinv, om, r));
+    else
+      DISPATCH_G(G, MG_TRY(rows_launch(h, "k_resid", k_resid<GG, T>, n, GG, n, L.ptr, L.col, val,
+                                       b_in, x, r, sc)));
+    MG_TRY(item_launch(h, "k_restrict", k_restrict<T>, 32ll * L.n_agg, L.n_agg, nk, L.mptr, L.mrow,
+                       Ps<T>(L), r, (T *)Lc.b, sc, dinv_c, (T)Lc.omega, x_c));
   }
-  const T *xc = (const T *)Lc.x;  // where the coarser level leaves its result
+  T *xc = nullptr;  // where the coarser level leaves its result
   if (tail_applies(h, l + 1)) {
     MG_TRY(launch_tail<T>(h, l + 1));
     xc = tail_result<T>(h, l + 1);
   } else {
-    MG_TRY(vcycle_level<T>(h, l + 1, (const T *)Lc.b, c_jac));
+    MG_TRY(vcycle_level<T>(h, l + 1, (const T *)Lc.b, &xc, c_jac));
   }
-  if (nk == 1)
-    MG_TRY(chain_launch(h, "k_prolong", k_prolong<T>,
-                        blocks_for((n + kProlongRows - 1) / kProlongRows, spread(n / kProlongRows)),
-                        spread(n / kProlongRows), n, L.agg, Ps<T>(L), xc, x, sc));
-  else
-    MG_TRY(chain_launch(h, "k_prolong", k_prolong_k<T>, blocks_for(n, 256), 256, n, nk, L.agg,
-                        Ps<T>(L), (const T *)Lc.x, x, sc));
+  int s = 0;  // post-smoothing sweeps done
+  if (jac && nk == 1 && !mf && n <= kFuseProlongRows && (sweeps > 1 || !top)) {
+    // the first sweep takes the prolongation with it
+    if (l == 0) MG_TRY(prof_begin(h));
+    DISPATCH_G(G, MG_TRY(rows_launch(h, "k_jacobi_prolong", k_jacobi_prolong<GG, T>, n, GG, n,
+                                     L.ptr, L.col, val, dinv, om, b_in, L.agg, Ps<T>(L), xc, x, x2, sc)));
+    if (l == 0) MG_TRY(prof_end(h));
+    std::swap(x, x2);
+    s = 1;
+  } else if (nk == 1) {
+    MG_TRY(item_launch(h, "k_prolong", k_prolong<T>, (n + kProlongRows - 1) / kProlongRows, n,
+                       L.agg, Ps<T>(L), xc, x, sc));
+  } else {
+    MG_TRY(item_launch(h, "k_prolong", k_prolong_k<T>, n, n, nk, L.agg, Ps<T>(L), xc, x, sc));
+  }
   if (gs) MG_TRY(gs_sweeps(true));
   if (cheb) MG_TRY(cheb_smooth(false));
   bool zw = false;
-  for (int s = 0; s < h->p.smooth_sweeps && !gs && !cheb; ++s) {
-    if (mf && top && s + 1 == h->p.smooth_sweeps) {
+  for (; s < sweeps; ++s) {
+    if (!top || s + 1 < sweeps) {
+      MG_TRY(sweep());
+      continue;
+    }
+    zw = true;
+    if (mf) {
       MG_TRY(mf_level0_final<T>(h, x, b_in, dinv, om, *top));
-      zw = true;
       break;
     }
-    if (l == 0) MG_TRY(prof_begin(h));
-    if (mf) {
-      MG_TRY(mf_level0<T>(h, kMfSweep, x, b_in, dinv, om, x2));
-    } else {
-      DISPATCH_G(G, MG_TRY(chain_launch(h, "k_jacobi", k_jacobi<GG, T>,
-                                        row_blocks(n, GG, spread(n * (int64_t)GG)),
-                                        spread(n * (int64_t)GG), n,
-                                        L.ptr, L.col, val, dinv, om, b_in, x, x2, sc)));
-    }
-    if (l == 0) MG_TRY(prof_end(h));
-    std::swap(x, x2);
+    MG_TRY(prof_begin(h));
+    DISPATCH_G(G, const int blocks = jacobi_final_blocks<GG, T>(n); if (top->dot) h->n_rz = blocks;
+               MG_TRY(chain_launch(h, "k_jacobi_final", k_jacobi_final<GG, T>, blocks, kDotThreads,
+                                   n, L.ptr, L.col, val, dinv, om, b_in, x, top->z, top->r,
+                                   top->dot, top->c)));
+    MG_TRY(prof_end(h));
   }
   if (z_written) *z_written = zw;
-  if (x != (T *)L.x && !zw) {  // keep the result in L.x
-    MG_CUDA(cudaMemcpyAsync(L.x, x, sizeof(T) * n, cudaMemcpyDeviceToDevice, h->stream));
-  }
+  *res = x;
   return MGPBD_OK;
 }
 
@@ -1627,20 +1750,20 @@ static mgpbd_status vcycle_top(Handle *h, const double *r, double *z, bool prepa
                           (float *)L.b, L.dinv32, (float)L.omega, jac ? (float *)L.x : nullptr,
                           h->sc));
     }
-    MG_TRY(vcycle_level<float>(h, 0, (const float *)L.b, jac, &o, &zw));
+    float *x = nullptr;
+    MG_TRY(vcycle_level<float>(h, 0, (const float *)L.b, &x, jac, &o, &zw));
     if (!zw) {
-      MG_TRY(chain_launch(h, "k_convert", k_convert<float, double>, blocks_for(m, spread(m)), spread(m), m,
-                          (const float *)L.x, z, h->sc));
+      MG_TRY(item_launch(h, "k_convert", k_convert<float, double>, m, m, x, z, h->sc));
     }
   } else {
     if (!prepared && jac) {
       MG_TRY(chain_launch(h, "k_top_prep", k_top_prep<double>, blocks_for(m, 256), 256, m, r,
                           nullptr, L.dinv, L.omega, (double *)L.x, h->sc));
     }
-    MG_TRY(vcycle_level<double>(h, 0, r, jac, &o, &zw));
+    double *x = nullptr;
+    MG_TRY(vcycle_level<double>(h, 0, r, &x, jac, &o, &zw));
     if (!zw) {
-      MG_TRY(chain_launch(h, "k_convert", k_convert<double, double>, blocks_for(m, spread(m)), spread(m), m,
-                          (const double *)L.x, z, h->sc));
+      MG_TRY(item_launch(h, "k_convert", k_convert<double, double>, m, m, x, z, h->sc));
     }
   }
   if (o.dot && !zw) MG_TRY(launch_dot(h, r, z, m, dot_mode, 1));
@@ -1664,7 +1787,8 @@ mgpbd_status apply_level0(Handle *h, int form, const double *x, double *y) {
   if (form == 0) {
     const int G = group_for(h, L, true);
     DISPATCH_G(G, MG_TRY(chain_launch(h, "k_spmv_pq", k_spmv_pq<GG, double, double>,
-                                      spmv_pq_blocks<GG>(m), kDotThreads, m, L.ptr, L.col, L.val, x, y, c)));
+                                      spmv_pq_blocks<GG>(m), kDotThreads, m, L.ptr, L.col, L.val,
+                                      x, y, c)));
     return MGPBD_OK;
   }
   if (form == 2) MG_TRY(mf_split(h, x, h->p_df, m));
@@ -1701,18 +1825,20 @@ static mgpbd_status pcg_iteration(Handle *h, double *x) {
   const bool jac = top_jacobi(h);
   if (h->p.precision == MGPBD_MIXED)
     MG_TRY(chain_launch(h, "k_xr_update", k_xr_update<float>,
-                        xr_blocks<float>(m),
-                        kDotThreads, m, x, r, p, q, make_ctx(h, DOT_RR), h->part_pq, h->n_pq,
+                        h->n_rr = xr_blocks<float>(m),
+                        kDotThreads, m, x, r, p, q, make_ctx(h, DOT_PART), h->part_pq, h->n_pq,
                         (float *)L.b, L.dinv32,
                         (float)L.omega, jac ? (float *)L.x : nullptr));
   else
     MG_TRY(chain_launch(h, "k_xr_update", k_xr_update<double>,
-                        xr_blocks<double>(m),
-                        kDotThreads, m, x, r, p, q, make_ctx(h, DOT_RR), h->part_pq, h->n_pq,
+                        h->n_rr = xr_blocks<double>(m),
+                        kDotThreads, m, x, r, p, q, make_ctx(h, DOT_PART), h->part_pq, h->n_pq,
                         nullptr, L.dinv, L.omega,
                         jac ? (double *)L.x : nullptr));
   MG_TRY(vcycle_top(h, r, z, true, DOT_PART));
-  MG_TRY(chain_launch(h, "k_p_update", k_p_update, p_blocks(m), kDotThreads, m, p, z, h->sc, h->part_rz, h->n_rz, h->p.ap_split ? h->p_df : nullptr));
+  MG_TRY(chain_launch(h, "k_p_update", k_p_update, p_blocks(m), kDotThreads, m, p, z, h->sc,
+                      h->p.pcg_maxiter, h->partials, h->n_rr, h->part_rz, h->n_rz,
+                      h->p.ap_split ? h->p_df : nullptr));
   return MGPBD_OK;
 }
 
