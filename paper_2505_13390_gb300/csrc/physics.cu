@@ -283,65 +283,93 @@ __device__ __forceinline__ double gdot(const double *a, const double *b) {
   return fma(a[2], b[2], fma(a[1], b[1], a[0] * b[0]));
 }
 
-// Values of A (eq. 3, Sec. 4.2 formulas); one warp per row, lanes over the
-// row's off-diagonals; lane 0 also forms the diagonal.  Also writes 1/A_ii
-// and, in mixed precision, the FP32 mirrors.
-__global__ void k_assemble(int m, int E, const int32_t *edge, const int32_t *tet, const double *w,
-                           const double *gd, const double *gt, const double *alpha_t,
-                           const int64_t *ptr, const int32_t *col, const uint16_t *map,
-                           double *val, double *dinv, float *val32, float *dinv32) {
-  const int lane = threadIdx.x & 31;
-  int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-  int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t ii = warp; ii < m; ii += nwarps) {
-    int i = (int)ii;
-    int32_t v[4];
-    int c;
-    if (i < E) {
-      v[0] = edge[2 * (int64_t)i];
-      v[1] = edge[2 * (int64_t)i + 1];
-      v[2] = v[3] = 0;
-      c = 2;
+__device__ __forceinline__ int row_setup(int i, int E, const int32_t *edge, const int32_t *tet,
+                                         const double *w, const double *gd, const double *gt,
+                                         double gi[4][3], double wi[4]) {
+  int32_t v[4];
+  int c;
+  if (i < E) {
+    v[0] = edge[2 * (int64_t)i];
+    v[1] = edge[2 * (int64_t)i + 1];
+    v[2] = v[3] = 0;
+    c = 2;
+  } else {
+    const int32_t *t = tet + 4 * (int64_t)(i - E);
+    v[0] = t[0]; v[1] = t[1]; v[2] = t[2]; v[3] = t[3];
+    c = 4;
+  }
+  for (int s = 0; s < 4; ++s) {
+    if (s < c) {
+      row_grad(i, s, E, gd, gt, gi[s]);
+      wi[s] = w[v[s]];
     } else {
-      const int32_t *t = tet + 4 * (int64_t)(i - E);
-      v[0] = t[0]; v[1] = t[1]; v[2] = t[2]; v[3] = t[3];
-      c = 4;
+      gi[s][0] = gi[s][1] = gi[s][2] = 0.0;
+      wi[s] = 0.0;
     }
+  }
+  return c;
+}
+
+// Off-diagonal values of A (eq. 3, Sec. 4.2 formulas), G lanes per row over its
+// entries, and in mixed precision their FP32 mirrors.  Bound by FP64 issue (a
+// warp's FP64 instruction holds its SM for 20 clocks whatever number of lanes
+// is active), so the lanes per row follow the row length, and the diagonal,
+// one value per row with a division, has a kernel of its own with one row per
+// lane: as lane 0's extra work here it took more issue slots than the
+// off-diagonals (2.2 ms for both on the 40x33x40 block's 60M entries).
+template <int G>
+__global__ void __launch_bounds__(256)
+    k_assemble(int m, int E, const int32_t *edge, const int32_t *tet, const double *w,
+               const double *gd, const double *gt, const int64_t *ptr, const int32_t *col,
+               const uint16_t *map, double *val, float *val32) {
+  const int g = threadIdx.x & (G - 1);
+  const int64_t ii = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / G;
+  if (ii >= m) return;
+  const int i = (int)ii;
+  const int64_t e = ptr[i + 1] - 1;
+  double gi[4][3], wi[4];
+  row_setup(i, E, edge, tet, w, gd, gt, gi, wi);
+  for (int64_t k = ptr[i] + g; k < e; k += G) {
+    int j = col[k];
+    unsigned code = map[k];
+    int ns = code & 3;
+    double acc = 0.0;
+    for (int p = 0; p < ns; ++p) {
+      const int si = (code >> (2 + 4 * p)) & 3, sj = (code >> (4 + 4 * p)) & 3;
+      double gj[3];
+      row_grad(j, sj, E, gd, gt, gj);
+      // (selected, not indexed: the row's gradients stay in registers)
+      double gs[3], ws;
+#pragma unroll
+      for (int d = 0; d < 3; ++d)
+        gs[d] = si == 0 ? gi[0][d] : (si == 1 ? gi[1][d] : (si == 2 ? gi[2][d] : gi[3][d]));
+      ws = si == 0 ? wi[0] : (si == 1 ? wi[1] : (si == 2 ? wi[2] : wi[3]));
+      acc = fma(ws, gdot(gs, gj), acc);
+    }
+    val[k] = acc;
+    if (val32) val32[k] = f64_to_f32(acc);
+  }
+}
+
+// diagonal of A and its reciprocal, one row per thread
+__global__ void k_assemble_diag(int m, int E, const int32_t *edge, const int32_t *tet,
+                                const double *w, const double *gd, const double *gt,
+                                const double *alpha_t, const int64_t *ptr, double *val,
+                                double *dinv, float *val32, float *dinv32) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < m; i += gridDim.x * blockDim.x) {
     double gi[4][3], wi[4];
-    for (int s = 0; s < 4; ++s) {
-      if (s < c) {
-        row_grad(i, s, E, gd, gt, gi[s]);
-        wi[s] = w[v[s]];
-      } else {
-        gi[s][0] = gi[s][1] = gi[s][2] = 0.0;
-        wi[s] = 0.0;
-      }
-    }
-    int64_t s0 = ptr[i], e = ptr[i + 1] - 1;
-    for (int64_t k = s0 + lane; k < e; k += 32) {
-      int j = col[k];
-      unsigned code = map[k];
-      int ns = code & 3;
-      double acc = 0.0;
-      for (int p = 0; p < ns; ++p) {
-        int si = (code >> (2 + 4 * p)) & 3, sj = (code >> (4 + 4 * p)) & 3;
-        double gj[3];
-        row_grad(j, sj, E, gd, gt, gj);
-        acc = fma(wi[si], gdot(gi[si], gj), acc);
-      }
-      val[k] = acc;
-      if (val32) val32[k] = f64_to_f32(acc);
-    }
-    if (lane == 0) {
-      double acc = 0.0;
-      for (int s = 0; s < c; ++s) acc = fma(wi[s], gdot(gi[s], gi[s]), acc);
-      double d = acc + alpha_t[i];
-      val[e] = d;
-      dinv[i] = 1.0 / d;
-      if (val32) {
-        val32[e] = f64_to_f32(d);
-        dinv32[i] = f64_to_f32(1.0 / d);
-      }
+    const int c = row_setup(i, E, edge, tet, w, gd, gt, gi, wi);
+    double acc = 0.0;
+#pragma unroll
+    for (int s = 0; s < 4; ++s)
+      if (s < c) acc = fma(wi[s], gdot(gi[s], gi[s]), acc);
+    const double d = acc + alpha_t[i], r = 1.0 / d;
+    const int64_t e = ptr[i + 1] - 1;
+    val[e] = d;
+    dinv[i] = r;
+    if (val32) {
+      val32[e] = f64_to_f32(d);
+      dinv32[i] = f64_to_f32(r);
     }
   }
 }
@@ -349,13 +377,20 @@ __global__ void k_assemble(int m, int E, const int32_t *edge, const int32_t *tet
 mgpbd_status launch_assemble(Handle *h) {
   if (h->m == 0) return MGPBD_OK;
   Level &L = h->lev[0];
-  const int th = 256;
-  int64_t warps = h->m;
-  int blocks = blocks_for(warps * 32, th);
-  k_assemble<<<blocks, th, 0, h->stream>>>(h->m, h->E, h->edge, h->tet, h->w, h->gd, h->gt,
-                                            h->alpha_t, L.ptr, L.col, h->map, L.val, L.dinv,
-                                            L.val32, L.dinv32);
-  MG_LAUNCH("k_assemble");
+  const double avg = (double)L.nnz / h->m;
+  auto off = [&](auto *kernel, int G) -> mgpbd_status {
+    const int64_t blocks = ((int64_t)h->m * G + 255) / 256;
+    kernel<<<(unsigned)blocks, 256, 0, h->stream>>>(h->m, h->E, h->edge, h->tet, h->w, h->gd,
+                                                    h->gt, L.ptr, L.col, h->map, L.val, L.val32);
+    MG_LAUNCH("k_assemble");
+    return MGPBD_OK;
+  };
+  MG_TRY(avg <= 12 ? off(k_assemble<8>, 8) : (avg <= 48 ? off(k_assemble<16>, 16)
+                                                        : off(k_assemble<32>, 32)));
+  k_assemble_diag<<<blocks_for(h->m, 128), 128, 0, h->stream>>>(
+      h->m, h->E, h->edge, h->tet, h->w, h->gd, h->gt, h->alpha_t, L.ptr, L.val, L.dinv, L.val32,
+      L.dinv32);
+  MG_LAUNCH("k_assemble_diag");
   return MGPBD_OK;
 }
 

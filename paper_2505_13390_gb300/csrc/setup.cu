@@ -81,36 +81,43 @@ __global__ void k_nk_init(int n, uint64_t seed, const unsigned long long *amax_b
     x[i] = u01(h64(hkey(seed, 0, i))) * amax;
 }
 
-// row sum in storage order: s = fma(A_ij, x_j, s), folded sequentially
-__device__ __forceinline__ double row_dot_canonical(const int64_t s0, const int64_t e,
-                                                    const int32_t *col, const double *val,
-                                                    const double *x, int lane) {
+// Weighted-Jacobi sweep with row sums in storage order, s = fma(A_ij, x_j, s).
+// The sum of a row is one chain of fused multiply-adds, so a warp runs the
+// chains of 32 rows side by side, one per lane: it loads 32 entries of each row
+// at a time (coalesced, the row's lanes together) into shared memory and every
+// lane folds its own row from there.  (One row per warp, folded by one lane,
+// spent a warp's FP64 instruction, 20 clocks of an SM on this part, on each
+// entry: 286 us per sweep of a 46,760-row beam.)
+constexpr int kNkWarps = 4, kNkPitch = 33;
+__global__ void __launch_bounds__(32 * kNkWarps)
+    k_nk_sweep(int n, const int64_t *ptr, const int32_t *col, const double *val, double omega,
+               const double *x, double *xn) {
+  extern __shared__ double2 nk_smem[];
+  double2 *buf = nk_smem + (threadIdx.x >> 5) * (32 * kNkPitch);
+  const int lane = threadIdx.x & 31;
+  const int64_t base = ((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5) * 32;
+  if (base >= n) return;
+  const int rows = (int)min((int64_t)32, n - base);
+  const int64_t s0 = lane < rows ? ptr[base + lane] : 0, e = lane < rows ? ptr[base + lane + 1] : 0;
+  int longest = (int)(e - s0);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) longest = max(longest, __shfl_xor_sync(0xffffffffu, longest, o));
   double s = 0.0;
-  for (int64_t base = s0; base < e; base += 32) {
-    int64_t k = base + lane;
-    double a = 0.0, xv = 0.0;
-    if (k < e) {
-      a = val[k];
-      xv = x[col[k]];
+  for (int c = 0; c < longest; c += 32) {
+#pragma unroll 4
+    for (int r = 0; r < 32; ++r) {
+      const int64_t k = __shfl_sync(0xffffffffu, s0, r) + c + lane;
+      if (k < __shfl_sync(0xffffffffu, e, r)) buf[r * kNkPitch + lane] = make_double2(val[k], x[col[k]]);
     }
-    int cnt = (int)min((int64_t)32, e - base);
+    __syncwarp();
+    const int cnt = (int)min((int64_t)32, e - s0 - c);
     for (int t = 0; t < cnt; ++t) {
-      double at = __shfl_sync(0xffffffffu, a, t);
-      double xt = __shfl_sync(0xffffffffu, xv, t);
-      if (lane == 0) s = fma(at, xt, s);
+      const double2 v = buf[lane * kNkPitch + t];
+      s = fma(v.x, v.y, s);
     }
+    __syncwarp();
   }
-  return __shfl_sync(0xffffffffu, s, 0);
-}
-
-__global__ void k_nk_sweep(int n, const int64_t *ptr, const int32_t *col, const double *val,
-                           double omega, const double *x, double *xn) {
-  WARP_LOOP(n) {
-    int i = (int)row_;
-    int64_t s0 = ptr[i], e = ptr[i + 1];
-    double s = row_dot_canonical(s0, e, col, val, x, lane);
-    if (lane == 0) xn[i] = fma(-omega, s / val[e - 1], x[i]);
-  }
+  if (lane < rows) xn[base + lane] = fma(-omega, s / val[e - 1], x[base + lane]);
 }
 
 // ---------------------------------------------------------------------------
@@ -435,67 +442,172 @@ __global__ void k_gal_pattern(int na, const int64_t *mptr, const int32_t *mrow,
 }
 
 // ---------------------------------------------------------------------------
-// Galerkin values, canonical order (warp per coarse row, shared accumulators)
+// Galerkin values, canonical order
 // ---------------------------------------------------------------------------
-__global__ void k_gal_values(int na, const int64_t *mptr, const int32_t *mrow,
-                             const int64_t *ptr, const int32_t *col, const double *val,
-                             const int32_t *agg, const double *P, const int64_t *cptr,
-                             const int32_t *ccol, double *cval, int maxlen) {
+// Every coarse entry (a, b), b >= a, is one chain of fused multiply-adds over
+// the member rows of a and their storage order; the chains of different
+// entries are independent.  A block takes up to 16 coarse rows.  Seven warps
+// produce: per round each coarse row advances by up to 32 entries of a member
+// row, loaded coalesced a round ahead, whose terms (P_i A_ij, P_j) for b = a and
+// for b > a go to the two ends of a small queue in shared memory, in order.  One
+// warp consumes the queues of the round before: lane r runs the diagonal chain
+// of coarse row r, lane 16 + r its off-diagonal ones, so that one FP64
+// instruction (20 clocks of an SM on this part) advances up to 32 chains.  (One
+// warp per coarse row with a single lane adding advanced one: 5.7 ms on the
+// 40x33x40 block, 1.4 ms on the 26x10x10 beam.)
+constexpr int kGalRows = 16, kGalWarps = 8;
+constexpr int kGalPer = (kGalRows + kGalWarps - 2) / (kGalWarps - 1);  // rows per producer warp
+
+__global__ void __launch_bounds__(32 * kGalWarps)
+    k_gal_values(int na, int rows, const int64_t *mptr, const int32_t *mrow, const int64_t *ptr,
+                 const int32_t *col, const double *val, const int32_t *agg, const double *P,
+                 const int64_t *cptr, const int32_t *ccol, double *cval, int maxlen) {
   extern __shared__ unsigned char smem_raw[];
-  const int wib = threadIdx.x >> 5;
-  double *acc = reinterpret_cast<double *>(smem_raw) + (size_t)wib * maxlen;
-  int *cols = reinterpret_cast<int *>(reinterpret_cast<double *>(smem_raw) +
-                                      (size_t)(blockDim.x >> 5) * maxlen) +
-              (size_t)wib * maxlen;
-  WARP_LOOP(na) {
-    int a = (int)row_;
-    int64_t cb = cptr[a];
-    int len = (int)(cptr[a + 1] - cb);
-    for (int t = lane; t < len; t += 32) {
-      acc[t] = 0.0;
-      cols[t] = ccol[cb + t];
+  double *const acc = reinterpret_cast<double *>(smem_raw);
+  int *const cols = reinterpret_cast<int *>(acc + (size_t)rows * maxlen);
+  __shared__ double2 term[2][kGalRows][32];
+  __shared__ uint16_t slot[2][kGalRows][32];
+  __shared__ int n_diag[2][kGalRows], n_off[2][kGalRows];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const unsigned below = (1u << lane) - 1u;
+  const int a0 = blockIdx.x * rows, nr = min(rows, na - a0);
+  for (int r = 0; r < nr; ++r) {
+    const int64_t cb = cptr[a0 + r];
+    const int len = (int)(cptr[a0 + r + 1] - cb);
+    for (int t = threadIdx.x; t < len; t += blockDim.x) {
+      acc[r * maxlen + t] = 0.0;
+      cols[r * maxlen + t] = ccol[cb + t];
     }
-    __syncwarp();
-    for (int64_t q = mptr[a]; q < mptr[a + 1]; ++q) {
-      int i = mrow[q];
-      double pi = P[i];
-      int64_t s0 = ptr[i], e = ptr[i + 1];
-      for (int64_t base = s0; base < e; base += 32) {
-        int64_t k = base + lane;
-        int slot = -1;
-        double tt = 0.0, pj = 0.0;
-        if (k < e) {
-          int j = col[k];
-          int b = agg[j];
-          if (b >= a) {
-            tt = pi * val[k];
-            pj = P[j];
-            if (b == a) {
-              slot = len - 1;
-            } else {
-              int lo = 0, hi = len - 1;
-              while (lo < hi) {
-                int mid = (lo + hi) >> 1;
-                if (cols[mid] < b) lo = mid + 1;
-                else hi = mid;
-              }
-              slot = lo;
-            }
+  }
+  if (threadIdx.x < 2 * kGalRows) (&n_diag[0][0])[threadIdx.x] = (&n_off[0][0])[threadIdx.x] = 0;
+
+  // producers: per owned coarse row the member being read, its entry range and
+  // weight, the next member's, and the chunk in flight
+  int64_t q[kGalPer], qe[kGalPer], k[kGalPer], e[kGalPer], kn[kGalPer], en[kGalPer];
+  double pi[kGalPer], pn[kGalPer], v[kGalPer];
+  int c[kGalPer], len[kGalPer];
+  auto next_member = [&](int o) {  // the member after q, ahead of time
+    if (q[o] + 1 < qe[o]) {
+      const int i = mrow[q[o] + 1];
+      kn[o] = ptr[i];
+      en[o] = ptr[i + 1];
+      pn[o] = P[i];
+    }
+  };
+  auto load_chunk = [&](int o) {
+    if (q[o] < qe[o] && k[o] + lane < e[o]) {
+      c[o] = col[k[o] + lane];
+      v[o] = val[k[o] + lane];
+    }
+  };
+#pragma unroll
+  for (int o = 0; o < kGalPer; ++o) {
+    const int r = warp - 1 + o * (kGalWarps - 1);
+    q[o] = qe[o] = 0;
+    if (warp > 0 && r < nr) {
+      q[o] = mptr[a0 + r];
+      qe[o] = mptr[a0 + r + 1];
+      len[o] = (int)(cptr[a0 + r + 1] - cptr[a0 + r]);
+      if (q[o] < qe[o]) {
+        const int i = mrow[q[o]];
+        k[o] = ptr[i];
+        e[o] = ptr[i + 1];
+        pi[o] = P[i];
+        next_member(o);
+        load_chunk(o);
+      }
+    }
+  }
+  __syncthreads();
+
+  int cur = -1;       // consumer: the entry whose chain is in a register
+  double sum = 0.0;
+  for (int buf = 0;; buf ^= 1) {
+    int produced = 0;
+    if (warp == 0) {
+      const int r = lane & (kGalRows - 1);
+      const bool diag = lane < kGalRows;
+      if (r < nr) {
+        const int b = buf ^ 1, n = diag ? n_diag[b][r] : n_off[b][r];
+        double *const A = acc + r * maxlen;
+        for (int t = 0; t < n; ++t) {
+          const int at = diag ? t : 31 - t;
+          const double2 x = term[b][r][at];
+          const int s = diag ? 0 : slot[b][r][at];  // the diagonal stays in the register
+          if (s != cur) {
+            if (cur >= 0) A[cur] = sum;
+            sum = diag ? 0.0 : A[s];
+            cur = s;
           }
+          sum = fma(x.x, x.y, sum);
         }
-        int cnt = (int)min((int64_t)32, e - base);
-        for (int t = 0; t < cnt; ++t) {
-          int st = __shfl_sync(0xffffffffu, slot, t);
-          double tv = __shfl_sync(0xffffffffu, tt, t);
-          double pv = __shfl_sync(0xffffffffu, pj, t);
-          if (lane == 0 && st >= 0) acc[st] = fma(tv, pv, acc[st]);
+      }
+    } else {
+#pragma unroll
+      for (int o = 0; o < kGalPer; ++o) {
+        const int r = warp - 1 + o * (kGalWarps - 1);
+        if (r >= nr) break;
+        const int a = a0 + r;
+        if (q[o] >= qe[o]) {
+          if (lane == 0) n_diag[buf][r] = n_off[buf][r] = 0;
+          continue;
+        }
+        produced = 1;
+        const bool in = k[o] + lane < e[o];
+        int b = -1;
+        double pj = 0.0;
+        const double t = pi[o] * v[o];
+        if (in) {
+          b = agg[c[o]];
+          pj = P[c[o]];
+        }
+        // the next chunk's loads before this one is placed
+        k[o] += 32;
+        if (k[o] >= e[o]) {
+          ++q[o];
+          k[o] = kn[o];
+          e[o] = en[o];
+          pi[o] = pn[o];
+          next_member(o);
+        }
+        load_chunk(o);
+        const bool isd = in && b == a, iso = in && b > a;
+        const unsigned md = __ballot_sync(0xffffffffu, isd), mo = __ballot_sync(0xffffffffu, iso);
+        if (isd) term[buf][r][__popc(md & below)] = make_double2(t, pj);
+        if (iso) {
+          const int *C = cols + r * maxlen;
+          int lo = 0, hi = len[o] - 1;
+          while (lo < hi) {
+            const int mid = (lo + hi) >> 1;
+            if (C[mid] < b) lo = mid + 1;
+            else hi = mid;
+          }
+          const int at = 31 - __popc(mo & below);
+          term[buf][r][at] = make_double2(t, pj);
+          slot[buf][r][at] = (uint16_t)lo;
+        }
+        if (lane == 0) {
+          n_diag[buf][r] = __popc(md);
+          n_off[buf][r] = __popc(mo);
         }
       }
     }
-    __syncwarp();
-    for (int t = lane; t < len; t += 32)
-      if (cols[t] >= a) cval[cb + t] = acc[t];
-    __syncwarp();
+    if (!__syncthreads_or(produced)) break;
+  }
+  if (warp == 0) {  // the chains still in registers
+    const int r = lane & (kGalRows - 1);
+    if (r < nr) {
+      const int last = (int)(cptr[a0 + r + 1] - cptr[a0 + r]) - 1;
+      if (lane < kGalRows) acc[r * maxlen + last] = sum;
+      else if (cur >= 0) acc[r * maxlen + cur] = sum;
+    }
+  }
+  __syncthreads();
+  for (int r = 0; r < nr; ++r) {
+    const int64_t cb = cptr[a0 + r];
+    const int n = (int)(cptr[a0 + r + 1] - cb);
+    for (int t = threadIdx.x; t < n; t += blockDim.x)
+      if (cols[r * maxlen + t] >= a0 + r) cval[cb + t] = acc[r * maxlen + t];
   }
 }
 
@@ -700,6 +812,7 @@ mgpbd_status level_precision_copies(Handle *h, int l) {
 // per launch: per launch, one thread could lower it between another thread's
 // setting and that thread's launch, which then fails.
 constexpr int kGalerkinSmemMax = 200 * 1024;
+constexpr int kNkSmem = kNkWarps * 32 * kNkPitch * (int)sizeof(double2);
 
 __global__ void k_gal_values_k(int na, int k, const int64_t *mptr, const int32_t *mrow,
                                const int64_t *ptr, const int32_t *col, const double *val,
@@ -714,6 +827,7 @@ static mgpbd_status galerkin_smem_limits() {
   if (done) return MGPBD_OK;
   MG_CUDA(cudaFuncSetAttribute(k_gal_values, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                kGalerkinSmemMax));
+  MG_CUDA(cudaFuncSetAttribute(k_nk_sweep, cudaFuncAttributeMaxDynamicSharedMemorySize, kNkSmem));
   MG_CUDA(cudaFuncSetAttribute(k_gal_values_k, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                kGalerkinSmemMax));
   done = true;
@@ -723,17 +837,19 @@ static mgpbd_status galerkin_smem_limits() {
 static mgpbd_status galerkin_values(Handle *h, int l) {
   Level &L = h->lev[l], &Lc = h->lev[l + 1];
   int maxlen = std::max(L.max_coarse_row, 1);
-  int warps = maxlen > 1536 ? 1 : (maxlen > 384 ? 2 : 4);
-  size_t smem = (size_t)warps * maxlen * (sizeof(double) + sizeof(int));
+  // coarse rows per block: sixteen, fewer where their accumulators need more
+  // than about 48 KB
+  int rows = kGalRows;
+  while (rows > 1 && (size_t)rows * maxlen * (sizeof(double) + sizeof(int)) > 48 * 1024) rows >>= 1;
+  size_t smem = (size_t)rows * maxlen * (sizeof(double) + sizeof(int));
   if (smem > (size_t)kGalerkinSmemMax) {
     set_error("Galerkin: coarse row too long for shared memory");
     return MGPBD_E_SETUP;
   }
   MG_TRY(galerkin_smem_limits());
-  int blocks = (int)std::min<int64_t>((L.n_agg + warps - 1) / warps, 1 << 20);
-  k_gal_values<<<blocks, warps * 32, smem, h->stream>>>(L.n_agg, L.mptr, L.mrow, L.ptr, L.col,
-                                                       L.val, L.agg, L.P, Lc.ptr, Lc.col, Lc.val,
-                                                       maxlen);
+  k_gal_values<<<(L.n_agg + rows - 1) / rows, 32 * kGalWarps, smem, h->stream>>>(
+      L.n_agg, rows, L.mptr, L.mrow, L.ptr, L.col, L.val, L.agg, L.P, Lc.ptr, Lc.col, Lc.val,
+      maxlen);
   MG_LAUNCH("k_gal_values");
   k_gal_mirror<<<warp_blocks(L.n_agg), 256, 0, h->stream>>>(L.n_agg, Lc.ptr, Lc.col, Lc.val);
   MG_LAUNCH("k_gal_mirror");
@@ -1237,6 +1353,7 @@ mgpbd_status amg_setup(Handle *h) {
   }
   Level &L0 = h->lev[0];
   MG_TRY(ensure_level(h, 0, h->m, L0.nnz));
+  MG_TRY(galerkin_smem_limits());
   const int th = 256;
   // near-kernel on level 0 (Sec. 4.3)
   {
@@ -1255,8 +1372,8 @@ mgpbd_status amg_setup(Handle *h) {
                                                             amax, xa);
       MG_LAUNCH("k_nk_init");
       for (int s = 0; s < h->p.nk_sweeps; ++s) {
-        k_nk_sweep<<<warp_blocks(h->m), th, 0, h->stream>>>(h->m, L0.ptr, L0.col, L0.val,
-                                                            h->p.nk_omega, xa, xb);
+        k_nk_sweep<<<blocks_for(h->m, 32 * kNkWarps), 32 * kNkWarps, kNkSmem, h->stream>>>(
+            h->m, L0.ptr, L0.col, L0.val, h->p.nk_omega, xa, xb);
         MG_LAUNCH("k_nk_sweep");
         MG_CUDA(cudaMemcpyAsync(xa, xb, sizeof(double) * h->m, cudaMemcpyDeviceToDevice,
                                 h->stream));

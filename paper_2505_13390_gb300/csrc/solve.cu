@@ -2137,48 +2137,70 @@ mgpbd_status xpbd_step(Handle *h, mgpbd_solve_info *info) {
 // ---------------------------------------------------------------------------
 // power method for lambda_max(D^-1 A) (Sec. 4.5)
 // ---------------------------------------------------------------------------
-__global__ void k_pow_init(int n, uint64_t seed, int l, double *y) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-    y[i] = u01(h64(hkey(seed, l, i)));
+// One launch per iteration: z = D^-1 A (y / |y|) for the vector y of the step
+// before, whose norm every block folds from its partials, and the partials of
+// z.z.  lambda = |z| of the last step.
+__global__ void __launch_bounds__(kDotThreads)
+    k_pow_init(int n, uint64_t seed, int l, double *y, double *part) {
+  double acc = 0.0;
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    const double v = u01(h64(hkey(seed, l, i)));
+    y[i] = v;
+    acc = fma(v, v, acc);
+  }
+  const double s = block_sum(acc);
+  if (threadIdx.x == 0) part[blockIdx.x] = s;
 }
 
-// z_i = (A y)_i / A_ii
-__global__ void k_pow_apply(int n, const int64_t *ptr, const int32_t *col, const double *val,
-                            const double *y, double *z) {
+__global__ void __launch_bounds__(kDotThreads)
+    k_pow_step(int n, const int64_t *ptr, const int32_t *col, const double *val, const double *y,
+               const double *part_in, int n_in, double *z, double *part_out) {
+  __shared__ double scale;
+  const double yy = fold_partials(part_in, n_in);
+  if (threadIdx.x == 0) scale = yy > 0.0 ? 1.0 / sqrt(yy) : 0.0;
+  __syncthreads();
+  double acc = 0.0;
   GROUP_ROWS(4, n) {
     double s = valid ? row_dot<4, double, double, double>(ptr, col, val, y, (int)i, g) : 0.0;
     s = group_sum<4>(s);
-    if (valid && g == 0) z[i] = s / val[ptr[i + 1] - 1];
+    if (valid && g == 0) {
+      const double zi = scale * s / val[ptr[i + 1] - 1];
+      z[i] = zi;
+      acc = fma(zi, zi, acc);
+    }
   }
+  const double s = block_sum(acc);
+  if (threadIdx.x == 0) part_out[blockIdx.x] = s;
 }
 
-// lam = |z|/|y|; y = z/|z|  (s[0] = z.z, s[1] = y.y)
-__global__ void k_pow_scale(int n, const double *z, double *y, const double *s, double *lam) {
-  double nz = sqrt(s[0]), ny = sqrt(s[1]);
-  if (blockIdx.x == 0 && threadIdx.x == 0) *lam = nz / ny;
-  if (!(nz > 0.0)) return;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-    y[i] = z[i] / nz;
+__global__ void __launch_bounds__(kDotThreads)
+    k_pow_lambda(const double *part, int n, double *lam) {
+  const double s = fold_partials(part, n);
+  if (threadIdx.x == 0) *lam = sqrt(s);
 }
 
 mgpbd_status power_method(Handle *h, int l) {
   Level &L = h->lev[l];
   const int n = L.n;
   double *y = h->pp, *z = h->pq;
-  double *s = h->partials + 4096;  // 3 scalars after the partial area used by dots
-  k_pow_init<<<blocks_for(n, 256), 256, 0, h->stream>>>(n, h->p.seed_pow, l, y);
+  double *part[2] = {h->part_pq, h->part_rz};
+  int np = std::min(blocks_for(n, kDotThreads), 4 * num_sms());
+  k_pow_init<<<np, kDotThreads, 0, h->stream>>>(n, h->p.seed_pow, l, y, part[0]);
   MG_LAUNCH("k_pow_init");
+  const int blocks = std::min(row_blocks(n, 4, kDotThreads),
+                              wave_blocks((const void *)k_pow_step, kDotThreads));
   for (int it = 0; it < h->p.power_iters; ++it) {
-    k_pow_apply<<<row_blocks(n, 4), 256, 0, h->stream>>>(
-        n, L.ptr, L.col, L.val, y, z);
-    MG_LAUNCH("k_pow_apply");
-    MG_TRY(launch_dot(h, z, z, n, DOT_STORE, 0, s));
-    MG_TRY(launch_dot(h, y, y, n, DOT_STORE, 0, s + 1));
-    k_pow_scale<<<blocks_for(n, 256), 256, 0, h->stream>>>(n, z, y, s, s + 2);
-    MG_LAUNCH("k_pow_scale");
+    k_pow_step<<<blocks, kDotThreads, 0, h->stream>>>(n, L.ptr, L.col, L.val, y, part[it & 1], np,
+                                                     z, part[(it & 1) ^ 1]);
+    MG_LAUNCH("k_pow_step");
+    np = blocks;
+    std::swap(y, z);
   }
+  double *d_lam = h->partials + 4096 + 2;  // a scalar after the partials
+  k_pow_lambda<<<1, kDotThreads, 0, h->stream>>>(part[h->p.power_iters & 1], np, d_lam);
+  MG_LAUNCH("k_pow_lambda");
   double lam = 0.0;
-  MG_CUDA(cudaMemcpyAsync(&lam, s + 2, sizeof(double), cudaMemcpyDeviceToHost, h->stream));
+  MG_CUDA(cudaMemcpyAsync(&lam, d_lam, sizeof(double), cudaMemcpyDeviceToHost, h->stream));
   MG_CUDA(cudaStreamSynchronize(h->stream));
   L.lmax = lam;
   L.omega = 2.0 / (h->p.power_safety * lam + h->p.lambda_min_est);
