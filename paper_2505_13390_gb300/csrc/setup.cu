@@ -104,7 +104,7 @@ __global__ void __launch_bounds__(32 * kNkWarps)
   for (int o = 16; o > 0; o >>= 1) longest = max(longest, __shfl_xor_sync(0xffffffffu, longest, o));
   double s = 0.0;
   for (int c = 0; c < longest; c += 32) {
-#pragma unroll 4
+#pragma unroll 8
     for (int r = 0; r < 32; ++r) {
       const int64_t k = __shfl_sync(0xffffffffu, s0, r) + c + lane;
       if (k < __shfl_sync(0xffffffffu, e, r)) buf[r * kNkPitch + lane] = make_double2(val[k], x[col[k]]);
@@ -446,19 +446,23 @@ __global__ void k_gal_pattern(int na, const int64_t *mptr, const int32_t *mrow,
 // ---------------------------------------------------------------------------
 // Every coarse entry (a, b), b >= a, is one chain of fused multiply-adds over
 // the member rows of a and their storage order; the chains of different
-// entries are independent.  A block takes up to 16 coarse rows.  Seven warps
-// produce: per round each coarse row advances by up to 32 entries of a member
-// row, loaded coalesced a round ahead, whose terms (P_i A_ij, P_j) for b = a and
-// for b > a go to the two ends of a small queue in shared memory, in order.  One
-// warp consumes the queues of the round before: lane r runs the diagonal chain
-// of coarse row r, lane 16 + r its off-diagonal ones, so that one FP64
-// instruction (20 clocks of an SM on this part) advances up to 32 chains.  (One
-// warp per coarse row with a single lane adding advanced one: 5.7 ms on the
-// 40x33x40 block, 1.4 ms on the 26x10x10 beam.)
-constexpr int kGalRows = 16, kGalWarps = 8;
-constexpr int kGalPer = (kGalRows + kGalWarps - 2) / (kGalWarps - 1);  // rows per producer warp
+// entries are independent.  A block takes up to eight coarse rows.  One warp
+// per coarse row produces: each round it takes up to 32 entries of a member
+// row (loaded coalesced two rounds ahead, aggregate and weight of their columns
+// one round ahead) and puts their terms (P_i A_ij, P_j), for b = a and b > a, in
+// order, into the row's five queues in shared memory (the diagonal's, and the
+// off-diagonal entries' by their index modulo four).  Two warps consume the
+// queues of the round before: lane r of the first runs the diagonal chain of
+// coarse row r, four lanes per coarse row of the second its off-diagonal ones.
+// What bounds it is the chains' latency and, with one lane adding per warp,
+// FP64 issue (a warp's FP64 instruction holds its SM for 20 clocks).  On the
+// 40x33x40 block's 60M entries one warp per coarse row that folded through lane
+// 0 took 5.7 ms; sixteen rows per block, three to a producer warp and one lane
+// per row for its off-diagonal chains 3.8 ms; eight rows, a producer each 2.28
+// ms; four lanes that skip each other's terms 2.49 ms; a queue per lane 1.93 ms.
+constexpr int kGalRows = 8, kGalWarps = kGalRows + 2;
 
-__global__ void __launch_bounds__(32 * kGalWarps)
+__global__ void __launch_bounds__(32 * kGalWarps, 3)
     k_gal_values(int na, int rows, const int64_t *mptr, const int32_t *mrow, const int64_t *ptr,
                  const int32_t *col, const double *val, const int32_t *agg, const double *P,
                  const int64_t *cptr, const int32_t *ccol, double *cval, int maxlen) {
@@ -467,147 +471,152 @@ __global__ void __launch_bounds__(32 * kGalWarps)
   int *const cols = reinterpret_cast<int *>(acc + (size_t)rows * maxlen);
   __shared__ double2 term[2][kGalRows][32];
   __shared__ uint16_t slot[2][kGalRows][32];
-  __shared__ int n_diag[2][kGalRows], n_off[2][kGalRows];
+  __shared__ uint8_t ends[2][kGalRows][8];  // queue q of a row: terms ends[q-1] .. ends[q]
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const unsigned below = (1u << lane) - 1u;
   const int a0 = blockIdx.x * rows, nr = min(rows, na - a0);
   for (int r = 0; r < nr; ++r) {
     const int64_t cb = cptr[a0 + r];
-    const int len = (int)(cptr[a0 + r + 1] - cb);
-    for (int t = threadIdx.x; t < len; t += blockDim.x) {
+    const int n = (int)(cptr[a0 + r + 1] - cb);
+    for (int t = threadIdx.x; t < n; t += blockDim.x) {
       acc[r * maxlen + t] = 0.0;
       cols[r * maxlen + t] = ccol[cb + t];
     }
   }
-  if (threadIdx.x < 2 * kGalRows) (&n_diag[0][0])[threadIdx.x] = (&n_off[0][0])[threadIdx.x] = 0;
+  for (int t = threadIdx.x; t < 2 * kGalRows * 8; t += blockDim.x) (&ends[0][0][0])[t] = 0;
 
-  // producers: per owned coarse row the member being read, its entry range and
-  // weight, the next member's, and the chunk in flight
-  int64_t q[kGalPer], qe[kGalPer], k[kGalPer], e[kGalPer], kn[kGalPer], en[kGalPer];
-  double pi[kGalPer], pn[kGalPer], v[kGalPer];
-  int c[kGalPer], len[kGalPer];
-  auto next_member = [&](int o) {  // the member after q, ahead of time
-    if (q[o] + 1 < qe[o]) {
-      const int i = mrow[q[o] + 1];
-      kn[o] = ptr[i];
-      en[o] = ptr[i + 1];
-      pn[o] = P[i];
+  // a producer's coarse row, the member row being read, the next one, the
+  // chunk whose entries are in flight (1) and the one whose columns' aggregates
+  // and weights are (0)
+  const int r = warp - 2;
+  const int a = a0 + r;
+  int64_t q = 0, qe = 0, k = 0, e = 0, kn = 0, en = 0;
+  double pi = 0.0, pn = 0.0, v1 = 0.0, p1 = 0.0, t0 = 0.0, pj0 = 0.0;
+  int c1 = 0, b0 = -1, len = 0;
+  bool have0 = false, have1 = false, in0 = false, in1 = false;
+  auto next_member = [&]() {  // the member after q, ahead of time
+    if (q + 1 < qe) {
+      const int i = mrow[q + 1];
+      kn = ptr[i];
+      en = ptr[i + 1];
+      pn = P[i];
     }
   };
-  auto load_chunk = [&](int o) {
-    if (q[o] < qe[o] && k[o] + lane < e[o]) {
-      c[o] = col[k[o] + lane];
-      v[o] = val[k[o] + lane];
+  auto load_chunk = [&]() {  // the next chunk's entries; then step past it
+    have1 = q < qe;
+    if (!have1) return;
+    in1 = k + lane < e;
+    if (in1) {
+      c1 = col[k + lane];
+      v1 = val[k + lane];
+    }
+    p1 = pi;
+    k += 32;
+    if (k >= e) {
+      ++q;
+      k = kn;
+      e = en;
+      pi = pn;
+      next_member();
     }
   };
-#pragma unroll
-  for (int o = 0; o < kGalPer; ++o) {
-    const int r = warp - 1 + o * (kGalWarps - 1);
-    q[o] = qe[o] = 0;
-    if (warp > 0 && r < nr) {
-      q[o] = mptr[a0 + r];
-      qe[o] = mptr[a0 + r + 1];
-      len[o] = (int)(cptr[a0 + r + 1] - cptr[a0 + r]);
-      if (q[o] < qe[o]) {
-        const int i = mrow[q[o]];
-        k[o] = ptr[i];
-        e[o] = ptr[i + 1];
-        pi[o] = P[i];
-        next_member(o);
-        load_chunk(o);
-      }
+  auto gather_chunk = [&]() {  // chunk 1 becomes chunk 0
+    have0 = have1;
+    in0 = have0 && in1;
+    if (!in0) return;
+    b0 = agg[c1];
+    pj0 = P[c1];
+    t0 = p1 * v1;
+  };
+  if (warp >= 2 && r < nr) {
+    q = mptr[a];
+    qe = mptr[a + 1];
+    len = (int)(cptr[a + 1] - cptr[a]);
+    if (q < qe) {
+      const int i = mrow[q];
+      k = ptr[i];
+      e = ptr[i + 1];
+      pi = P[i];
+      next_member();
     }
+    load_chunk();
+    gather_chunk();
+    load_chunk();
   }
   __syncthreads();
 
-  int cur = -1;       // consumer: the entry whose chain is in a register
+  const int ro = lane >> 2;  // second consumer: coarse row
+  int cur = -1;              // the entry whose chain is in a register
   double sum = 0.0;
   for (int buf = 0;; buf ^= 1) {
     int produced = 0;
-    if (warp == 0) {
-      const int r = lane & (kGalRows - 1);
-      const bool diag = lane < kGalRows;
+    if (warp >= 2) {
       if (r < nr) {
-        const int b = buf ^ 1, n = diag ? n_diag[b][r] : n_off[b][r];
-        double *const A = acc + r * maxlen;
-        for (int t = 0; t < n; ++t) {
-          const int at = diag ? t : 31 - t;
-          const double2 x = term[b][r][at];
-          const int s = diag ? 0 : slot[b][r][at];  // the diagonal stays in the register
-          if (s != cur) {
-            if (cur >= 0) A[cur] = sum;
-            sum = diag ? 0.0 : A[s];
-            cur = s;
+        if (have0) {
+          produced = 1;
+          const bool isd = in0 && b0 == a, iso = in0 && b0 > a;
+          int lo = 0, queue = isd ? 0 : -1;
+          if (iso) {
+            const int *C = cols + r * maxlen;
+            int hi = len - 1;
+            while (lo < hi) {
+              const int mid = (lo + hi) >> 1;
+              if (C[mid] < b0) lo = mid + 1;
+              else hi = mid;
+            }
+            queue = 1 + (lo & 3);
           }
-          sum = fma(x.x, x.y, sum);
+          int at = 0, end = 0;
+#pragma unroll
+          for (int t = 0; t < 5; ++t) {
+            const unsigned m = __ballot_sync(0xffffffffu, queue == t);
+            if (queue == t) at = end + __popc(m & below);
+            end += __popc(m);
+            if (lane == t) ends[buf][r][t] = (uint8_t)end;
+          }
+          if (queue >= 0) {
+            term[buf][r][at] = make_double2(t0, pj0);
+            slot[buf][r][at] = (uint16_t)lo;
+          }
+          gather_chunk();
+          load_chunk();
+        } else if (lane < 5) {
+          ends[buf][r][lane] = 0;
         }
       }
-    } else {
-#pragma unroll
-      for (int o = 0; o < kGalPer; ++o) {
-        const int r = warp - 1 + o * (kGalWarps - 1);
-        if (r >= nr) break;
-        const int a = a0 + r;
-        if (q[o] >= qe[o]) {
-          if (lane == 0) n_diag[buf][r] = n_off[buf][r] = 0;
-          continue;
+    } else if (warp == 0) {
+      if (lane < nr) {
+        const double2 *const x = term[buf ^ 1][lane];
+        const int n = ends[buf ^ 1][lane][0];
+#pragma unroll 4
+        for (int t = 0; t < n; ++t) sum = fma(x[t].x, x[t].y, sum);
+      }
+    } else if (ro < nr) {
+      const int n = ends[buf ^ 1][ro][1 + (lane & 3)];
+      double *const A = acc + ro * maxlen;
+      for (int t = ends[buf ^ 1][ro][lane & 3]; t < n; ++t) {
+        const double2 y = term[buf ^ 1][ro][t];
+        const int s = slot[buf ^ 1][ro][t];
+        if (s != cur) {
+          if (cur >= 0) A[cur] = sum;
+          sum = A[s];
+          cur = s;
         }
-        produced = 1;
-        const bool in = k[o] + lane < e[o];
-        int b = -1;
-        double pj = 0.0;
-        const double t = pi[o] * v[o];
-        if (in) {
-          b = agg[c[o]];
-          pj = P[c[o]];
-        }
-        // the next chunk's loads before this one is placed
-        k[o] += 32;
-        if (k[o] >= e[o]) {
-          ++q[o];
-          k[o] = kn[o];
-          e[o] = en[o];
-          pi[o] = pn[o];
-          next_member(o);
-        }
-        load_chunk(o);
-        const bool isd = in && b == a, iso = in && b > a;
-        const unsigned md = __ballot_sync(0xffffffffu, isd), mo = __ballot_sync(0xffffffffu, iso);
-        if (isd) term[buf][r][__popc(md & below)] = make_double2(t, pj);
-        if (iso) {
-          const int *C = cols + r * maxlen;
-          int lo = 0, hi = len[o] - 1;
-          while (lo < hi) {
-            const int mid = (lo + hi) >> 1;
-            if (C[mid] < b) lo = mid + 1;
-            else hi = mid;
-          }
-          const int at = 31 - __popc(mo & below);
-          term[buf][r][at] = make_double2(t, pj);
-          slot[buf][r][at] = (uint16_t)lo;
-        }
-        if (lane == 0) {
-          n_diag[buf][r] = __popc(md);
-          n_off[buf][r] = __popc(mo);
-        }
+        sum = fma(y.x, y.y, sum);
       }
     }
     if (!__syncthreads_or(produced)) break;
   }
-  if (warp == 0) {  // the chains still in registers
-    const int r = lane & (kGalRows - 1);
-    if (r < nr) {
-      const int last = (int)(cptr[a0 + r + 1] - cptr[a0 + r]) - 1;
-      if (lane < kGalRows) acc[r * maxlen + last] = sum;
-      else if (cur >= 0) acc[r * maxlen + cur] = sum;
-    }
-  }
+  // the chains still in registers
+  if (warp == 0 && lane < nr)
+    acc[lane * maxlen + (int)(cptr[a0 + lane + 1] - cptr[a0 + lane]) - 1] = sum;
+  if (warp == 1 && ro < nr && cur >= 0) acc[ro * maxlen + cur] = sum;
   __syncthreads();
-  for (int r = 0; r < nr; ++r) {
-    const int64_t cb = cptr[a0 + r];
-    const int n = (int)(cptr[a0 + r + 1] - cb);
+  for (int o = 0; o < nr; ++o) {
+    const int64_t cb = cptr[a0 + o];
+    const int n = (int)(cptr[a0 + o + 1] - cb);
     for (int t = threadIdx.x; t < n; t += blockDim.x)
-      if (cols[r * maxlen + t] >= a0 + r) cval[cb + t] = acc[r * maxlen + t];
+      if (cols[o * maxlen + t] >= a0 + o) cval[cb + t] = acc[o * maxlen + t];
   }
 }
 
@@ -837,7 +846,7 @@ static mgpbd_status galerkin_smem_limits() {
 static mgpbd_status galerkin_values(Handle *h, int l) {
   Level &L = h->lev[l], &Lc = h->lev[l + 1];
   int maxlen = std::max(L.max_coarse_row, 1);
-  // coarse rows per block: sixteen, fewer where their accumulators need more
+  // coarse rows per block: eight, fewer where their accumulators need more
   // than about 48 KB
   int rows = kGalRows;
   while (rows > 1 && (size_t)rows * maxlen * (sizeof(double) + sizeof(int)) > 48 * 1024) rows >>= 1;
