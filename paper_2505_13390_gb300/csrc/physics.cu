@@ -313,42 +313,109 @@ __device__ __forceinline__ int row_setup(int i, int E, const int32_t *edge, cons
 // Off-diagonal values of A (eq. 3, Sec. 4.2 formulas), G lanes per row over its
 // entries, and in mixed precision their FP32 mirrors.  Bound by FP64 issue (a
 // warp's FP64 instruction holds its SM for 20 clocks whatever number of lanes
-// is active), so the lanes per row follow the row length, and the diagonal,
-// one value per row with a division, has a kernel of its own with one row per
-// lane: as lane 0's extra work here it took more issue slots than the
-// off-diagonals (2.2 ms for both on the 40x33x40 block's 60M entries).
+// is active).  So the lanes per row follow the row length; the diagonal, one
+// value per row with a division, has a kernel of its own with one row per lane;
+// and every entry adds its first shared vertex at once, while those with a
+// second and third one (tets that share an edge or a face) go to the warp's
+// stack in shared memory and are worked off 32 at a time, one vertex per turn.
+// On the 40x33x40 block's 60M entries: 2.2 ms with the diagonal as lane 0's
+// extra work, 1.45 ms with every lane looping over its own entry's vertices,
+// 1.08 ms with the stack.
+constexpr int kAsmWarps = 8, kAsmBatches = 8;
+
+struct AsmItem {
+  double acc;
+  int64_t k;
+  int i, j;
+};
+
 template <int G>
-__global__ void __launch_bounds__(256)
-    k_assemble(int m, int E, const int32_t *edge, const int32_t *tet, const double *w,
+__global__ void __launch_bounds__(32 * kAsmWarps)
+    k_assemble(int m, int E, int batches, const int32_t *edge, const int32_t *tet, const double *w,
                const double *gd, const double *gt, const int64_t *ptr, const int32_t *col,
                const uint16_t *map, double *val, float *val32) {
-  const int g = threadIdx.x & (G - 1);
-  const int64_t ii = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / G;
-  if (ii >= m) return;
-  const int i = (int)ii;
-  const int64_t e = ptr[i + 1] - 1;
-  double gi[4][3], wi[4];
-  row_setup(i, E, edge, tet, w, gd, gt, gi, wi);
-  for (int64_t k = ptr[i] + g; k < e; k += G) {
-    int j = col[k];
-    unsigned code = map[k];
-    int ns = code & 3;
-    double acc = 0.0;
-    for (int p = 0; p < ns; ++p) {
-      const int si = (code >> (2 + 4 * p)) & 3, sj = (code >> (4 + 4 * p)) & 3;
-      double gj[3];
-      row_grad(j, sj, E, gd, gt, gj);
-      // (selected, not indexed: the row's gradients stay in registers)
-      double gs[3], ws;
-#pragma unroll
-      for (int d = 0; d < 3; ++d)
-        gs[d] = si == 0 ? gi[0][d] : (si == 1 ? gi[1][d] : (si == 2 ? gi[2][d] : gi[3][d]));
-      ws = si == 0 ? wi[0] : (si == 1 ? wi[1] : (si == 2 ? wi[2] : wi[3]));
-      acc = fma(ws, gdot(gs, gj), acc);
-    }
+  __shared__ AsmItem items[kAsmWarps][64];
+  __shared__ uint16_t codes[kAsmWarps][64];
+  const int lane = threadIdx.x & 31, g = threadIdx.x & (G - 1);
+  AsmItem *const item = items[threadIdx.x >> 5];
+  uint16_t *const code_of = codes[threadIdx.x >> 5];
+  const unsigned below = (1u << lane) - 1u;
+  int n = 0;  // items on the warp's stack
+
+  auto put = [&](int64_t k, double acc) {
     val[k] = acc;
     if (val32) val32[k] = f64_to_f32(acc);
+  };
+  // code: vertices left (2 bits), then the slots in i and j of each
+  auto push = [&](bool more, const AsmItem &x, unsigned code) {
+    const unsigned mask = __ballot_sync(0xffffffffu, more);
+    if (more) {
+      const int at = n + __popc(mask & below);
+      item[at] = x;
+      code_of[at] = (uint16_t)(((code >> 6) << 2) | ((code & 3) - 1));
+    }
+    n += __popc(mask);
+    __syncwarp();
+  };
+  auto work_off = [&]() {  // one vertex of the top 32 items
+    const int take = min(n, 32);
+    n -= take;
+    AsmItem x;
+    unsigned code = 0;
+    if (lane < take) {
+      x = item[n + lane];
+      code = code_of[n + lane];
+    }
+    __syncwarp();
+    if (lane < take) {
+      const int si = (code >> 2) & 3, sj = (code >> 4) & 3;
+      double gi[3], gj[3];
+      row_grad(x.i, si, E, gd, gt, gi);
+      row_grad(x.j, sj, E, gd, gt, gj);
+      const int v = x.i < E ? edge[2 * (int64_t)x.i + si] : tet[4 * (int64_t)(x.i - E) + si];
+      x.acc = fma(w[v], gdot(gi, gj), x.acc);
+      if ((code & 3) == 1) put(x.k, x.acc);
+    }
+    push((code & 3) > 1, x, code);
+  };
+
+  const int64_t warp = blockIdx.x * (int64_t)kAsmWarps + (threadIdx.x >> 5);
+  for (int b = 0; b < batches; ++b) {
+    const int64_t row = (warp * batches + b) * (32 / G) + lane / G;
+    const int i = (int)min(row, (int64_t)m - 1);
+    int64_t k = ptr[i] + g;
+    const int64_t e = row < m ? ptr[i + 1] - 1 : 0;
+    double gi[4][3], wi[4];
+    row_setup(i, E, edge, tet, w, gd, gt, gi, wi);
+    while (__any_sync(0xffffffffu, k < e)) {
+      AsmItem x;
+      unsigned code = 0;
+      if (k < e) {
+        x.j = col[k];
+        code = map[k];
+        x.acc = 0.0;
+        x.k = k;
+        x.i = i;
+        const int si = (code >> 2) & 3, sj = (code >> 4) & 3;
+        if (code & 3) {
+          double gj[3];
+          row_grad(x.j, sj, E, gd, gt, gj);
+          // (selected, not indexed: the row's gradients stay in registers)
+          double gs[3], ws;
+#pragma unroll
+          for (int d = 0; d < 3; ++d)
+            gs[d] = si == 0 ? gi[0][d] : (si == 1 ? gi[1][d] : (si == 2 ? gi[2][d] : gi[3][d]));
+          ws = si == 0 ? wi[0] : (si == 1 ? wi[1] : (si == 2 ? wi[2] : wi[3]));
+          x.acc = fma(ws, gdot(gs, gj), 0.0);
+        }
+        if ((code & 3) < 2) put(k, x.acc);
+      }
+      push((code & 3) > 1, x, code);
+      while (n >= 32) work_off();
+      k += G;
+    }
   }
+  while (n) work_off();
 }
 
 // diagonal of A and its reciprocal, one row per thread
@@ -379,9 +446,13 @@ mgpbd_status launch_assemble(Handle *h) {
   Level &L = h->lev[0];
   const double avg = (double)L.nnz / h->m;
   auto off = [&](auto *kernel, int G) -> mgpbd_status {
-    const int64_t blocks = ((int64_t)h->m * G + 255) / 256;
-    kernel<<<(unsigned)blocks, 256, 0, h->stream>>>(h->m, h->E, h->edge, h->tet, h->w, h->gd,
-                                                    h->gt, L.ptr, L.col, h->map, L.val, L.val32);
+    // more rows per warp fill the stack better, once every SM has its 64 warps
+    const int64_t warps = ((int64_t)h->m * G + 31) / 32;
+    const int batches = (int)std::min<int64_t>(std::max<int64_t>(warps / (64 * num_sms()), 1), kAsmBatches);
+    const int64_t per = (int64_t)kAsmWarps * batches;
+    kernel<<<(unsigned)((warps + per - 1) / per), 32 * kAsmWarps, 0, h->stream>>>(
+        h->m, h->E, batches, h->edge, h->tet, h->w, h->gd, h->gt, L.ptr, L.col, h->map, L.val,
+        L.val32);
     MG_LAUNCH("k_assemble");
     return MGPBD_OK;
   };
