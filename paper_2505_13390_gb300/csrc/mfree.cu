@@ -40,8 +40,17 @@ constexpr int kUStride = 3, kUStrideDf = 4;
 // one, its time is that of its dependent loads, and its 40 to 80 registers
 // cost nothing.  Above it the plain form's occupancy counts.
 constexpr int kEarlyRows = 1 << 17;
+// tet instances of up to this many rows start with eight FP64 lanes per vertex
+constexpr int kShortListRows = 1 << 17;
 // threads of the early vertex passes: small blocks, for more SMs (reduce.cuh)
 constexpr int kVertexThreads = 64;
+// The early forms have one thread per row and one group per vertex, without a
+// loop: the vertices are limited too, and a pass with a dot product, which
+// leaves one partial per block, by the partials the handle holds.
+constexpr int kEarlyDotRows = 4096 * kDotThreads;
+static bool early(const Handle *h, bool dot = false) {
+  return h->m <= (dot ? std::min(kEarlyRows, kEarlyDotRows) : kEarlyRows) && h->N <= kEarlyRows;
+}
 
 // slot of vertex v in each incident row (create time)
 __global__ void k_vslot(int N, int E, const int32_t *edge, const int32_t *tet, const int64_t *vptr,
@@ -716,7 +725,7 @@ mgpbd_status mf_create(Handle *h) {
   // FP64 lanes per vertex until the autotuner says otherwise: four (fewest FP64
   // additions), but on small instances of long incidence lists (tet meshes:
   // about thirty) eight, so that most lists are one batch of loads
-  if (h->m <= kEarlyRows && ninc > 16 * (int64_t)h->N) h->mf_g64 = 8;
+  if (h->m <= kShortListRows && ninc > 16 * (int64_t)h->N) h->mf_g64 = 8;
   // Vertex-pass order: within windows of kOrderWindow consecutive vertices,
   // by incidence count (then id).  A G-lane group loops over its vertex's
   // incidences, so a warp costs its longest vertex; neighbouring vertices of
@@ -754,9 +763,10 @@ static int mf_grid(int64_t rows, int threads) {
 
 // blocks of a row pass with a dot product (its partials are one per block)
 template <class T, int MODE>
-static int mf_dot_grid(int m) {
-  return std::min((m + kDotThreads - 1) / kDotThreads,
-                  wave_blocks((const void *)k_mf_row<T, MODE>, kDotThreads));
+static int mf_dot_grid(const Handle *h) {
+  const int blocks = blocks_for(h->m, kDotThreads);
+  if (early(h, true)) return blocks;  // one row per thread, as mf_row_launch has it
+  return std::min(blocks, wave_blocks((const void *)k_mf_row<T, MODE>, kDotThreads));
 }
 
 template <class T, int MODE>
@@ -764,11 +774,11 @@ static mgpbd_status mf_row_launch(Handle *h, const char *what, int blocks, const
                                   const T *gt, const T *u, const T *at, const T *x, const T *b,
                                   const T *dinv, T omega, T *out, const DotCtx &c, double *z,
                                   const double *rr, const int32_t *pos) {
-  if (h->m <= kEarlyRows)
+  const bool dot = MODE == MF_APPLY_DOT || MODE == MF_SWEEP_ZDOT;
+  if (early(h, dot))
     return chain_launch(h, what, k_mf_row_early<T, MODE>, blocks_for(h->m, kDotThreads),
                         kDotThreads, h->E, h->m, h->edge, h->tet, gd, gt, u, at, x, b, dinv,
                         omega, out, c, z, rr, pos);
-  const bool dot = MODE == MF_APPLY_DOT || MODE == MF_SWEEP_ZDOT;
   return chain_launch(h, what, k_mf_row<T, MODE>, blocks, dot ? kDotThreads : 256, h->E, h->m,
                       h->edge, h->tet, gd, gt, u, at, x, b, dinv, omega, out, c, z, rr, pos);
 }
@@ -892,9 +902,9 @@ void mf_cohort_grids(const Handle *h, int grid[CS_STEPS]) {
   const int g32 = h->force_vert32 ? h->force_vert32 : h->mf_g32;
   MF_G_DISPATCH(g64, (grid[CS_VERT64] = mf_vertex_blocks(h, GG)));
   MF_G_DISPATCH(g32, (grid[CS_VERT32] = mf_vertex_blocks(h, GG)));
-  grid[CS_ROW_PQ] = mf_dot_grid<double, MF_APPLY_DOT>(h->m);
+  grid[CS_ROW_PQ] = mf_dot_grid<double, MF_APPLY_DOT>(h);
   grid[CS_ROW] = mf_grid(h->m, 256);
-  grid[CS_ROW_FINAL] = mf_dot_grid<float, MF_SWEEP_ZDOT>(h->m);
+  grid[CS_ROW_FINAL] = mf_dot_grid<float, MF_SWEEP_ZDOT>(h);
 }
 
 mgpbd_status mf_cohort_step(int which, int sel, const CohortMember *d_mem,
@@ -928,7 +938,7 @@ mgpbd_status mf_cohort_step(int which, int sel, const CohortMember *d_mem,
 static mgpbd_status mf_vertex(Handle *h, const double *x, int G = 0, bool check_done = true) {
   if (G == 0) G = h->force_vert64 ? h->force_vert64 : h->mf_g64;
   const PcgScalars *sc = check_done ? h->sc : nullptr;
-  if (h->m <= kEarlyRows) {
+  if (early(h)) {
     MF_G_DISPATCH(G, MG_TRY(chain_launch(h, "k_mf_vertex64", k_mf_vertex64_early<GG>,
                                           blocks_for((int64_t)h->N * GG, kVertexThreads),
                                           kVertexThreads, h->N, h->vorder, h->vptr, h->vrow,
@@ -944,7 +954,7 @@ static mgpbd_status mf_vertex(Handle *h, const double *x, int G = 0, bool check_
 static mgpbd_status mf_vertex(Handle *h, const float *x, int G = 0, bool check_done = true) {
   if (G == 0) G = h->force_vert32 ? h->force_vert32 : h->mf_g32;
   const PcgScalars *sc = check_done ? h->sc : nullptr;
-  if (h->m <= kEarlyRows) {
+  if (early(h)) {
     MF_G_DISPATCH(G, MG_TRY(chain_launch(h, "k_mf_vertex32", k_mf_vertex32_early<GG>,
                                           blocks_for((int64_t)h->N * GG, kVertexThreads),
                                           kVertexThreads, h->N, h->vorder, h->vptr, h->ginc4,
@@ -1022,7 +1032,7 @@ mgpbd_status mf_apply_pq_form(Handle *h, bool pairs, const double *p, double *q,
     return MGPBD_OK;
   }
   MG_TRY(mf_vertex(h, p));
-  h->n_pq = mf_dot_grid<double, MF_APPLY_DOT>(h->m);
+  h->n_pq = mf_dot_grid<double, MF_APPLY_DOT>(h);
   MG_TRY(mf_row_launch<double, MF_APPLY_DOT>(
       h, "k_mf_row(A.p)", h->n_pq, h->gd, h->gt, h->u64, h->alpha_t, p, nullptr, nullptr, 0.0, q, c,
       nullptr, nullptr, nullptr));
@@ -1118,7 +1128,7 @@ mgpbd_status mf_level0_final(Handle *h, const T *x, const T *b, const T *dinv, T
   const T *at = dbl ? (const T *)h->alpha_t : (const T *)h->at32;
   DotCtx c = o.c;
   c.sc = h->sc;
-  if (o.dot) h->n_rz = mf_dot_grid<T, MF_SWEEP_ZDOT>(h->m);
+  if (o.dot) h->n_rz = mf_dot_grid<T, MF_SWEEP_ZDOT>(h);
   if (o.dot)
     MG_TRY(mf_row_launch<T, MF_SWEEP_ZDOT>(
         h, "k_mf_row(final sweep)",
