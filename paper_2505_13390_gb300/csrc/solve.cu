@@ -773,32 +773,43 @@ __device__ __forceinline__ void tile_put(double *M, int n, int ti, int tj, int r
   if (gr < n && gc < n) M[(int64_t)gr * n + gc] = v;
 }
 
-// Cholesky of the tile in D (lower part, in place) and, in the same
-// right-looking loop, the inverse X of the lower factor (X starts as the
-// identity; step j scales row j of X by 1/L_jj and subtracts L_ij times it
-// from the rows below).  False on a pivot <= 0 (the same in every thread).
-__device__ bool tile_factor(double (*D)[kCT + 1], double (*X)[kCT + 1], double *rinv, int *bad) {
+// Cholesky of the tile in D (lower part) and, in the same right-looking loop,
+// the inverse X of the lower factor (X starts as the identity; step j scales
+// row j of X by 1/L_jj and subtracts L_ij times it from the rows below).
+// Thread (r, c) keeps one element in a register, D_rc while c > j and X_rc from
+// step c on, so a step is one multiply-add for the whole tile; column j of D
+// and row j of X pass through `col` and `row` to the first warp, which scales
+// both by 1 / sqrt(D_jj) in one instruction (L_jj itself is not needed).  The
+// chain of that root bounds it (a warp's dependent FP64 instructions are 80
+// clocks apart): a panel launch took 20.4 us with a root, a division and three
+// barriers per step, 24.2 us with the whole tile in one warp, 11.8 us so.
+// False on a pivot <= 0 (the same in every thread).
+struct TileStep {
+  double col[kCT], row[kCT];   // D_rj, X_jc before the scaling
+  double lcol[kCT], lrow[kCT]; // and after
+  int bad;
+};
+
+__device__ __forceinline__ bool tile_factor(double x, double (*X)[kCT + 1], TileStep &s) {
   const int t = threadIdx.x, r = t / kCT, c = t % kCT;
-  X[r][c] = r == c ? 1.0 : 0.0;
+  if (t == 0) s.bad = 0;
+  if (c == 0) s.col[r] = x;
+  if (r == 0) s.row[c] = c == 0 ? 1.0 : 0.0;
+  __syncthreads();
   for (int j = 0; j < kCT; ++j) {
-    if (t == 0) {
-      const double d = D[j][j];
-      if (!(d > 0.0)) {
-        *bad = 1;
-      } else {
-        const double l = sqrt(d);
-        D[j][j] = l;
-        *rinv = 1.0 / l;
-      }
+    if (t < 2 * kCT) {
+      const double d = s.col[j];
+      const double v = (t < kCT ? s.col[t] : s.row[t - kCT]) * rsqrt(d);
+      if (!(d > 0.0)) s.bad = 1;
+      (t < kCT ? s.lcol[t] : s.lrow[t - kCT]) = v;
     }
     __syncthreads();
-    if (*bad) return false;
-    const double inv = *rinv;
-    if (c == j && r > j) D[r][j] = D[r][j] * inv;
-    if (r == j && c <= j) X[j][c] = X[j][c] * inv;
-    __syncthreads();
-    if (c > j && r >= c) D[r][c] = fma(-D[r][j], D[c][j], D[r][c]);
-    if (r > j && c <= j) X[r][c] = fma(-D[r][j], X[j][c], X[r][c]);
+    if (s.bad) return false;
+    if (c == j) x = r == j ? 1.0 : 0.0;  // X_rj: still the identity's
+    if (r == j) X[j][c] = c <= j ? s.lrow[c] : 0.0;
+    if (r > j) x = fma(-s.lcol[r], c > j ? s.lcol[c] : s.lrow[c], x);
+    if (c == j + 1) s.col[r] = x;
+    if (r == j + 1) s.row[c] = c <= j ? x : (c == j + 1 ? 1.0 : 0.0);
     __syncthreads();
   }
   return true;
@@ -811,37 +822,34 @@ __device__ bool tile_factor(double (*D)[kCT + 1], double (*X)[kCT + 1], double *
 __global__ void __launch_bounds__(kCThreads) k_chol_panel(int n, int T, int k, double *A,
                                                           double *Li, int *status) {
   __shared__ double D[kCT][kCT + 1], X[kCT][kCT + 1];
-  __shared__ double rinv;
-  __shared__ int bad;
+  __shared__ TileStep step;
   if (chol_failed(status)) return;
   const int t = threadIdx.x, r = t / kCT, c = t % kCT;
-  if (t == 0) bad = 0;
-  D[r][c] = tile_get(A, n, k, k, r, c, true);
-  __syncthreads();
-  if (!tile_factor(D, X, &rinv, &bad)) {
-    if (blockIdx.x == 0 && t == 0) *status = MGPBD_E_SINGULAR;
+  const int b = blockIdx.x, i = k + b, j = b - (T - k);
+  const bool below = b < T - k;
+  const double akk = tile_get(A, n, k, k, r, c, true);
+  // this block's own tile, loaded while the factor is formed
+  const double own = b == 0 ? 0.0
+                            : (below ? tile_get(A, n, i, k, r, c, false)
+                                     : tile_get(Li, n, k, j, r, c, false));
+  if (!tile_factor(akk, X, step)) {
+    if (b == 0 && t == 0) *status = MGPBD_E_SINGULAR;
     return;
   }
-  const int b = blockIdx.x;
   if (b == 0) {
     tile_put(Li, n, k, k, r, c, X[r][c]);
     return;
   }
-  if (b < T - k) {  // L_ik = A_ik L_kk^-T, i = k + b
-    const int i = k + b;
-    D[r][c] = tile_get(A, n, i, k, r, c, false);  // D is free after the factor
-    __syncthreads();
-    double s = 0.0;
-    for (int q = 0; q <= c; ++q) s = fma(D[r][q], X[c][q], s);
-    tile_put(A, n, i, k, r, c, s);
-    return;
-  }
-  const int j = b - (T - k);  // Li_kj = L_kk^-1 S_kj
-  D[r][c] = tile_get(Li, n, k, j, r, c, false);
+  D[r][c] = own;
   __syncthreads();
   double s = 0.0;
-  for (int q = 0; q <= r; ++q) s = fma(X[r][q], D[q][c], s);
-  tile_put(Li, n, k, j, r, c, s);
+  if (below) {  // L_ik = A_ik L_kk^-T, i = k + b
+    for (int q = 0; q <= c; ++q) s = fma(D[r][q], X[c][q], s);
+    tile_put(A, n, i, k, r, c, s);
+  } else {  // Li_kj = L_kk^-1 S_kj
+    for (int q = 0; q <= r; ++q) s = fma(X[r][q], D[q][c], s);
+    tile_put(Li, n, k, j, r, c, s);
+  }
 }
 
 // trailing update after tile column k: block (x, y) is tile column x of tile
