@@ -36,10 +36,12 @@ constexpr int kUStride = 3, kUStrideDf = 4;
 
 // Up to this many rows the passes run in their early form (k_mf_row_early,
 // k_mf_vertex32_early, k_mf_vertex64_early: one row or vertex per thread
-// group, static loads before the wait): the kernel is a small part of a wave or
-// one, its time is that of its dependent loads, and its 40 to 80 registers
-// cost nothing.  Above it the plain form's occupancy counts.
-constexpr int kEarlyRows = 1 << 17;
+// group, static loads before the wait): the kernel is a few waves or less, its
+// time is that of its dependent loads, and its 40 to 80 registers cost little.
+// Above it the plain form's occupancy counts.  Early against plain form: V-cycle
+// on 594,000 rows 201 against 210 us; Chebyshev frame on 195,585 rows 62.3
+// against 62.5 ms; 300 PCG iterations on 3.7M rows 255 against 241 ms.
+constexpr int kEarlyRows = 1 << 20;
 // tet instances of up to this many rows start with eight FP64 lanes per vertex
 constexpr int kShortListRows = 1 << 17;
 // threads of the early vertex passes: small blocks, for more SMs (reduce.cuh)
