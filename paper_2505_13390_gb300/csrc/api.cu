@@ -69,9 +69,9 @@ mgpbd_status prof_end(Handle *h, int ch) {
   return MGPBD_OK;
 }
 
-// Whether the timed launch of PCG iteration `it` ran in a solve that took
-// `iters` iterations: iteration k's A.p runs before its convergence test,
-// its V-cycle after it (kernels return at once after the solve has finished).
+// Whether the timed launch of PCG iteration `it` counts in a solve that took
+// `iters` iterations.  Convergence is tested at an iteration's end, so the last
+// one's V-cycle runs as well, but nothing uses it: its sweeps are left out.
 static bool prof_ran(int ch, int it, int iters) {
   return ch == PROF_AP ? it <= iters - 1 : it <= iters - 2;
 }

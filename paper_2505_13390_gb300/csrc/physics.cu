@@ -448,7 +448,8 @@ mgpbd_status launch_assemble(Handle *h) {
   auto off = [&](auto *kernel, int G) -> mgpbd_status {
     // more rows per warp fill the stack better, once every SM has its 64 warps
     const int64_t warps = ((int64_t)h->m * G + 31) / 32;
-    const int batches = (int)std::min<int64_t>(std::max<int64_t>(warps / (64 * num_sms()), 1), kAsmBatches);
+    const int64_t full = warps / (64 * num_sms());
+    const int batches = (int)std::min<int64_t>(std::max<int64_t>(full, 1), kAsmBatches);
     const int64_t per = (int64_t)kAsmWarps * batches;
     kernel<<<(unsigned)((warps + per - 1) / per), 32 * kAsmWarps, 0, h->stream>>>(
         h->m, h->E, batches, h->edge, h->tet, h->w, h->gd, h->gt, L.ptr, L.col, h->map, L.val,

@@ -87,7 +87,7 @@ __global__ void k_nk_init(int n, uint64_t seed, const unsigned long long *amax_b
 // at a time (coalesced, the row's lanes together) into shared memory and every
 // lane folds its own row from there.  (One row per warp, folded by one lane,
 // spent a warp's FP64 instruction, 20 clocks of an SM on this part, on each
-// entry: 286 us per sweep of a 46,760-row beam.)
+// entry: 286 us per sweep of a 46,760-row beam, 104 us so.)
 constexpr int kNkWarps = 4, kNkPitch = 33;
 __global__ void __launch_bounds__(32 * kNkWarps)
     k_nk_sweep(int n, const int64_t *ptr, const int32_t *col, const double *val, double omega,
@@ -107,7 +107,8 @@ __global__ void __launch_bounds__(32 * kNkWarps)
 #pragma unroll 8
     for (int r = 0; r < 32; ++r) {
       const int64_t k = __shfl_sync(0xffffffffu, s0, r) + c + lane;
-      if (k < __shfl_sync(0xffffffffu, e, r)) buf[r * kNkPitch + lane] = make_double2(val[k], x[col[k]]);
+      if (k < __shfl_sync(0xffffffffu, e, r))
+        buf[r * kNkPitch + lane] = make_double2(val[k], x[col[k]]);
     }
     __syncwarp();
     const int cnt = (int)min((int64_t)32, e - s0 - c);

@@ -3,12 +3,12 @@
 // the coarsest dense Cholesky, and the power method for lambda_max(D^-1 A).
 //
 // Scalars of the PCG recurrence (r.z, p.q, alpha, beta, |r|) stay on the
-// device: every dot product is a fixed-grid two-stage reduction whose last
-// block folds the per-block partials in a fixed order and applies the next
-// recurrence step, so results are deterministic run to run and no host round
-// trip is needed inside an iteration.  Kernels of an iteration return at once
-// when the device flag `done` is set, so the host launches iterations in
-// chunks and polls the flag between chunks.
+// device: a dot product leaves one partial per block, and every block of the
+// kernel that needs it (x/r update, p update) folds the partials in one fixed
+// order, so results are deterministic run to run and no host round trip is
+// needed inside an iteration.  Kernels of an iteration return at once when the
+// device flag `done` is set, so the host launches iterations in chunks and
+// reads the flag once per chunk.
 //
 // Precision: MGPBD_FP64 runs everything in FP64.  MGPBD_MIXED runs the
 // V-cycle bulk (smoothing, residuals, restriction, prolongation) with FP32
@@ -1689,7 +1689,8 @@ static mgpbd_status vcycle_level(Handle *h, int l, const T *b_in, T **res, bool 
     // the first sweep takes the prolongation with it
     if (l == 0) MG_TRY(prof_begin(h));
     DISPATCH_G(G, MG_TRY(rows_launch(h, "k_jacobi_prolong", k_jacobi_prolong<GG, T>, n, GG, n,
-                                     L.ptr, L.col, val, dinv, om, b_in, L.agg, Ps<T>(L), xc, x, x2, sc)));
+                                     L.ptr, L.col, val, dinv, om, b_in, L.agg, Ps<T>(L), xc, x,
+                                     x2, sc)));
     if (l == 0) MG_TRY(prof_end(h));
     std::swap(x, x2);
     s = 1;
