@@ -1193,8 +1193,19 @@ static mgpbd_status launch_tail(Handle *h, int first) {
   const CohortMember &M = mem[cb_.k];                                             \
   const int vb = cb_.vb, vn = cb_.vn
 
+// The same for the steps that can end an instance's solve (x/r update, p
+// update): the instance's block 0 raises `done` while other blocks of it may be
+// starting, and every block goes through barriers behind the test.  So a block
+// reads the flag once and leaves as a whole or not at all; one that is late and
+// leaves skips what the fold would have made it skip as well.
+#define COHORT_BLOCK_ENDING                                                       \
+  const CohortBlock cb_ = blk[blockIdx.x];                                        \
+  if (__syncthreads_or(threadIdx.x == 0 && is_done(cb_.sc))) return;              \
+  const CohortMember &M = mem[cb_.k];                                             \
+  const int vb = cb_.vb, vn = cb_.vn
+
 __global__ void kb_xr(const CohortMember *mem, const CohortBlock *blk) {
-  COHORT_BLOCK;
+  COHORT_BLOCK_ENDING;
   xr_update_body<float>(vb, vn, M.m, M.x, M.r, M.p, M.q, M.c_rr,
                         M.c_pq.partials, M.grid[CS_ROW_PQ], M.b0, M.dinv0, M.om0, M.x0, NoGate{});
 }
@@ -1213,7 +1224,7 @@ __global__ void kb_prolong0(const CohortMember *mem, const CohortBlock *blk) {
 }
 
 __global__ void kb_pupdate(const CohortMember *mem, const CohortBlock *blk) {
-  COHORT_BLOCK;
+  COHORT_BLOCK_ENDING;
   p_update_body(vb, vn, M.m, M.p, M.z, M.sc, M.c_rr.maxiter, M.c_rr.partials, M.grid[CS_XR],
                 M.c_rz.partials, M.grid[CS_ROW_FINAL], nullptr, NoGate{});
 }
