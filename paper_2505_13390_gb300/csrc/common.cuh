@@ -14,6 +14,7 @@
 #include <vector>
 
 #include "../../include/mgpbd.h"
+#include "launch_rules.h"
 
 namespace mg {
 

@@ -87,7 +87,8 @@ __global__ void k_nk_init(int n, uint64_t seed, const unsigned long long *amax_b
 // at a time (coalesced, the row's lanes together) into shared memory and every
 // lane folds its own row from there.  (One row per warp, folded by one lane,
 // spent a warp's FP64 instruction, 20 clocks of an SM on this part, on each
-// entry: 286 us per sweep of a 46,760-row beam, 104 us so.)
+// entry: 286 us per sweep of a 46,760-row beam, 104 us so.)  There is no loop
+// over the rows: the grid covers them (blocks_covering).
 constexpr int kNkWarps = 4, kNkPitch = 33;
 __global__ void __launch_bounds__(32 * kNkWarps)
     k_nk_sweep(int n, const int64_t *ptr, const int32_t *col, const double *val, double omega,
@@ -1382,7 +1383,7 @@ mgpbd_status amg_setup(Handle *h) {
                                                             amax, xa);
       MG_LAUNCH("k_nk_init");
       for (int s = 0; s < h->p.nk_sweeps; ++s) {
-        k_nk_sweep<<<blocks_for(h->m, 32 * kNkWarps), 32 * kNkWarps, kNkSmem, h->stream>>>(
+        k_nk_sweep<<<blocks_covering(h->m, 32 * kNkWarps), 32 * kNkWarps, kNkSmem, h->stream>>>(
             h->m, L0.ptr, L0.col, L0.val, h->p.nk_omega, xa, xb);
         MG_LAUNCH("k_nk_sweep");
         MG_CUDA(cudaMemcpyAsync(xa, xb, sizeof(double) * h->m, cudaMemcpyDeviceToDevice,

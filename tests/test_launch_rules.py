@@ -1,0 +1,77 @@
+"""The rules of launch shapes (csrc/launch_rules.h), compiled for the host."""
+import os
+import re
+import shutil
+import subprocess
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))),
+                    "paper_2505_13390_gb300", "csrc")
+
+
+def run_host(tmp_path, body):
+    """Output lines of a C++ program around `body` with the rules included."""
+    if not shutil.which("g++"):
+        pytest.skip("g++ not found")
+    src, exe = tmp_path / "t.cpp", tmp_path / "t"
+    src.write_text('#include <stdio.h>\n#include <initializer_list>\n#include "launch_rules.h"\n'
+                   "using namespace mg;\nint main() {\n" + body + "\n}\n")
+    subprocess.run(["g++", "-std=c++17", "-pthread", "-I", CSRC, str(src), "-o", str(exe)],
+                   check=True)
+    return subprocess.run([str(exe)], check=True, capture_output=True, text=True).stdout.split("\n")
+
+
+def launch(kernel, source):
+    """The launch configuration of `kernel` in a source file."""
+    return re.search(kernel + r"<<<(.*?)>>>", open(os.path.join(CSRC, source)).read(), re.S)[1]
+
+
+def test_near_kernel_sweep_covers_every_row(tmp_path):
+    """One warp takes 32 rows and does not loop: 2^20 blocks of 128 rows would
+    stop at row 134,217,728."""
+    assert launch("k_nk_sweep", "setup.cu").startswith("blocks_covering(h->m, 32 * kNkWarps)")
+    out = run_host(tmp_path, """
+  for (long long n : {1LL, 31LL, 128LL, 129LL, (1LL << 27), (1LL << 27) + 1, (1LL << 31) - 1})
+    printf("%lld %d\\n", n, blocks_covering(n, 128));""")
+    for n, b in (map(int, line.split()) for line in out if line):
+        assert 1 <= b < 2 ** 31 and 128 * (b - 1) < n <= 128 * b
+
+
+@pytest.mark.gpu
+def test_near_kernel_beyond_two_to_the_27_rows():
+    """A chain of 2^27 + 3,000 rows whose rows are dead (both ends pinned) but
+    for the last 2,500: one sweep x - omega D^-1 A x on those, from the start
+    that a setup without sweeps leaves."""
+    import numpy as np
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available() or torch.cuda.mem_get_info()[0] < 80 << 30:
+        pytest.skip("needs a CUDA device with 80 GB free")
+    from paper_2505_13390_gb300.meshgen import Mesh, default_params
+    from paper_2505_13390_gb300.mgpbd import Solver
+    rows, live = (1 << 27) + 3000, 2500
+    x = np.zeros((rows + 1, 3))
+    x[:, 0] = 0.01 * np.arange(rows + 1)
+    w = np.zeros(rows + 1)
+    w[-live:] = 1.0
+    e = np.empty((rows, 2), np.int32)
+    e[:, 0] = np.arange(rows)
+    e[:, 1] = e[:, 0] + 1
+    mesh = Mesh("long", x, w, e, np.zeros((0, 4), np.int32), np.full(rows, 1e-6), x, np.zeros_like(x))
+    vec = {}
+    for sweeps in (0, 1):
+        g = Solver(mesh, default_params(nk_sweeps=sweeps, nk_omega=0.5, coarse_max=2000, max_levels=3))
+        g.begin_frame()
+        g.eval_assemble()
+        g.setup()
+        if not sweeps:
+            ptr, col, val = (a[-n:].cpu().numpy() for a, n in zip(g.matrix(0, device=True), (2901, 10000, 10000)))
+        vec[sweeps] = g.level_agg(0)[4]
+        g.close()
+        torch.cuda.empty_cache()
+    first, shift = rows - 2900, ptr[-1] - 10000
+    for i in range(first, rows):
+        a, b = ptr[i - first] - shift, ptr[i - first + 1] - shift
+        want = vec[0][i] - 0.5 * (val[a:b] @ vec[0][col[a:b]]) / val[b - 1]
+        # three products per row, each below 2 max |x| (|A_ij| <= 2 A_ii here)
+        assert abs(vec[1][i] - want) <= 1e-14 * np.abs(vec[0][first:]).max(), i
