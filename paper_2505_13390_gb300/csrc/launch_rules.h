@@ -4,6 +4,9 @@
 
 #include <stdint.h>
 
+#include <mutex>
+#include <set>
+
 namespace mg {
 
 // Blocks of a kernel without a loop over its rows: every row has its place,
@@ -13,5 +16,23 @@ inline int blocks_covering(int64_t rows, int rows_per_block) {
   const int64_t b = (rows + rows_per_block - 1) / rows_per_block;
   return (int)(b < 1 ? 1 : b);
 }
+
+// A setting that the runtime keeps per device (a kernel's shared-memory limit,
+// for one) and that is made once: `f` runs for each device until it has
+// succeeded there (a status >= 0), one thread at a time.
+class OncePerDevice {
+  std::mutex mu;
+  std::set<int> made;
+
+ public:
+  template <class F>
+  int operator()(int device, F f) {
+    std::lock_guard<std::mutex> lock(mu);
+    if (made.count(device)) return 0;
+    const int status = f();
+    if (status >= 0) made.insert(device);
+    return status;
+  }
+};
 
 }  // namespace mg

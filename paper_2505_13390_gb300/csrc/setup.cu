@@ -27,7 +27,6 @@
 // operation order as a plain sequential FP64 program, so aggregates, P, B and
 // colours are reproducible bit for bit.
 #include <algorithm>
-#include <mutex>
 
 #include "common.cuh"
 
@@ -818,10 +817,10 @@ mgpbd_status level_precision_copies(Handle *h, int l) {
 }
 
 // The largest dynamic shared memory a Galerkin launch requests.  The limit a
-// kernel may request is one setting per kernel for the whole process, so it is
-// raised once to this bound (under a mutex, before the first launch), never
-// per launch: per launch, one thread could lower it between another thread's
-// setting and that thread's launch, which then fails.
+// kernel may request is one setting per kernel and device for the whole process,
+// so it is raised once on each device to this bound (under a mutex, before the
+// first launch there), never per launch: per launch, one thread could lower it
+// between another thread's setting and that thread's launch, which then fails.
 constexpr int kGalerkinSmemMax = 200 * 1024;
 constexpr int kNkSmem = kNkWarps * 32 * kNkPitch * (int)sizeof(double2);
 
@@ -832,17 +831,16 @@ __global__ void k_gal_values_k(int na, int k, const int64_t *mptr, const int32_t
                                int maxblk, double *acc_global);
 
 static mgpbd_status galerkin_smem_limits() {
-  static std::mutex mu;
-  static bool done = false;
-  std::lock_guard<std::mutex> lock(mu);
-  if (done) return MGPBD_OK;
-  MG_CUDA(cudaFuncSetAttribute(k_gal_values, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               kGalerkinSmemMax));
-  MG_CUDA(cudaFuncSetAttribute(k_nk_sweep, cudaFuncAttributeMaxDynamicSharedMemorySize, kNkSmem));
-  MG_CUDA(cudaFuncSetAttribute(k_gal_values_k, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               kGalerkinSmemMax));
-  done = true;
-  return MGPBD_OK;
+  static OncePerDevice once;
+  int device = 0;
+  MG_CUDA(cudaGetDevice(&device));
+  return once(device, []() -> mgpbd_status {
+    const cudaFuncAttribute limit = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    MG_CUDA(cudaFuncSetAttribute(k_gal_values, limit, kGalerkinSmemMax));
+    MG_CUDA(cudaFuncSetAttribute(k_nk_sweep, limit, kNkSmem));
+    MG_CUDA(cudaFuncSetAttribute(k_gal_values_k, limit, kGalerkinSmemMax));
+    return MGPBD_OK;
+  });
 }
 
 static mgpbd_status galerkin_values(Handle *h, int l) {

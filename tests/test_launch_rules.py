@@ -15,7 +15,7 @@ def run_host(tmp_path, body):
     if not shutil.which("g++"):
         pytest.skip("g++ not found")
     src, exe = tmp_path / "t.cpp", tmp_path / "t"
-    src.write_text('#include <stdio.h>\n#include <initializer_list>\n#include "launch_rules.h"\n'
+    src.write_text('#include <stdio.h>\n#include <initializer_list>\n#include <thread>\n#include <vector>\n#include "launch_rules.h"\n'
                    "using namespace mg;\nint main() {\n" + body + "\n}\n")
     subprocess.run(["g++", "-std=c++17", "-pthread", "-I", CSRC, str(src), "-o", str(exe)],
                    check=True)
@@ -36,6 +36,27 @@ def test_near_kernel_sweep_covers_every_row(tmp_path):
     printf("%lld %d\\n", n, blocks_covering(n, 128));""")
     for n, b in (map(int, line.split()) for line in out if line):
         assert 1 <= b < 2 ** 31 and 128 * (b - 1) < n <= 128 * b
+
+
+def test_settings_are_made_on_each_device(tmp_path):
+    """A kernel's shared-memory limit belongs to the device it was set on: every
+    device has it made once, again after a failure, and once under threads."""
+    body = open(os.path.join(CSRC, "setup.cu")).read()
+    body = body[body.index("mgpbd_status galerkin_smem_limits()"):]
+    assert "OncePerDevice" in body[:body.index("\n}\n")]
+    out = run_host(tmp_path, """
+  OncePerDevice once;
+  int made[3] = {0, 0, 0}, bad = 0;
+  auto use = [&](int d) { return once(d, [&] { made[d]++; return 0; }); };
+  bool ok = use(0) == 0 && use(1) == 0 && use(0) == 0;
+  ok = ok && once(2, [&] { bad++; return -6; }) == -6 && use(2) == 0 && use(2) == 0;
+  OncePerDevice shared;
+  int n = 0;
+  std::vector<std::thread> ts;
+  for (int k = 0; k < 8; ++k) ts.emplace_back([&] { shared(k % 2, [&] { n++; return 0; }); });
+  for (auto &t : ts) t.join();
+  printf("%d %d %d %d %d %d\\n", ok, made[0], made[1], made[2], bad, n);""")
+    assert out[0] == "1 1 1 1 1 2"
 
 
 @pytest.mark.gpu
