@@ -246,9 +246,11 @@ __device__ __forceinline__ AT row_fin(const RowPre<VT> &p, const int32_t *col, c
 // The gate between the loads a kernel may make early and the rest: `open`
 // waits for the chain's predecessor on its first call and reads the solve's
 // done flag beside the loads that follow it; `closed` tells whether the solve
-// has finished (checked before anything is written).  Outside a chain (the
-// cooperative tail, whose blocks have checked already) NoGate does nothing.
+// has finished (checked before anything is written).  Behind a check that has
+// been made already (the plain form of a kernel, the cooperative tail) NoGate
+// does nothing, and the bodies that differ take their lean form (kEarly).
 struct ChainGate {
+  static constexpr bool kEarly = true;
   const PcgScalars *sc;
   int state = -1;
   __device__ __forceinline__ explicit ChainGate(const PcgScalars *s) : sc(s) {}
@@ -261,9 +263,23 @@ struct ChainGate {
   __device__ __forceinline__ bool closed() const { return state != 0; }
 };
 struct NoGate {
+  static constexpr bool kEarly = false;
   __device__ __forceinline__ void open() {}
   __device__ __forceinline__ bool closed() const { return false; }
 };
+
+// Runs body(gate) in a kernel's early form, or in its plain form behind the
+// wait and the flag.
+template <bool EARLY, class F>
+__device__ __forceinline__ void behind_gate(const PcgScalars *sc, F body) {
+  if constexpr (EARLY) {
+    body(ChainGate(sc));
+  } else {
+    chain_wait();
+    if (sc && is_done(sc)) return;
+    body(NoGate{});
+  }
+}
 
 // Rows handled by G-lane groups, 32/G rows per warp per trip, over warps
 // w0, w0 + nw, ...  The loop bound is uniform across the warp, so full-mask

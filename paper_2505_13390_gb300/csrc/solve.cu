@@ -321,27 +321,35 @@ __global__ void k_convert(int64_t n, const S *a, D *b, const PcgScalars *sc) {
 // sparse kernels: G lanes per row (G in 4, 8, 16, 32)
 // ---------------------------------------------------------------------------
 // q = A p (PCG operator) fused with p.q
-template <int G, class VT, class AT>
+template <int G, class VT, class AT, bool EARLY>
 __global__ void k_spmv_pq(int n, const int64_t *ptr, const int32_t *col, const VT *val,
                           const double *p, double *q, DotCtx c) {
-  ChainGate gate(c.sc);
-  double acc = 0.0;
-  GROUP_ROWS(G, n) {
-    const RowPre<VT> pre = row_pre<G>(ptr, col, val, i, g, valid);
-    gate.open();
-    const double pi = valid && g == 0 ? p[i] : 0.0;
-    AT s = row_fin<G, AT>(pre, col, val, p);
-    s = group_sum<G>(s);
-    if (gate.closed()) break;
-    if (valid && g == 0) {
-      double qi = (double)s;
-      q[i] = qi;
-      acc = fma(pi, qi, acc);
+  behind_gate<EARLY>(c.sc, [&](auto gate) {
+    double acc = 0.0;
+    GROUP_ROWS(G, n) {
+      AT s;
+      double pi = 0.0;
+      if constexpr (EARLY) {
+        const RowPre<VT> pre = row_pre<G>(ptr, col, val, i, g, valid);
+        gate.open();
+        if (valid && g == 0) pi = p[i];
+        s = row_fin<G, AT>(pre, col, val, p);
+      } else {
+        s = valid ? row_dot<G, VT, AT, double>(ptr, col, val, p, (int)i, g) : (AT)0;
+      }
+      s = group_sum<G>(s);
+      if (gate.closed()) break;
+      if (valid && g == 0) {
+        if constexpr (!EARLY) pi = p[i];
+        double qi = (double)s;
+        q[i] = qi;
+        acc = fma(pi, qi, acc);
+      }
     }
-  }
-  gate.open();  // warps without a row
-  if (gate.closed()) return;
-  block_dot_finish(acc, c);
+    gate.open();  // warps without a row
+    if (gate.closed()) return;
+    block_dot_finish(acc, c);
+  });
 }
 
 // r_t = b - A x in FP64, |r_t|^2
@@ -436,15 +444,21 @@ __device__ __forceinline__ void jacobi_rows(int64_t w0, int64_t nw, int n, const
                                             const int32_t *col, const T *val, const T *dinv,
                                             T omega, const T *b, const T *x, T *xn, Gate gate) {
   GROUP_ROWS_OVER(G, n, w0, nw) {
-    const RowPre<T> p = row_pre<G>(ptr, col, val, i, g, valid);
     const bool head = valid && g == 0;
-    const T di = head ? dinv[i] : (T)0;
-    gate.open();
-    const T bi = head ? b[i] : (T)0, xi = head ? x[i] : (T)0;
-    T s = row_fin<G, T>(p, col, val, x);
-    s = group_sum<G>(s);
-    if (gate.closed()) return;
-    if (head) xn[i] = fma(omega, (bi - s) * di, xi);
+    if constexpr (Gate::kEarly) {
+      const RowPre<T> p = row_pre<G>(ptr, col, val, i, g, valid);
+      const T di = head ? dinv[i] : (T)0;
+      gate.open();
+      const T bi = head ? b[i] : (T)0, xi = head ? x[i] : (T)0;
+      T s = row_fin<G, T>(p, col, val, x);
+      s = group_sum<G>(s);
+      if (gate.closed()) return;
+      if (head) xn[i] = fma(omega, (bi - s) * di, xi);
+    } else {
+      T s = valid ? row_dot<G, T, T, T>(ptr, col, val, x, (int)i, g) : (T)0;
+      s = group_sum<G>(s);
+      if (head) xn[i] = fma(omega, (b[i] - s) * dinv[i], x[i]);
+    }
   }
 }
 
@@ -454,33 +468,43 @@ __device__ __forceinline__ void resid_rows(int64_t w0, int64_t nw, int n, const 
                                            const int32_t *col, const T *val, const T *b,
                                            const T *x, T *r, Gate gate) {
   GROUP_ROWS_OVER(G, n, w0, nw) {
-    const RowPre<T> p = row_pre<G>(ptr, col, val, i, g, valid);
-    gate.open();
-    const T bi = valid && g == 0 ? b[i] : (T)0;
-    T s = row_fin<G, T>(p, col, val, x);
-    s = group_sum<G>(s);
-    if (gate.closed()) return;
-    if (valid && g == 0) r[i] = bi - s;
+    if constexpr (Gate::kEarly) {
+      const RowPre<T> p = row_pre<G>(ptr, col, val, i, g, valid);
+      gate.open();
+      const T bi = valid && g == 0 ? b[i] : (T)0;
+      T s = row_fin<G, T>(p, col, val, x);
+      s = group_sum<G>(s);
+      if (gate.closed()) return;
+      if (valid && g == 0) r[i] = bi - s;
+    } else {
+      T s = valid ? row_dot<G, T, T, T>(ptr, col, val, x, (int)i, g) : (T)0;
+      s = group_sum<G>(s);
+      if (valid && g == 0) r[i] = b[i] - s;
+    }
   }
 }
 
-template <int G, class T>
+template <int G, class T, bool EARLY>
 __global__ void k_jacobi(int n, const int64_t *ptr, const int32_t *col, const T *val,
                          const T *dinv, T omega, const T *b, const T *x, T *xn,
                          const PcgScalars *sc) {
-  jacobi_rows<G, T>(HW_WARPS, n, ptr, col, val, dinv, omega, b, x, xn, ChainGate(sc));
+  behind_gate<EARLY>(sc, [&](auto gate) {
+    jacobi_rows<G, T>(HW_WARPS, n, ptr, col, val, dinv, omega, b, x, xn, gate);
+  });
 }
 
-template <int G, class T>
+template <int G, class T, bool EARLY>
 __global__ void k_resid(int n, const int64_t *ptr, const int32_t *col, const T *val, const T *b,
                         const T *x, T *r, const PcgScalars *sc) {
-  resid_rows<G, T>(HW_WARPS, n, ptr, col, val, b, x, r, ChainGate(sc));
+  behind_gate<EARLY>(sc, [&](auto gate) {
+    resid_rows<G, T>(HW_WARPS, n, ptr, col, val, b, x, r, gate);
+  });
 }
 
 // The first post-smoothing sweep with the prolongation taken along: every x_j
 // it reads is x_j + P_j x_c[agg_j], the value k_prolong would have stored (one
 // launch less per level; on large levels the two gathers more per entry cost
-// more than the launch, see kFuseProlongRows)
+// more than the launch, see fuse_prolong)
 template <int G, class T>
 __global__ void k_jacobi_prolong(int n, const int64_t *ptr, const int32_t *col, const T *val,
                                  const T *dinv, T omega, const T *b, const int32_t *agg,
@@ -525,38 +549,44 @@ __global__ void k_jacobi_prolong(int n, const int64_t *ptr, const int32_t *col, 
     if (head) xn[i] = fma(omega, (bi - s) * di, xi);
   }
 }
-// up to this many rows: a frame of the 32x32 cloth in FP64 takes 72.8 ms with
-// the fused sweep and 74.5 without; on 1.3M rows of cloth (coarse levels above
-// the line) the two differ by nothing
-constexpr int kFuseProlongRows = 1 << 16;
-
 // The last post-smoothing sweep of level 0: z = the new iterate in FP64, with
 // r.z when `dot` is set
-template <int G, class T>
+template <int G, class T, bool EARLY>
 __global__ void k_jacobi_final(int n, const int64_t *ptr, const int32_t *col, const T *val,
                                const T *dinv, T omega, const T *b, const T *x, double *z,
                                const double *r, bool dot, DotCtx c) {
-  ChainGate gate(c.sc);
-  double acc = 0.0;
-  GROUP_ROWS(G, n) {
-    const RowPre<T> p = row_pre<G>(ptr, col, val, i, g, valid);
-    const bool head = valid && g == 0;
-    const T di = head ? dinv[i] : (T)0;
-    gate.open();
-    const T bi = head ? b[i] : (T)0, xi = head ? x[i] : (T)0;
-    const double ri = head && dot ? r[i] : 0.0;
-    T s = row_fin<G, T>(p, col, val, x);
-    s = group_sum<G>(s);
-    if (gate.closed()) break;
-    if (head) {
-      const double zi = widen(fma(omega, (bi - s) * di, xi));
-      z[i] = zi;
-      acc = fma(ri, zi, acc);
+  behind_gate<EARLY>(c.sc, [&](auto gate) {
+    double acc = 0.0;
+    GROUP_ROWS(G, n) {
+      const bool head = valid && g == 0;
+      T s, di = 0, bi = 0, xi = 0;
+      double ri = 0.0;
+      if constexpr (EARLY) {
+        const RowPre<T> p = row_pre<G>(ptr, col, val, i, g, valid);
+        if (head) di = dinv[i];
+        gate.open();
+        if (head) bi = b[i], xi = x[i];
+        if (head && dot) ri = r[i];
+        s = row_fin<G, T>(p, col, val, x);
+      } else {
+        s = valid ? row_dot<G, T, T, T>(ptr, col, val, x, (int)i, g) : (T)0;
+      }
+      s = group_sum<G>(s);
+      if (gate.closed()) break;
+      if (head) {
+        if constexpr (!EARLY) {
+          di = dinv[i], bi = b[i], xi = x[i];
+          if (dot) ri = r[i];
+        }
+        const double zi = widen(fma(omega, (bi - s) * di, xi));
+        z[i] = zi;
+        acc = fma(ri, zi, acc);
+      }
     }
-  }
-  gate.open();  // warps without a row
-  if (gate.closed()) return;
-  if (dot) block_dot_finish(acc, c);
+    gate.open();  // warps without a row
+    if (gate.closed()) return;
+    if (dot) block_dot_finish(acc, c);
+  });
 }
 
 // b_c[a*k+c] = sum_{i in a} P_ic r_i (warp per aggregate, k columns of P per
@@ -976,16 +1006,55 @@ static int row_blocks(int64_t rows, int G, int th = 256) {
   return (int)std::max<int64_t>(1, std::min<int64_t>(b, cap));
 }
 
+// CSR row kernels over matrices of up to this many entries run in their early
+// form (matrix entries loaded before the wait): it needs 48 to 70 registers a
+// thread against 32 to 40, so a matrix that fills the GPU for longer than the
+// loads' latency is better off with the plain form's occupancy.  Both forms of
+// whole solves (FP64) and V-cycles (FP32), early against plain: FP64 6.94 / 7.27
+// ms at 2.9M entries (beam), 9.99 / 10.14 at 3.6M (cloth), 10.63 / 10.52 at 4.4M
+// (beam), 13.90 / 13.51 at 5.3M (cloth), 70.8 / 56.6 at 60M (block); FP32 199 /
+// 206 us at 8.9M (beam), 299 / 306 at 10.3M (cloth), 272 / 261 at 14.3M (block),
+// 415 / 410 at 16.1M (cloth), 775 / 703 at 60M (block).
+constexpr int64_t kEarlyNnz64 = 1 << 22, kEarlyNnz32 = 3 << 22;
+template <class T>
+static bool early_rows(const Level &L) {
+  return L.nnz <= (sizeof(T) == 8 ? kEarlyNnz64 : kEarlyNnz32);
+}
+
+// Whether a level's first post-sweep takes the prolongation along
+// (k_jacobi_prolong).  With rows of up to 16 entries all of a row's aggregates
+// and weights are loaded before the gate; the rest of a longer row is a serial
+// loop with two more gathers per entry, which only FP32's wider groups keep
+// short.  Whole solves, fused against not: FP64 2.09 / 2.12 ms at 132K entries,
+// 3.65 / 3.56 at 543K (cloths), 5.15 / 4.99 with the fusion on a beam's levels of
+// up to 64K; FP32 2.82 / 2.87 at 543K, 5.10 / 5.03 at 2.1M (cloths), 3.20 / 3.26 on
+// a beam's levels of up to 192K and 3.22 with those of up to 768K.
+template <class T>
+static bool fuse_prolong(const Level &L) {
+  const bool short_rows = L.nnz <= 16 * (int64_t)L.n;
+  if (sizeof(T) == 8) return short_rows && L.nnz <= 1 << 18;
+  return L.nnz <= (short_rows ? 3 << 18 : 3 << 16);
+}
+
+#define DISPATCH_EARLY(early, ...)                 \
+  if (early) {                                     \
+    constexpr bool EE = true;                      \
+    __VA_ARGS__;                                   \
+  } else {                                         \
+    constexpr bool EE = false;                     \
+    __VA_ARGS__;                                   \
+  }
+
 // grids of the kernels that end in a dot product: one resident wave at most
-template <int G>
+template <int G, bool EARLY>
 static int spmv_pq_blocks(int m) {
   return std::min(row_blocks(m, G, kDotThreads),
-                  wave_blocks((const void *)k_spmv_pq<G, double, double>, kDotThreads));
+                  wave_blocks((const void *)k_spmv_pq<G, double, double, EARLY>, kDotThreads));
 }
-template <int G, class T>
+template <int G, class T, bool EARLY>
 static int jacobi_final_blocks(int n) {
   return std::min(row_blocks(n, G, kDotThreads),
-                  wave_blocks((const void *)k_jacobi_final<G, T>, kDotThreads));
+                  wave_blocks((const void *)k_jacobi_final<G, T, EARLY>, kDotThreads));
 }
 // p update: four entries per thread, at most sixteen blocks per SM (every block
 // folds r.z's partials)
@@ -1582,6 +1651,14 @@ static mgpbd_status rows_launch(Handle *h, const char *what, void (*k)(P...), in
   return chain_launch(h, what, k, row_blocks(rows, G, th), th, args...);
 }
 
+static mgpbd_status launch_dot(Handle *h, const double *x, const double *y, int64_t n, int mode,
+                               int check_done, double *out = nullptr) {
+  const DotCtx c = mode == DOT_PART ? rz_ctx(h) : make_ctx(h, mode, out);
+  const int blocks = std::min(dot_grid(n), wave_blocks((const void *)k_dot, kDotThreads));
+  if (mode == DOT_PART) h->n_rz = blocks;
+  return chain_launch(h, "k_dot", k_dot, blocks, kDotThreads, n, x, y, c, check_done);
+}
+
 // V-cycle on level l in precision T from its right-hand side (zero start);
 // *res is the vector of the level that holds the result.  On level 0 of a top
 // V-cycle, `x0_ready` says the first Jacobi sweep is already in L.x, and `top`
@@ -1653,8 +1730,9 @@ static mgpbd_status vcycle_level(Handle *h, int l, const T *b_in, T **res, bool 
     if (mf) {
       MG_TRY(mf_level0<T>(h, kMfSweep, x, b_in, dinv, om, x2));
     } else {
-      DISPATCH_G(G, MG_TRY(rows_launch(h, "k_jacobi", k_jacobi<GG, T>, n, GG, n, L.ptr, L.col, val,
-                                       dinv, om, b_in, x, x2, sc)));
+      DISPATCH_G(G, DISPATCH_EARLY(early_rows<T>(L), MG_TRY(rows_launch(
+                        h, "k_jacobi", k_jacobi<GG, T, EE>, n, GG, n, L.ptr, L.col, val, dinv, om,
+                        b_in, x, x2, sc))));
     }
     if (l == 0) MG_TRY(prof_end(h));
     std::swap(x, x2);
@@ -1686,8 +1764,9 @@ static mgpbd_status vcycle_level(Handle *h, int l, const T *b_in, T **res, bool 
     if (mf)
       MG_TRY(mf_level0<T>(h, kMfResid, x, b_in, dinv, om, r));
     else
-      DISPATCH_G(G, MG_TRY(rows_launch(h, "k_resid", k_resid<GG, T>, n, GG, n, L.ptr, L.col, val,
-                                       b_in, x, r, sc)));
+      DISPATCH_G(G, DISPATCH_EARLY(early_rows<T>(L), MG_TRY(rows_launch(
+                        h, "k_resid", k_resid<GG, T, EE>, n, GG, n, L.ptr, L.col, val, b_in, x, r,
+                        sc))));
     MG_TRY(item_launch(h, "k_restrict", k_restrict<T>, 32ll * L.n_agg, L.n_agg, nk, L.mptr, L.mrow,
                        Ps<T>(L), r, (T *)Lc.b, sc, dinv_c, (T)Lc.omega, x_c));
   }
@@ -1699,7 +1778,7 @@ static mgpbd_status vcycle_level(Handle *h, int l, const T *b_in, T **res, bool 
     MG_TRY(vcycle_level<T>(h, l + 1, (const T *)Lc.b, &xc, c_jac));
   }
   int s = 0;  // post-smoothing sweeps done
-  if (jac && nk == 1 && !mf && n <= kFuseProlongRows && (sweeps > 1 || !top)) {
+  if (jac && nk == 1 && !mf && fuse_prolong<T>(L) && (sweeps > 1 || !top)) {
     // the first sweep takes the prolongation with it
     if (l == 0) MG_TRY(prof_begin(h));
     DISPATCH_G(G, MG_TRY(rows_launch(h, "k_jacobi_prolong", k_jacobi_prolong<GG, T>, n, GG, n,
@@ -1728,23 +1807,27 @@ static mgpbd_status vcycle_level(Handle *h, int l, const T *b_in, T **res, bool 
       break;
     }
     MG_TRY(prof_begin(h));
-    DISPATCH_G(G, const int blocks = jacobi_final_blocks<GG, T>(n); if (top->dot) h->n_rz = blocks;
-               MG_TRY(chain_launch(h, "k_jacobi_final", k_jacobi_final<GG, T>, blocks, kDotThreads,
-                                   n, L.ptr, L.col, val, dinv, om, b_in, x, top->z, top->r,
-                                   top->dot, top->c)));
+    DISPATCH_G(G, DISPATCH_EARLY(early_rows<T>(L), {
+      if constexpr (sizeof(T) == 8 && !EE) {
+        // z is the sweep's own output here; with the dot product in it the
+        // sweep of long rows lacks registers (113.9 against 110.1 ms for 48
+        // iterations on 1.3M rows of the block, r.z in a launch of its own)
+        MG_TRY(rows_launch(h, "k_jacobi", k_jacobi<GG, T, EE>, n, GG, n, L.ptr, L.col, val, dinv,
+                           om, b_in, x, (T *)top->z, sc));
+        if (top->dot) MG_TRY(launch_dot(h, top->r, top->z, n, top->c.mode, 1));
+      } else {
+        const int blocks = jacobi_final_blocks<GG, T, EE>(n);
+        if (top->dot) h->n_rz = blocks;
+        MG_TRY(chain_launch(h, "k_jacobi_final", k_jacobi_final<GG, T, EE>, blocks, kDotThreads,
+                            n, L.ptr, L.col, val, dinv, om, b_in, x, top->z, top->r, top->dot,
+                            top->c));
+      }
+    }));
     MG_TRY(prof_end(h));
   }
   if (z_written) *z_written = zw;
   *res = x;
   return MGPBD_OK;
-}
-
-static mgpbd_status launch_dot(Handle *h, const double *x, const double *y, int64_t n, int mode,
-                               int check_done, double *out = nullptr) {
-  const DotCtx c = mode == DOT_PART ? rz_ctx(h) : make_ctx(h, mode, out);
-  const int blocks = std::min(dot_grid(n), wave_blocks((const void *)k_dot, kDotThreads));
-  if (mode == DOT_PART) h->n_rz = blocks;
-  return chain_launch(h, "k_dot", k_dot, blocks, kDotThreads, n, x, y, c, check_done);
 }
 
 // level 0 starts its V-cycle with a Jacobi sweep from zero (not the coarsest)
@@ -1809,9 +1892,9 @@ mgpbd_status apply_level0(Handle *h, int form, const double *x, double *y) {
   DotCtx c = make_ctx(h, DOT_STORE, &h->sc->tr2);  // x.Ax lands in a scratch scalar
   if (form == 0) {
     const int G = group_for(h, L, true);
-    DISPATCH_G(G, MG_TRY(chain_launch(h, "k_spmv_pq", k_spmv_pq<GG, double, double>,
-                                      spmv_pq_blocks<GG>(m), kDotThreads, m, L.ptr, L.col, L.val,
-                                      x, y, c)));
+    DISPATCH_G(G, DISPATCH_EARLY(early_rows<double>(L), MG_TRY(chain_launch(
+                      h, "k_spmv_pq", k_spmv_pq<GG, double, double, EE>, spmv_pq_blocks<GG, EE>(m),
+                      kDotThreads, m, L.ptr, L.col, L.val, x, y, c))));
     return MGPBD_OK;
   }
   if (form == 2) MG_TRY(mf_split(h, x, h->p_df, m));
@@ -1839,9 +1922,10 @@ static mgpbd_status pcg_iteration(Handle *h, double *x) {
   if (h->p.level0_op == 1) {
     MG_TRY(mf_apply_pq(h, p, q, cpq));
   } else {
-    DISPATCH_G(G, MG_TRY(chain_launch(h, "k_spmv_pq", k_spmv_pq<GG, double, double>,
-                                      h->n_pq = spmv_pq_blocks<GG>(m), kDotThreads, m, L.ptr,
-                                      L.col, L.val, p, q, cpq)));
+    DISPATCH_G(G, DISPATCH_EARLY(early_rows<double>(L), MG_TRY(chain_launch(
+                      h, "k_spmv_pq", k_spmv_pq<GG, double, double, EE>,
+                      h->n_pq = spmv_pq_blocks<GG, EE>(m), kDotThreads, m, L.ptr, L.col, L.val, p,
+                      q, cpq))));
   }
   MG_TRY(prof_end(h, PROF_AP));
   // the update also starts the V-cycle (right-hand side, first Jacobi sweep)
@@ -2042,8 +2126,8 @@ static mgpbd_status time_resid(Handle *h, const Level &L, int G, const T *val, c
   for (int rep = 0; rep < 5; ++rep) {
     MG_TRY(evict_l2(h));
     MG_CUDA(cudaEventRecord(h->ev0, h->stream));
-    DISPATCH_G(G, (k_resid<GG, T><<<row_blocks(n, GG), 256, 0, h->stream>>>(n, L.ptr, L.col, val,
-                                                                           b, x, r, nullptr)));
+    DISPATCH_G(G, DISPATCH_EARLY(early_rows<T>(L), k_resid<GG, T, EE><<<row_blocks(n, GG), 256, 0, h->stream>>>(
+                                            n, L.ptr, L.col, val, b, x, r, nullptr)));
     MG_LAUNCH("k_resid(tune)");
     MG_CUDA(cudaEventRecord(h->ev1, h->stream));
     MG_CUDA(cudaEventSynchronize(h->ev1));

@@ -1,0 +1,124 @@
+"""The kernel forms a solve picks by size, against plain FP64 references.
+
+The products and V-cycles on both sides of every size rule are compared with
+the same formulas in torch, in FP64, from the instance's matrices, aggregates,
+prolongators and weights (which the setup tests pin to the oracle bit for bit).
+The meshes are soft (alpha 1e-4), so that the V-cycle is well conditioned: its
+FP64 sums in another order stay within 1e-9 of each other and its FP32 bulk
+within 1e-4, as for the V-cycle tests against the oracle.  A product's row is a
+sum of at most a few hundred terms: 1e-13 of the sum of their magnitudes.
+"""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+from paper_2505_13390_gb300.meshgen import Mesh, cloth, default_params, hex_block  # noqa: E402
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _gpu():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    torch.cuda.set_device(0)
+
+
+def cut_cloth(rows):
+    """A soft cloth with exactly `rows` distance rows."""
+    m = cloth(int((rows / 3) ** 0.5) + 3, alpha=1e-4, noise=1e-3, seed=3)
+    return Mesh("cut", m.rest_pos, m.inv_mass, m.dist[:rows], m.tet, m.alpha[:rows], m.x0, m.v0)
+
+
+def cut_block(rows, ny, nz):
+    """A soft block, pinned at one end, with exactly `rows` rows: all of its
+    edges and as many of its tets."""
+    n = 1
+    while len((m := hex_block(n, ny, nz, h=0.01, jitter=0.1, alpha=1e-4, pin="x0", seed=2)).alpha) < rows:
+        n = max(n + 1, int(n * rows / len(m.alpha)))
+    tets = rows - len(m.dist)
+    assert 0 < tets
+    return Mesh("cut", m.rest_pos, m.inv_mass, m.dist, m.tet[:tets], m.alpha[:rows], m.x0, m.v0)
+
+
+def ready(mesh, **over):
+    from paper_2505_13390_gb300.mgpbd import Solver
+    g = Solver(mesh, default_params(**over))
+    g.begin_frame()
+    g.eval_assemble()
+    g.prepare_solve()
+    torch.cuda.synchronize()
+    return g
+
+
+def matrices(g):
+    out = []
+    for level in range(g.levels):
+        ptr, col, val = g.matrix(level, device=True)
+        n = len(ptr) - 1
+        out.append((torch.sparse_csr_tensor(ptr, col.long(), val, (n, n)), val[ptr[1:] - 1]))
+    return out
+
+
+def vcycle(g, mats, level, b):
+    a, diag = mats[level]
+    if level == len(mats) - 1:
+        return torch.linalg.solve(a.to_dense(), b)
+    _, agg, _, weight, _ = g.level_agg(level)
+    agg, weight = torch.from_numpy(agg).long().cuda(), torch.from_numpy(weight).cuda()
+    omega, take, keep = g.level_omega(level)[1], agg.clamp(min=0), agg >= 0
+    x = torch.zeros_like(b)
+    for _ in range(2):
+        x = x + omega * (b - a @ x) / diag
+    r = torch.where(keep, weight * (b - a @ x), 0.0)
+    bc = torch.zeros(len(mats[level + 1][1]), dtype=torch.float64, device="cuda")
+    bc.index_add_(0, take, r)
+    x = x + torch.where(keep, weight * vcycle(g, mats, level + 1, bc)[take], 0.0)
+    for _ in range(2):
+        x = x + omega * (b - a @ x) / diag
+    return x
+
+
+def rel(a, b):
+    return float((a - b).norm() / b.norm())
+
+
+def check_forms(mesh, op, prec):
+    with torch.cuda.stream(torch.cuda.Stream()):  # graphs need a stream of their own
+        _check_forms(mesh, op, prec)
+
+
+def _check_forms(mesh, op, prec):
+    g = ready(mesh, level0_op=op, precision=prec, pcg_rtol=1e-14, pcg_maxiter=9)
+    mats = matrices(g)
+    gen = torch.Generator(device="cuda").manual_seed(4)
+    r = torch.randn(g.m, dtype=torch.float64, device="cuda", generator=gen)
+    a = mats[0][0]
+    size = torch.sparse_csr_tensor(a.crow_indices(), a.col_indices(), a.values().abs(), a.shape) @ r.abs()
+    if op:  # the matrix-free terms: at most |A| with its diagonal's magnitudes
+        size = size + mats[0][1] * r.abs()
+    y = g.apply(r, op)
+    assert float(((y - a @ r).abs() / size).max()) <= 1e-13
+    assert rel(g.vcycle(r), vcycle(g, mats, 0, r)) <= (1e-4 if prec else 1e-9)
+    # nine iterations, one chunk of eight replayed from a graph, bit for bit
+    # the plain launches
+    x, info = g.solve(r)
+    assert info["pcg_iters"] == 9
+    g.close()
+    g = ready(mesh, level0_op=op, precision=prec, pcg_rtol=1e-14, pcg_maxiter=9, use_graphs=1)
+    x2, info2 = g.solve(r)
+    assert torch.equal(x, x2) and info2["pcg_iters"] == 9
+    g.close()
+
+
+# entries: 2^18 and 3 * 2^18 (fused prolongation), 2^22 and 3 * 2^22 (early
+# form); rows of 11 entries (cloth) and of about 90 (beam)
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("make", [
+    *(lambda n=n: cut_cloth(n) for n in (23500, 24100, 71000, 72000, 379000, 383000, 1135000, 1150000)),
+    *(lambda n=n: cut_block(n, 10, 10) for n in (3000, 30000, 48000, 141000))],
+    ids=["c23500", "c24100", "c71000", "c72000", "c379000", "c383000", "c1135000", "c1150000",
+         "b3000", "b30000", "b48000", "b141000"])
+def test_csr_forms(make, prec):
+    check_forms(make(), 0, prec)
