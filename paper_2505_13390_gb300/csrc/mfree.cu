@@ -38,10 +38,13 @@ constexpr int kUStride = 3, kUStrideDf = 4;
 // k_mf_vertex32_early, k_mf_vertex64_early: one row or vertex per thread
 // group, static loads before the wait): the kernel is a few waves or less, its
 // time is that of its dependent loads, and its 40 to 80 registers cost little.
-// Above it the plain form's occupancy counts.  Early against plain form: V-cycle
-// on 594,000 rows 201 against 210 us; Chebyshev frame on 195,585 rows 62.3
-// against 62.5 ms; 300 PCG iterations on 3.7M rows 255 against 241 ms.
-constexpr int kEarlyRows = 1 << 20;
+// Above it the plain form's occupancy counts, in FP64 sooner (the gradients take
+// twice the registers).  48 iterations, early against plain: FP64 passes on
+// 11,930 rows 3.95 / 4.09 ms, 93,200 7.25 / 7.38, 96,481 4.83 / 4.84, 150,433 7.59 /
+// 7.32, 195,585 7.34 / 7.06, 478,401 14.2 / 12.8; FP32 passes (the FP64 ones plain)
+// on 195,585 rows 5.07 / 5.30, 689,281 12.90 / 13.29, 925,033 13.52 / 13.69,
+// 938,561 16.16 / 16.40, 1,226,241 20.60 / 19.84.
+constexpr int kEarlyRows32 = 1 << 20, kEarlyRows64 = 1 << 17;
 // tet instances of up to this many rows start with eight FP64 lanes per vertex:
 // a beam's frame takes 191 ms, 201 with four lanes and unfused prolongations;
 // on 3.7M rows A.p takes 224 us with eight and 213 with four
@@ -52,8 +55,10 @@ constexpr int kVertexThreads = 64;
 // loop: the vertices are limited too, and a pass with a dot product, which
 // leaves one partial per block, by the partials the handle holds.
 constexpr int kEarlyDotRows = 4096 * kDotThreads;
+template <class T>
 static bool early(const Handle *h, bool dot = false) {
-  return h->m <= (dot ? std::min(kEarlyRows, kEarlyDotRows) : kEarlyRows) && h->N <= kEarlyRows;
+  const int rows = sizeof(T) == 8 ? kEarlyRows64 : kEarlyRows32;
+  return h->m <= (dot ? std::min(rows, kEarlyDotRows) : rows) && h->N <= rows;
 }
 
 // slot of vertex v in each incident row (create time)
@@ -769,7 +774,7 @@ static int mf_grid(int64_t rows, int threads) {
 template <class T, int MODE>
 static int mf_dot_grid(const Handle *h) {
   const int blocks = blocks_for(h->m, kDotThreads);
-  if (early(h, true)) return blocks;  // one row per thread, as mf_row_launch has it
+  if (early<T>(h, true)) return blocks;  // one row per thread, as mf_row_launch has it
   return std::min(blocks, wave_blocks((const void *)k_mf_row<T, MODE>, kDotThreads));
 }
 
@@ -779,7 +784,7 @@ static mgpbd_status mf_row_launch(Handle *h, const char *what, int blocks, const
                                   const T *dinv, T omega, T *out, const DotCtx &c, double *z,
                                   const double *rr, const int32_t *pos) {
   const bool dot = MODE == MF_APPLY_DOT || MODE == MF_SWEEP_ZDOT;
-  if (early(h, dot))
+  if (early<T>(h, dot))
     return chain_launch(h, what, k_mf_row_early<T, MODE>, blocks_for(h->m, kDotThreads),
                         kDotThreads, h->E, h->m, h->edge, h->tet, gd, gt, u, at, x, b, dinv,
                         omega, out, c, z, rr, pos);
@@ -942,7 +947,7 @@ mgpbd_status mf_cohort_step(int which, int sel, const CohortMember *d_mem,
 static mgpbd_status mf_vertex(Handle *h, const double *x, int G = 0, bool check_done = true) {
   if (G == 0) G = h->force_vert64 ? h->force_vert64 : h->mf_g64;
   const PcgScalars *sc = check_done ? h->sc : nullptr;
-  if (early(h)) {
+  if (early<double>(h)) {
     MF_G_DISPATCH(G, MG_TRY(chain_launch(h, "k_mf_vertex64", k_mf_vertex64_early<GG>,
                                           blocks_for((int64_t)h->N * GG, kVertexThreads),
                                           kVertexThreads, h->N, h->vorder, h->vptr, h->vrow,
@@ -958,7 +963,7 @@ static mgpbd_status mf_vertex(Handle *h, const double *x, int G = 0, bool check_
 static mgpbd_status mf_vertex(Handle *h, const float *x, int G = 0, bool check_done = true) {
   if (G == 0) G = h->force_vert32 ? h->force_vert32 : h->mf_g32;
   const PcgScalars *sc = check_done ? h->sc : nullptr;
-  if (early(h)) {
+  if (early<float>(h)) {
     MF_G_DISPATCH(G, MG_TRY(chain_launch(h, "k_mf_vertex32", k_mf_vertex32_early<GG>,
                                           blocks_for((int64_t)h->N * GG, kVertexThreads),
                                           kVertexThreads, h->N, h->vorder, h->vptr, h->ginc4,
