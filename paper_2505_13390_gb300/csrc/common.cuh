@@ -211,6 +211,7 @@ struct Handle {
   // and their number
   double *part_pq = nullptr, *part_rz = nullptr;
   int n_pq = 0, n_rz = 0, n_rr = 0;
+  bool rr_test = false;  // the next kernel that can test r.r does (RRTest, reduce.cuh)
   unsigned int *counter = nullptr;
   // scratch for setup
   void *tmp = nullptr;

@@ -61,6 +61,8 @@ static bool early(const Handle *h, bool dot = false) {
   return h->m <= (dot ? std::min(rows, kEarlyDotRows) : rows) && h->N <= rows;
 }
 
+bool mf_early(const Handle *h, bool fp64) { return fp64 ? early<double>(h) : early<float>(h); }
+
 // slot of vertex v in each incident row (create time)
 __global__ void k_vslot(int N, int E, const int32_t *edge, const int32_t *tet, const int64_t *vptr,
                         const int32_t *vrow, uint8_t *vslot) {
@@ -158,13 +160,15 @@ __device__ __forceinline__ void mf_vertex64_rows(int64_t w0, int64_t nw, int N,
   }
 }
 
-template <int G>
+// (TEST: with the test on r.r, which takes eight registers more)
+template <int G, bool TEST>
 __global__ void k_mf_vertex64(int N, const int32_t *vorder, const int64_t *vptr,
                               const int32_t *vrow, const double *ginc, const double *w,
-                              const double *x, double *u, const PcgScalars *sc) {
+                              const double *x, double *u, const PcgScalars *sc, RRTest test) {
   chain_wait();
-  if (sc && is_done(sc)) return;
+  if (warp_is_done(sc)) return;
   mf_vertex64_rows<G>(HW_WARPS, N, vorder, vptr, vrow, ginc, w, x, u);
+  if constexpr (TEST) rr_test(test);
 }
 
 template <int G>
@@ -206,13 +210,14 @@ __device__ __forceinline__ void mf_vertex32_rows(int64_t w0, int64_t nw, int N,
   }
 }
 
-template <int G>
+template <int G, bool TEST>
 __global__ void __launch_bounds__(256, 8)
     k_mf_vertex32(int N, const int32_t *vorder, const int64_t *vptr, const float4 *ginc,
-                  const float *w, const float *x, float *u, const PcgScalars *sc) {
+                  const float *w, const float *x, float *u, const PcgScalars *sc, RRTest test) {
   chain_wait();
-  if (sc && is_done(sc)) return;
+  if (warp_is_done(sc)) return;
   mf_vertex32_rows<G>(HW_WARPS, N, vorder, vptr, ginc, w, x, u);
+  if constexpr (TEST) rr_test(test);
 }
 
 // The vertex passes for one group of G lanes per vertex, with the vertex's
@@ -954,9 +959,11 @@ static mgpbd_status mf_vertex(Handle *h, const double *x, int G = 0, bool check_
                                           h->ginc64, h->w, x, h->u64, sc)));
     return MGPBD_OK;
   }
-  MF_G_DISPATCH(G, MG_TRY(chain_launch(h, "k_mf_vertex64", k_mf_vertex64<GG>,
-                                        mf_vertex_blocks(h, GG), 256, h->N, h->vorder, h->vptr,
-                                        h->vrow, h->ginc64, h->w, x, h->u64, sc)));
+  const RRTest test = take_rr_test(h);
+  MF_G_DISPATCH(G, MG_TRY(chain_launch(
+                       h, "k_mf_vertex64", test.sc ? k_mf_vertex64<GG, true> : k_mf_vertex64<GG, false>,
+                       mf_vertex_blocks(h, GG), 256, h->N, h->vorder, h->vptr, h->vrow, h->ginc64,
+                       h->w, x, h->u64, sc, test)));
   return MGPBD_OK;
 }
 
@@ -970,9 +977,11 @@ static mgpbd_status mf_vertex(Handle *h, const float *x, int G = 0, bool check_d
                                           h->w32, x, h->u32, sc)));
     return MGPBD_OK;
   }
-  MF_G_DISPATCH(G, MG_TRY(chain_launch(h, "k_mf_vertex32", k_mf_vertex32<GG>,
-                                        mf_vertex_blocks(h, GG), 256, h->N, h->vorder, h->vptr,
-                                        h->ginc4, h->w32, x, h->u32, sc)));
+  const RRTest test = take_rr_test(h);
+  MF_G_DISPATCH(G, MG_TRY(chain_launch(
+                       h, "k_mf_vertex32", test.sc ? k_mf_vertex32<GG, true> : k_mf_vertex32<GG, false>,
+                       mf_vertex_blocks(h, GG), 256, h->N, h->vorder, h->vptr, h->ginc4, h->w32, x,
+                       h->u32, sc, test)));
   return MGPBD_OK;
 }
 

@@ -25,6 +25,7 @@ enum DotMode {
   DOT_BNORM,      // |b|^2; zero right-hand side finishes at once
   DOT_RZ0,        // initial r.z
   DOT_PART,       // block partials only (p.q, r.r, r.z)
+  DOT_RR,         // r.r's partials and the test on it
   DOT_TR          // |b - A x|^2
 };
 
@@ -37,6 +38,15 @@ struct DotCtx {
   double rtol;
   int maxiter;
 };
+
+// the end of a PCG iteration by its r.r: tolerance, NaN or the iteration cap;
+// true with the status when the solve ends
+static __device__ __forceinline__ bool rr_ends(double rr, double thr2, int iters, int maxiter,
+                                               int *status) {
+  if (rr == rr && rr > thr2 && iters < maxiter) return false;
+  *status = !(rr == rr) ? MGPBD_E_BREAKDOWN : (rr <= thr2 ? MGPBD_OK : MGPBD_W_NOT_CONVERGED);
+  return true;
+}
 
 static __device__ void dot_finalize(const DotCtx &c, double s) {
   PcgScalars *sc = c.sc;
@@ -66,17 +76,21 @@ static __device__ void dot_finalize(const DotCtx &c, double s) {
     case DOT_TR:
       sc->tr2 = s;
       break;
+    case DOT_RR:
+      sc->rr = s;
+      if (rr_ends(s, sc->thr2, sc->iters, c.maxiter, &sc->status)) sc->done = 1;
+      break;
     case DOT_PART:
       break;
   }
 }
 
-// Sum of one value per thread of a block of kDotThreads: through shared memory
-// and one warp, nine FP64 additions instead of five per warp and a serial tail.
-// The result is in thread 0.
+// Sum of one value per thread of a block of kDotThreads (the first kDotThreads
+// of a larger block): through shared memory and one warp, nine FP64 additions
+// instead of five per warp and a serial tail.  The result is in thread 0.
 static __device__ __forceinline__ double block_sum(double v) {
   __shared__ double sd[kDotThreads];
-  sd[threadIdx.x] = v;
+  if (threadIdx.x < kDotThreads) sd[threadIdx.x] = v;
   __syncthreads();
   if (threadIdx.x >= 32) return 0.0;
 #pragma unroll
@@ -88,15 +102,38 @@ static __device__ __forceinline__ double block_sum(double v) {
 // order whatever block does it; the result is in thread 0
 static __device__ __forceinline__ double fold_partials(const double *partials, int vn) {
   double s = 0.0;
-  for (int b = threadIdx.x; b < vn; b += 4 * kDotThreads) {
-    double t[4];
+  if (threadIdx.x < kDotThreads)
+    for (int b = threadIdx.x; b < vn; b += 4 * kDotThreads) {
+      double t[4];
 #pragma unroll
-    for (int k = 0; k < 4; ++k)
-      t[k] = b + k * kDotThreads < vn ? __ldcg(partials + b + k * kDotThreads) : 0.0;
+      for (int k = 0; k < 4; ++k)
+        t[k] = b + k * kDotThreads < vn ? __ldcg(partials + b + k * kDotThreads) : 0.0;
 #pragma unroll
-    for (int k = 0; k < 4; ++k) s += t[k];
-  }
+      for (int k = 0; k < 4; ++k) s += t[k];
+    }
   return block_sum(s);
+}
+
+// The test on r.r by block 0 (of at least kDotThreads threads) of a kernel
+// behind the x/r update, after its own share of the work, so that the rest of the
+// V-cycle does not run once the solve has ended.  Other blocks of the kernel may
+// find the flag raised in their midst: they read it a warp at a time and have no
+// barrier behind it.  sc = nullptr: no test.
+struct RRTest {
+  PcgScalars *sc = nullptr;
+  const double *part = nullptr;
+  int n = 0, maxiter = 0;
+};
+
+static __device__ __forceinline__ void rr_test(const RRTest &t) {
+  if (!t.sc || blockIdx.x != 0) return;
+  const double rr = fold_partials(t.part, t.n);
+  int st;
+  if (threadIdx.x == 0 && rr_ends(rr, t.sc->thr2, t.sc->iters, t.maxiter, &st)) {
+    t.sc->rr = rr;
+    t.sc->status = st;
+    t.sc->done = 1;
+  }
 }
 
 // block reduce of one value per thread in a fixed order, then the last block
@@ -132,6 +169,10 @@ static __device__ __forceinline__ bool is_done(const PcgScalars *sc) {
   return ((volatile const PcgScalars *)sc)->done != 0;
 }
 
+// the same for a warp as a whole
+static __device__ __forceinline__ bool warp_is_done(const PcgScalars *sc) {
+  return sc && __any_sync(0xffffffffu, is_done(sc));
+}
 
 template <int G, class T>
 __device__ __forceinline__ T group_sum(T v) {
@@ -271,13 +312,15 @@ struct NoGate {
 // Runs body(gate) in a kernel's early form, or in its plain form behind the
 // wait and the flag.
 template <bool EARLY, class F>
-__device__ __forceinline__ void behind_gate(const PcgScalars *sc, F body) {
+__device__ __forceinline__ void behind_gate(const PcgScalars *sc, F body,
+                                            const RRTest &test = RRTest()) {
   if constexpr (EARLY) {
     body(ChainGate(sc));
   } else {
     chain_wait();
-    if (sc && is_done(sc)) return;
+    if (warp_is_done(sc)) return;
     body(NoGate{});
+    rr_test(test);
   }
 }
 
@@ -309,7 +352,16 @@ __device__ __forceinline__ void behind_gate(const PcgScalars *sc, F body) {
 #define VG_WARPS(vb, vn)                                                          \
   ((int64_t)(vb) * blockDim.x + threadIdx.x) >> 5, ((int64_t)(vn) * blockDim.x) >> 5
 
+// the test on r.r for the launch being made, if one is due
+inline RRTest take_rr_test(Handle *h) {
+  RRTest t;
+  if (h->rr_test) t = RRTest{h->sc, h->partials, h->n_rr, h->p.pcg_maxiter};
+  h->rr_test = false;
+  return t;
+}
+
 // matrix-free level-0 products (mfree.cu)
+bool mf_early(const Handle *h, bool fp64);  // the V-cycle's passes run in their early form
 mgpbd_status mf_apply_pq(Handle *h, const double *p, double *q, const DotCtx &c);
 mgpbd_status mf_apply_pq_form(Handle *h, bool pairs, const double *p, double *q,
                               const DotCtx &c);

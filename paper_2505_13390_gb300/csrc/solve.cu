@@ -233,12 +233,8 @@ __device__ __forceinline__ void p_update_body(int vb, int vn, int64_t n, double 
   __syncthreads();  // before the buffer of block_sum is used again
   const double rz = fold_partials(part_rz, n_rz);
   if (threadIdx.x == 0) {
-    int go = 0, st = MGPBD_OK;
-    if (!(rr == rr)) st = MGPBD_E_BREAKDOWN;
-    else if (rr <= thr2) st = MGPBD_OK;
-    else if (it >= maxiter) st = MGPBD_W_NOT_CONVERGED;
-    else if (!(rz > 0.0)) st = MGPBD_E_BREAKDOWN;
-    else go = 1;
+    int st = MGPBD_E_BREAKDOWN;
+    const int go = !rr_ends(rr, thr2, it, maxiter, &st) && rz > 0.0;
     sh_be = go ? rz / rz_old : 0.0;
     sh_go = go;
     if (vb == 0 && !gate.closed()) {
@@ -395,14 +391,15 @@ __global__ void k_gs_colour(int nrows, const int32_t *crow, const int64_t *ptr,
 // y = A v (Chebyshev products on CSR levels)
 template <int G, class T>
 __global__ void k_spmv_plain(int n, const int64_t *ptr, const int32_t *col, const T *val,
-                             const T *v, T *y, const PcgScalars *sc) {
+                             const T *v, T *y, const PcgScalars *sc, RRTest test) {
   chain_wait();
-  if (is_done(sc)) return;
+  if (warp_is_done(sc)) return;
   GROUP_ROWS(G, n) {
     T s = valid ? row_dot<G, T, T, T>(ptr, col, val, v, (int)i, g) : (T)0;
     s = group_sum<G>(s);
     if (valid && g == 0) y[i] = s;
   }
+  rr_test(test);
 }
 
 // Chebyshev recurrence: start r = D^-1 (b - A x), d = r / theta, x += d;
@@ -487,18 +484,18 @@ __device__ __forceinline__ void resid_rows(int64_t w0, int64_t nw, int n, const 
 template <int G, class T, bool EARLY>
 __global__ void k_jacobi(int n, const int64_t *ptr, const int32_t *col, const T *val,
                          const T *dinv, T omega, const T *b, const T *x, T *xn,
-                         const PcgScalars *sc) {
+                         const PcgScalars *sc, RRTest test) {
   behind_gate<EARLY>(sc, [&](auto gate) {
     jacobi_rows<G, T>(HW_WARPS, n, ptr, col, val, dinv, omega, b, x, xn, gate);
-  });
+  }, test);
 }
 
 template <int G, class T, bool EARLY>
 __global__ void k_resid(int n, const int64_t *ptr, const int32_t *col, const T *val, const T *b,
-                        const T *x, T *r, const PcgScalars *sc) {
+                        const T *x, T *r, const PcgScalars *sc, RRTest test) {
   behind_gate<EARLY>(sc, [&](auto gate) {
     resid_rows<G, T>(HW_WARPS, n, ptr, col, val, b, x, r, gate);
-  });
+  }, test);
 }
 
 // The first post-smoothing sweep with the prolongation taken along: every x_j
@@ -1700,10 +1697,12 @@ static mgpbd_status vcycle_level(Handle *h, int l, const T *b_in, T **res, bool 
   // smooth_sweeps products; coefficients follow from the lazily estimated
   // lambda_max of the setup (Sec. 4.5)
   const bool cheb = h->p.smoother == MGPBD_SMOOTH_CHEBYSHEV;
+  // the level-0 launches that take the test on r.r along (plain forms)
+  auto test = [&] { return l == 0 ? take_rr_test(h) : RRTest(); };
   auto apply = [&](const T *v, T *y) -> mgpbd_status {
     if (mf) return mf_level0<T>(h, kMfApply, v, b_in, dinv, om, y);
     DISPATCH_G(G, MG_TRY(rows_launch(h, "k_spmv_plain", k_spmv_plain<GG, T>, n, GG, n, L.ptr, L.col,
-                                     val, v, y, sc)));
+                                     val, v, y, sc, test())));
     return MGPBD_OK;
   };
   // (from_zero: x = 0 on entry, so A x = 0 needs no product)
@@ -1732,7 +1731,7 @@ static mgpbd_status vcycle_level(Handle *h, int l, const T *b_in, T **res, bool 
     } else {
       DISPATCH_G(G, DISPATCH_EARLY(early_rows<T>(L), MG_TRY(rows_launch(
                         h, "k_jacobi", k_jacobi<GG, T, EE>, n, GG, n, L.ptr, L.col, val, dinv, om,
-                        b_in, x, x2, sc))));
+                        b_in, x, x2, sc, EE ? RRTest() : test()))));
     }
     if (l == 0) MG_TRY(prof_end(h));
     std::swap(x, x2);
@@ -1766,7 +1765,7 @@ static mgpbd_status vcycle_level(Handle *h, int l, const T *b_in, T **res, bool 
     else
       DISPATCH_G(G, DISPATCH_EARLY(early_rows<T>(L), MG_TRY(rows_launch(
                         h, "k_resid", k_resid<GG, T, EE>, n, GG, n, L.ptr, L.col, val, b_in, x, r,
-                        sc))));
+                        sc, EE ? RRTest() : test()))));
     MG_TRY(item_launch(h, "k_restrict", k_restrict<T>, 32ll * L.n_agg, L.n_agg, nk, L.mptr, L.mrow,
                        Ps<T>(L), r, (T *)Lc.b, sc, dinv_c, (T)Lc.omega, x_c));
   }
@@ -1813,7 +1812,7 @@ static mgpbd_status vcycle_level(Handle *h, int l, const T *b_in, T **res, bool 
         // sweep of long rows lacks registers (113.9 against 110.1 ms for 48
         // iterations on 1.3M rows of the block, r.z in a launch of its own)
         MG_TRY(rows_launch(h, "k_jacobi", k_jacobi<GG, T, EE>, n, GG, n, L.ptr, L.col, val, dinv,
-                           om, b_in, x, (T *)top->z, sc));
+                           om, b_in, x, (T *)top->z, sc, RRTest()));
         if (top->dot) MG_TRY(launch_dot(h, top->r, top->z, n, top->c.mode, 1));
       } else {
         const int blocks = jacobi_final_blocks<GG, T, EE>(n);
@@ -1905,6 +1904,20 @@ mgpbd_status dot_dd(Handle *h, const double *x, const double *y, int64_t n, doub
   return launch_dot(h, x, y, n, DOT_STORE, 0, d_out);
 }
 
+// Whether the V-cycle's first level-0 pass tests r.r (rr_test).  The p update
+// tests it in any case, which costs the last iteration a V-cycle for nothing:
+// little on a small instance, but a solve of one iteration on the block of 1.33M
+// rows then takes 4.6 ms in FP64 against 3.0.  In the x/r update's last block
+// the test costs every iteration 3 us (that of the block 357 us against 354); in
+// the plain forms, which large instances run, block 0 makes it on the side.
+static bool hosts_rr_test(const Handle *h) {
+  const bool dbl = h->p.precision != MGPBD_MIXED;
+  if (h->p.level0_op == 1) return !mf_early(h, dbl);
+  const Level &L = h->lev[0];
+  if (dbl ? early_rows<double>(L) : early_rows<float>(L)) return false;
+  return spread((int64_t)L.n * group_for(h, L, dbl)) >= kDotThreads;
+}
+
 // one PCG iteration (kernels return early once `done` is set)
 static mgpbd_status pcg_iteration(Handle *h, double *x) {
   Level &L = h->lev[0];
@@ -1930,19 +1943,25 @@ static mgpbd_status pcg_iteration(Handle *h, double *x) {
   MG_TRY(prof_end(h, PROF_AP));
   // the update also starts the V-cycle (right-hand side, first Jacobi sweep)
   const bool jac = top_jacobi(h);
+  // Gauss-Seidel on a large matrix: an iteration of hundreds of launches, so the
+  // x/r update's last block may as well test r.r (3 us)
+  const bool gs = h->p.smoother == MGPBD_SMOOTH_MCGS;
+  const int rr_at = gs && !early_rows<double>(L) ? DOT_RR : DOT_PART;
   if (h->p.precision == MGPBD_MIXED)
     MG_TRY(chain_launch(h, "k_xr_update", k_xr_update<float>,
                         h->n_rr = xr_blocks<float>(m),
-                        kDotThreads, m, x, r, p, q, make_ctx(h, DOT_PART), h->part_pq, h->n_pq,
+                        kDotThreads, m, x, r, p, q, make_ctx(h, rr_at), h->part_pq, h->n_pq,
                         (float *)L.b, L.dinv32,
                         (float)L.omega, jac ? (float *)L.x : nullptr));
   else
     MG_TRY(chain_launch(h, "k_xr_update", k_xr_update<double>,
                         h->n_rr = xr_blocks<double>(m),
-                        kDotThreads, m, x, r, p, q, make_ctx(h, DOT_PART), h->part_pq, h->n_pq,
+                        kDotThreads, m, x, r, p, q, make_ctx(h, rr_at), h->part_pq, h->n_pq,
                         nullptr, L.dinv, L.omega,
                         jac ? (double *)L.x : nullptr));
+  h->rr_test = !gs && hosts_rr_test(h);
   MG_TRY(vcycle_top(h, r, z, true, DOT_PART));
+  h->rr_test = false;
   MG_TRY(chain_launch(h, "k_p_update", k_p_update, p_blocks(m), kDotThreads, m, p, z, h->sc,
                       h->p.pcg_maxiter, h->partials, h->n_rr, h->part_rz, h->n_rz,
                       h->p.ap_split ? h->p_df : nullptr));
@@ -2127,7 +2146,7 @@ static mgpbd_status time_resid(Handle *h, const Level &L, int G, const T *val, c
     MG_TRY(evict_l2(h));
     MG_CUDA(cudaEventRecord(h->ev0, h->stream));
     DISPATCH_G(G, DISPATCH_EARLY(early_rows<T>(L), k_resid<GG, T, EE><<<row_blocks(n, GG), 256, 0, h->stream>>>(
-                                            n, L.ptr, L.col, val, b, x, r, nullptr)));
+                                            n, L.ptr, L.col, val, b, x, r, nullptr, RRTest())));
     MG_LAUNCH("k_resid(tune)");
     MG_CUDA(cudaEventRecord(h->ev1, h->stream));
     MG_CUDA(cudaEventSynchronize(h->ev1));

@@ -139,3 +139,67 @@ def test_csr_forms(make, prec):
          "c1048577-1", "b131072-0", "b131073-0", "b524288-1", "b524289-1", "b3000-0", "b3000-1"])
 def test_matrix_free_forms(make, prec):
     check_forms(make(), 1, prec)
+
+
+# the places of the test on r.r: a large level 0's first pass in each form
+# (matrix-free and CSR, Jacobi with one and two sweeps, Chebyshev), the x/r update
+# (Gauss-Seidel on a large matrix) and the p update (small instances)
+@pytest.mark.parametrize("rows,over", [
+    (1100000, dict(precision=1, level0_op=1)), (200000, dict(precision=0, level0_op=1)),
+    (1100000, dict(precision=1, level0_op=1, smoother=2)), (390000, dict(precision=0)),
+    (1200000, dict(precision=1)), (390000, dict(precision=0, smooth_sweeps=1)),
+    (390000, dict(precision=0, smoother=2)), (390000, dict(precision=0, smoother=1)),
+    (9000, dict(precision=1, level0_op=1)), (9000, dict(precision=0, smoother=1))])
+@pytest.mark.parametrize("graphs", [0, 1])
+def test_solve_ends_where_it_should(rows, over, graphs):
+    """A solve to a tolerance ends in the first iteration at or below it, with
+    the solution and residual of a solve capped there; one iteration less is
+    above the tolerance and says so."""
+    mesh = cut_cloth(rows)
+    got = {}
+    with torch.cuda.stream(torch.cuda.Stream()):
+        gen = torch.Generator(device="cuda").manual_seed(5)
+        b = torch.randn(rows, dtype=torch.float64, device="cuda", generator=gen)
+        k = None
+        for case in ("tolerance", "before", "at"):
+            tol = 1e-2 if case != "at" else 1e-300
+            cap = {"tolerance": 5000, "before": (k or 1) - 1, "at": k}[case]
+            if cap == 0:
+                continue
+            g = ready(mesh, pcg_rtol=tol, pcg_maxiter=cap, use_graphs=graphs, **over)
+            x, info = g.solve(b)
+            got[case] = x, info
+            k = k or info["pcg_iters"]
+            g.close()
+    x, info = got["tolerance"]
+    assert info["status"] == 0 and info["pcg_iters"] == k and info["rel_res"] <= 1e-2
+    x2, info2 = got["at"]
+    assert torch.equal(x, x2) and info2["pcg_iters"] == k and info2["status"] == 1
+    assert info2["rel_res"] == info["rel_res"]
+    if k > 1:
+        _, info3 = got["before"]
+        assert info3["status"] == 1 and info3["pcg_iters"] == k - 1 and info3["rel_res"] > 1e-2
+
+
+def test_last_iteration_leaves_the_vcycle_out():
+    """One FP64 iteration on an assembled block of 0.6M rows: a V-cycle, a
+    product and the vector updates, not a second V-cycle (which would be 0.5
+    V-cycles above the line, and its absence is as far below it)."""
+    import time
+    mesh = hex_block(40, 33, 40, h=0.005, jitter=0.1, alpha=1e-10, pin="y0", seed=1)
+
+    def best(f):
+        ts = []
+        for _ in range(15):
+            torch.cuda.synchronize()
+            t = time.perf_counter()
+            f()
+            torch.cuda.synchronize()
+            ts.append(time.perf_counter() - t)
+        return min(ts)
+
+    g = ready(mesh, precision=0, pcg_maxiter=1, pcg_rtol=1e-300)
+    r = torch.randn(g.m, dtype=torch.float64, device="cuda")
+    cycle, product, solve = best(lambda: g.vcycle(r)), best(lambda: g.apply(r)), best(lambda: g.solve(r))
+    g.close()
+    assert solve <= 1.5 * cycle + 2 * product, (solve, cycle, product)
