@@ -1025,12 +1025,12 @@ static bool early_rows(const Level &L) {
 // short.  Whole solves, fused against not: FP64 2.09 / 2.12 ms at 132K entries,
 // 3.65 / 3.56 at 543K (cloths), 5.15 / 4.99 with the fusion on a beam's levels of
 // up to 64K; FP32 2.82 / 2.87 at 543K, 5.10 / 5.03 at 2.1M (cloths), 3.20 / 3.26 on
-// a beam's levels of up to 192K and 3.22 with those of up to 768K.
+// a beam's levels of up to 192K, 4.06 / 4.13 on one of 222K, 2.35 / 2.32 at 504K.
 template <class T>
 static bool fuse_prolong(const Level &L) {
   const bool short_rows = L.nnz <= 16 * (int64_t)L.n;
   if (sizeof(T) == 8) return short_rows && L.nnz <= 1 << 18;
-  return L.nnz <= (short_rows ? 3 << 18 : 3 << 16);
+  return L.nnz <= (short_rows ? 3 << 18 : 7 << 16);
 }
 
 #define DISPATCH_EARLY(early, ...)                 \
