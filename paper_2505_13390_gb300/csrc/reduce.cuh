@@ -129,10 +129,12 @@ static __device__ __forceinline__ void rr_test(const RRTest &t) {
   if (!t.sc || blockIdx.x != 0) return;
   const double rr = fold_partials(t.part, t.n);
   int st;
-  if (threadIdx.x == 0 && rr_ends(rr, t.sc->thr2, t.sc->iters, t.maxiter, &st)) {
+  if (threadIdx.x == 0) {
     t.sc->rr = rr;
-    t.sc->status = st;
-    t.sc->done = 1;
+    if (rr_ends(rr, t.sc->thr2, t.sc->iters, t.maxiter, &st)) {
+      t.sc->status = st;
+      t.sc->done = 1;
+    }
   }
 }
 

@@ -198,12 +198,14 @@ __global__ void k_top_prep(int64_t n, const double *r, T *bl, const T *dinv, T o
   }
 }
 
-// The convergence test on r.r and beta = r.z / (r.z of the iteration before),
-// both from block partials (r.r at the tolerance, the iteration cap and a
-// breakdown r.z <= 0 end the solve; the V-cycle of the last iteration has then
-// run for nothing); p = z + beta p, two entries per thread (16-byte
-// loads; p and z are 256-byte aligned); with pdf, p also as float-float pairs
-// for the pair form of A.p (params.ap_split)
+// The convergence test on r.r (n_rr = 0: made already, rr_test) and beta = r.z /
+// (r.z of the iteration before), both from block partials (r.r at the tolerance,
+// the iteration cap and a breakdown r.z <= 0 end the solve; the V-cycle of the
+// last iteration has then run for nothing); p = z + beta p, two entries per thread
+// (16-byte loads; p and z are 256-byte aligned); with pdf, p also as float-float
+// pairs for the pair form of A.p (params.ap_split).  Every block adds all of the
+// partials, one FP64 addition each (1.6 a clock and SM), so large instances take
+// few large blocks (p_threads).
 template <class Gate>
 __device__ __forceinline__ void p_update_body(int vb, int vn, int64_t n, double *p,
                                               const double *z, PcgScalars *sc, int maxiter,
@@ -229,16 +231,19 @@ __device__ __forceinline__ void p_update_body(int vb, int vn, int64_t n, double 
   const double rz_old = sc->rz[(it - 1) & 1], thr2 = sc->thr2;
   __shared__ double sh_be;
   __shared__ int sh_go;
-  const double rr = fold_partials(part_rr, n_rr);
-  __syncthreads();  // before the buffer of block_sum is used again
+  double rr = 0.0;
+  if (n_rr) {
+    rr = fold_partials(part_rr, n_rr);
+    __syncthreads();  // before the buffer of block_sum is used again
+  }
   const double rz = fold_partials(part_rz, n_rz);
   if (threadIdx.x == 0) {
     int st = MGPBD_E_BREAKDOWN;
-    const int go = !rr_ends(rr, thr2, it, maxiter, &st) && rz > 0.0;
+    const int go = !(n_rr && rr_ends(rr, thr2, it, maxiter, &st)) && rz > 0.0;
     sh_be = go ? rz / rz_old : 0.0;
     sh_go = go;
     if (vb == 0 && !gate.closed()) {
-      sc->rr = rr;
+      if (n_rr) sc->rr = rr;
       if (go) {
         sc->rz[it & 1] = rz;
         sc->beta = sh_be;
@@ -1053,10 +1058,16 @@ static int jacobi_final_blocks(int n) {
   return std::min(row_blocks(n, G, kDotThreads),
                   wave_blocks((const void *)k_jacobi_final<G, T, EARLY>, kDotThreads));
 }
-// p update: four entries per thread, at most sixteen blocks per SM (every block
-// folds r.z's partials)
-static int p_blocks(int m) {
-  return std::min(blocks_for(std::max(1, (m / 2 + 1) / 2), kDotThreads), 16 * num_sms());
+// p update: four entries per thread; on large instances two large blocks per SM,
+// which loop.  With up to sixteen blocks of 128 threads per SM, each adding 1,500
+// to 4,000 partials, the launch took 35.0 us on the 1.65M-tet block, of 72 MB of
+// vectors; 48 iterations there 36.06 ms and 35.60 so, 9.51 and 9.17 on 478,401 rows
+// of cloth, 5.09 and 5.08 on 195,585, 4.05 and 4.06 on a beam of 93,200.
+constexpr int kPLarge = 1 << 17, kPThreads = 512, kPBlocks = 2;
+static int p_threads(int m) { return m > kPLarge ? kPThreads : kDotThreads; }
+static int p_blocks(int m, int threads) {
+  return std::min(blocks_for(std::max(1, (m / 2 + 1) / 2), threads),
+                  (threads == kPThreads ? kPBlocks : 16) * num_sms());
 }
 template <class T>
 static int xr_blocks(int m) {
@@ -1507,7 +1518,7 @@ mgpbd_status cohort_build(Cohort *c) {
     M.grid[CS_XR] = xr_blocks<float>(m);
     M.grid[CS_RESTRICT] = blocks_for((int64_t)L0.n_agg * 32, 256);
     M.grid[CS_PROLONG] = blocks_for((m + kProlongRows - 1) / kProlongRows, 256);
-    M.grid[CS_PUPD] = p_blocks(m);
+    M.grid[CS_PUPD] = p_blocks(m, kDotThreads);
     c->gens[k] = h->gen;
   }
   c->gv32 = mem.empty() ? 0 : mem[0].gv32;
@@ -1960,10 +1971,13 @@ static mgpbd_status pcg_iteration(Handle *h, double *x) {
                         nullptr, L.dinv, L.omega,
                         jac ? (double *)L.x : nullptr));
   h->rr_test = !gs && hosts_rr_test(h);
+  const bool due = h->rr_test;
   MG_TRY(vcycle_top(h, r, z, true, DOT_PART));
+  const bool tested = due && !h->rr_test;
   h->rr_test = false;
-  MG_TRY(chain_launch(h, "k_p_update", k_p_update, p_blocks(m), kDotThreads, m, p, z, h->sc,
-                      h->p.pcg_maxiter, h->partials, h->n_rr, h->part_rz, h->n_rz,
+  MG_TRY(chain_launch(h, "k_p_update", k_p_update,
+                      p_blocks(m, p_threads(m)), p_threads(m), m, p, z, h->sc,
+                      h->p.pcg_maxiter, h->partials, tested ? 0 : h->n_rr, h->part_rz, h->n_rz,
                       h->p.ap_split ? h->p_df : nullptr));
   return MGPBD_OK;
 }
