@@ -85,12 +85,15 @@ static __device__ void dot_finalize(const DotCtx &c, double s) {
   }
 }
 
-// Sum of one value per thread of a block of kDotThreads (the first kDotThreads
-// of a larger block): through shared memory and one warp, nine FP64 additions
-// instead of five per warp and a serial tail.  The result is in thread 0.
+// Sum of one value per thread of a block of kDotThreads: through shared memory
+// and one warp, nine FP64 additions instead of five per warp and a serial tail.
+// The result is in thread 0.  LARGER: over the first kDotThreads of a larger
+// block (the guard costs a launch of few blocks up to 2 us, so the others go
+// without it).
+template <bool LARGER = false>
 static __device__ __forceinline__ double block_sum(double v) {
   __shared__ double sd[kDotThreads];
-  if (threadIdx.x < kDotThreads) sd[threadIdx.x] = v;
+  if (!LARGER || threadIdx.x < kDotThreads) sd[threadIdx.x] = v;
   __syncthreads();
   if (threadIdx.x >= 32) return 0.0;
 #pragma unroll
@@ -100,9 +103,10 @@ static __device__ __forceinline__ double block_sum(double v) {
 
 // sum over the partials of a reduction of vn blocks by one block, in a fixed
 // order whatever block does it; the result is in thread 0
+template <bool LARGER = false>
 static __device__ __forceinline__ double fold_partials(const double *partials, int vn) {
   double s = 0.0;
-  if (threadIdx.x < kDotThreads)
+  if (!LARGER || threadIdx.x < kDotThreads)
     for (int b = threadIdx.x; b < vn; b += 4 * kDotThreads) {
       double t[4];
 #pragma unroll
@@ -111,7 +115,7 @@ static __device__ __forceinline__ double fold_partials(const double *partials, i
 #pragma unroll
       for (int k = 0; k < 4; ++k) s += t[k];
     }
-  return block_sum(s);
+  return block_sum<LARGER>(s);
 }
 
 // The test on r.r by block 0 (of at least kDotThreads threads) of a kernel
@@ -127,7 +131,7 @@ struct RRTest {
 
 static __device__ __forceinline__ void rr_test(const RRTest &t) {
   if (!t.sc || blockIdx.x != 0) return;
-  const double rr = fold_partials(t.part, t.n);
+  const double rr = fold_partials<true>(t.part, t.n);
   int st;
   if (threadIdx.x == 0) {
     t.sc->rr = rr;

@@ -206,7 +206,7 @@ __global__ void k_top_prep(int64_t n, const double *r, T *bl, const T *dinv, T o
 // pairs for the pair form of A.p (params.ap_split).  Every block adds all of the
 // partials, one FP64 addition each (1.6 a clock and SM), so large instances take
 // few large blocks (p_threads).
-template <class Gate>
+template <bool LARGER, class Gate>
 __device__ __forceinline__ void p_update_body(int vb, int vn, int64_t n, double *p,
                                               const double *z, PcgScalars *sc, int maxiter,
                                               const double *part_rr, int n_rr,
@@ -233,10 +233,10 @@ __device__ __forceinline__ void p_update_body(int vb, int vn, int64_t n, double 
   __shared__ int sh_go;
   double rr = 0.0;
   if (n_rr) {
-    rr = fold_partials(part_rr, n_rr);
+    rr = fold_partials<LARGER>(part_rr, n_rr);
     __syncthreads();  // before the buffer of block_sum is used again
   }
-  const double rz = fold_partials(part_rz, n_rz);
+  const double rz = fold_partials<LARGER>(part_rz, n_rz);
   if (threadIdx.x == 0) {
     int st = MGPBD_E_BREAKDOWN;
     const int go = !(n_rr && rr_ends(rr, thr2, it, maxiter, &st)) && rz > 0.0;
@@ -284,10 +284,11 @@ __device__ __forceinline__ void p_update_body(int vb, int vn, int64_t n, double 
   }
 }
 
+template <bool LARGER>
 __global__ void k_p_update(int64_t n, double *p, const double *z, PcgScalars *sc, int maxiter,
                            const double *part_rr, int n_rr, const double *part_rz, int n_rz,
                            float2 *pdf) {
-  p_update_body(blockIdx.x, gridDim.x, n, p, z, sc, maxiter, part_rr, n_rr, part_rz, n_rz, pdf,
+  p_update_body<LARGER>(blockIdx.x, gridDim.x, n, p, z, sc, maxiter, part_rr, n_rr, part_rz, n_rz, pdf,
                 ChainGate(sc));
 }
 
@@ -394,17 +395,17 @@ __global__ void k_gs_colour(int nrows, const int32_t *crow, const int64_t *ptr,
 }
 
 // y = A v (Chebyshev products on CSR levels)
-template <int G, class T>
+template <int G, class T, bool TEST>
 __global__ void k_spmv_plain(int n, const int64_t *ptr, const int32_t *col, const T *val,
                              const T *v, T *y, const PcgScalars *sc, RRTest test) {
   chain_wait();
-  if (warp_is_done(sc)) return;
+  if (TEST ? warp_is_done(sc) : is_done(sc)) return;
   GROUP_ROWS(G, n) {
     T s = valid ? row_dot<G, T, T, T>(ptr, col, val, v, (int)i, g) : (T)0;
     s = group_sum<G>(s);
     if (valid && g == 0) y[i] = s;
   }
-  rr_test(test);
+  if constexpr (TEST) rr_test(test);
 }
 
 // Chebyshev recurrence: start r = D^-1 (b - A x), d = r / theta, x += d;
@@ -1315,7 +1316,7 @@ __global__ void kb_prolong0(const CohortMember *mem, const CohortBlock *blk) {
 
 __global__ void kb_pupdate(const CohortMember *mem, const CohortBlock *blk) {
   COHORT_BLOCK_ENDING;
-  p_update_body(vb, vn, M.m, M.p, M.z, M.sc, M.c_rr.maxiter, M.c_rr.partials, M.grid[CS_XR],
+  p_update_body<false>(vb, vn, M.m, M.p, M.z, M.sc, M.c_rr.maxiter, M.c_rr.partials, M.grid[CS_XR],
                 M.c_rz.partials, M.grid[CS_ROW_FINAL], nullptr, NoGate{});
 }
 
@@ -1725,8 +1726,11 @@ static mgpbd_status vcycle_level(Handle *h, int l, const T *b_in, T **res, bool 
   auto test = [&] { return l == 0 ? take_rr_test(h) : RRTest(); };
   auto apply = [&](const T *v, T *y) -> mgpbd_status {
     if (mf) return mf_level0<T>(h, kMfApply, v, b_in, dinv, om, y);
-    DISPATCH_G(G, MG_TRY(rows_launch(h, "k_spmv_plain", k_spmv_plain<GG, T>, n, GG, n, L.ptr, L.col,
-                                     val, v, y, sc, test())));
+    const RRTest t = test();
+    DISPATCH_G(G, MG_TRY(rows_launch(
+                      h, "k_spmv_plain",
+                      t.sc ? k_spmv_plain<GG, T, true> : k_spmv_plain<GG, T, false>, n, GG, n,
+                      L.ptr, L.col, val, v, y, sc, t)));
     return MGPBD_OK;
   };
   // (from_zero: x = 0 on entry, so A x = 0 needs no product)
@@ -1991,8 +1995,9 @@ static mgpbd_status pcg_iteration(Handle *h, double *x) {
   MG_TRY(vcycle_top(h, r, z, true, DOT_PART));
   const bool tested = due && !h->rr_test;
   h->rr_test = false;
-  MG_TRY(chain_launch(h, "k_p_update", k_p_update,
-                      p_blocks(m, p_threads(m)), p_threads(m), m, p, z, h->sc,
+  const int th = p_threads(m);
+  MG_TRY(chain_launch(h, "k_p_update", th > kDotThreads ? k_p_update<true> : k_p_update<false>,
+                      p_blocks(m, th), th, m, p, z, h->sc,
                       h->p.pcg_maxiter, h->partials, tested ? 0 : h->n_rr, h->part_rz, h->n_rz,
                       h->p.ap_split ? h->p_df : nullptr));
   return MGPBD_OK;
