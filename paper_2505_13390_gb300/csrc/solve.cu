@@ -1919,7 +1919,7 @@ mgpbd_status apply_level0(Handle *h, int form, const double *x, double *y) {
   const Level &L = h->lev[0];
   k_pcg_init<<<1, 1, 0, h->stream>>>(h->sc, h->gbar);
   MG_LAUNCH("k_pcg_init");
-  DotCtx c = make_ctx(h, DOT_STORE, &h->sc->tr2);  // x.Ax lands in a scratch scalar
+  const DotCtx c = pq_ctx(h);  // x.Ax stays in block partials, which nothing reads
   if (form == 0) {
     const int G = group_for(h, L, true);
     DISPATCH_G(G, DISPATCH_EARLY(early_rows<double>(L), MG_TRY(chain_launch(
