@@ -310,11 +310,35 @@ __device__ __forceinline__ int row_setup(int i, int E, const int32_t *edge, cons
   return c;
 }
 
+// diagonal of A and its reciprocal, one row per thread
+__device__ __forceinline__ void assemble_diag_row(int64_t i, int E, const int32_t *edge,
+                                                  const int32_t *tet, const double *w,
+                                                  const double *gd, const double *gt,
+                                                  const double *alpha_t, const int64_t *ptr,
+                                                  double *val, double *dinv, float *val32,
+                                                  float *dinv32) {
+  double gi[4][3], wi[4];
+  const int c = row_setup((int)i, E, edge, tet, w, gd, gt, gi, wi);
+  double acc = 0.0;
+#pragma unroll
+  for (int s = 0; s < 4; ++s)
+    if (s < c) acc = fma(wi[s], gdot(gi[s], gi[s]), acc);
+  const double d = acc + alpha_t[i], r = 1.0 / d;
+  const int64_t e = ptr[i + 1] - 1;
+  val[e] = d;
+  dinv[i] = r;
+  if (val32) {
+    val32[e] = f64_to_f32(d);
+    dinv32[i] = f64_to_f32(r);
+  }
+}
+
 // Off-diagonal values of A (eq. 3, Sec. 4.2 formulas), G lanes per row over its
 // entries, and in mixed precision their FP32 mirrors.  Bound by FP64 issue (a
 // warp's FP64 instruction holds its SM for 20 clocks whatever number of lanes
 // is active).  So the lanes per row follow the row length; the diagonal, one
-// value per row with a division, has a kernel of its own with one row per lane;
+// value per row with a division, is done one row per thread by further blocks of
+// the launch (a launch of its own costs small instances 4 us of host time);
 // and every entry adds its first shared vertex at once, while those with a
 // second and third one (tets that share an edge or a face) go to the warp's
 // stack in shared memory and are worked off 32 at a time, one vertex per turn.
@@ -333,7 +357,14 @@ template <int G>
 __global__ void __launch_bounds__(32 * kAsmWarps)
     k_assemble(int m, int E, int batches, const int32_t *edge, const int32_t *tet, const double *w,
                const double *gd, const double *gt, const int64_t *ptr, const int32_t *col,
-               const uint16_t *map, double *val, float *val32) {
+               const uint16_t *map, double *val, float *val32, int off_blocks,
+               const double *alpha_t, double *dinv, float *dinv32) {
+  if ((int)blockIdx.x >= off_blocks) {
+    const int64_t i = (int64_t)(blockIdx.x - off_blocks) * blockDim.x + threadIdx.x;
+    if (i < m)
+      assemble_diag_row(i, E, edge, tet, w, gd, gt, alpha_t, ptr, val, dinv, val32, dinv32);
+    return;
+  }
   __shared__ AsmItem items[kAsmWarps][64];
   __shared__ uint16_t codes[kAsmWarps][64];
   const int lane = threadIdx.x & 31, g = threadIdx.x & (G - 1);
@@ -418,29 +449,6 @@ __global__ void __launch_bounds__(32 * kAsmWarps)
   while (n) work_off();
 }
 
-// diagonal of A and its reciprocal, one row per thread
-__global__ void k_assemble_diag(int m, int E, const int32_t *edge, const int32_t *tet,
-                                const double *w, const double *gd, const double *gt,
-                                const double *alpha_t, const int64_t *ptr, double *val,
-                                double *dinv, float *val32, float *dinv32) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < m; i += gridDim.x * blockDim.x) {
-    double gi[4][3], wi[4];
-    const int c = row_setup(i, E, edge, tet, w, gd, gt, gi, wi);
-    double acc = 0.0;
-#pragma unroll
-    for (int s = 0; s < 4; ++s)
-      if (s < c) acc = fma(wi[s], gdot(gi[s], gi[s]), acc);
-    const double d = acc + alpha_t[i], r = 1.0 / d;
-    const int64_t e = ptr[i + 1] - 1;
-    val[e] = d;
-    dinv[i] = r;
-    if (val32) {
-      val32[e] = f64_to_f32(d);
-      dinv32[i] = f64_to_f32(r);
-    }
-  }
-}
-
 mgpbd_status launch_assemble(Handle *h) {
   if (h->m == 0) return MGPBD_OK;
   Level &L = h->lev[0];
@@ -450,20 +458,16 @@ mgpbd_status launch_assemble(Handle *h) {
     const int64_t warps = ((int64_t)h->m * G + 31) / 32;
     const int64_t full = warps / (64 * num_sms());
     const int batches = (int)std::min<int64_t>(std::max<int64_t>(full, 1), kAsmBatches);
-    const int64_t per = (int64_t)kAsmWarps * batches;
-    kernel<<<(unsigned)((warps + per - 1) / per), 32 * kAsmWarps, 0, h->stream>>>(
+    const int off_blocks = blocks_covering(warps, kAsmWarps * batches);
+    const int diag_blocks = blocks_covering(h->m, 32 * kAsmWarps);
+    kernel<<<off_blocks + diag_blocks, 32 * kAsmWarps, 0, h->stream>>>(
         h->m, h->E, batches, h->edge, h->tet, h->w, h->gd, h->gt, L.ptr, L.col, h->map, L.val,
-        L.val32);
+        L.val32, off_blocks, h->alpha_t, L.dinv, L.dinv32);
     MG_LAUNCH("k_assemble");
     return MGPBD_OK;
   };
-  MG_TRY(avg <= 12 ? off(k_assemble<8>, 8) : (avg <= 48 ? off(k_assemble<16>, 16)
-                                                        : off(k_assemble<32>, 32)));
-  k_assemble_diag<<<blocks_for(h->m, 128), 128, 0, h->stream>>>(
-      h->m, h->E, h->edge, h->tet, h->w, h->gd, h->gt, h->alpha_t, L.ptr, L.val, L.dinv, L.val32,
-      L.dinv32);
-  MG_LAUNCH("k_assemble_diag");
-  return MGPBD_OK;
+  return avg <= 12 ? off(k_assemble<8>, 8) : (avg <= 48 ? off(k_assemble<16>, 16)
+                                                        : off(k_assemble<32>, 32));
 }
 
 // ---------------------------------------------------------------------------
