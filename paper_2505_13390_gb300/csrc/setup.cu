@@ -82,22 +82,23 @@ __global__ void k_nk_init(int n, uint64_t seed, const unsigned long long *amax_b
 
 // Weighted-Jacobi sweep with row sums in storage order, s = fma(A_ij, x_j, s).
 // The sum of a row is one chain of fused multiply-adds, so a warp runs the
-// chains of 32 rows side by side, one per lane: it loads 32 entries of each row
+// chains of R rows side by side, one per lane: it loads 32 entries of each row
 // at a time (coalesced, the row's lanes together) into shared memory and every
 // lane folds its own row from there.  (One row per warp, folded by one lane,
 // spent a warp's FP64 instruction, 20 clocks of an SM on this part, on each
-// entry: 286 us per sweep of a 46,760-row beam, 104 us so.)  There is no loop
-// over the rows: the grid covers them (blocks_covering).
+// entry.)  There is no loop over the rows: the grid covers them
+// (blocks_covering).
 constexpr int kNkWarps = 4, kNkPitch = 33;
+template <int R>
 __global__ void __launch_bounds__(32 * kNkWarps)
     k_nk_sweep(int n, const int64_t *ptr, const int32_t *col, const double *val, double omega,
                const double *x, double *xn) {
   extern __shared__ double2 nk_smem[];
-  double2 *buf = nk_smem + (threadIdx.x >> 5) * (32 * kNkPitch);
+  double2 *buf = nk_smem + (threadIdx.x >> 5) * (R * kNkPitch);
   const int lane = threadIdx.x & 31;
-  const int64_t base = ((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5) * 32;
+  const int64_t base = ((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5) * R;
   if (base >= n) return;
-  const int rows = (int)min((int64_t)32, n - base);
+  const int rows = (int)min((int64_t)R, n - base);
   const int64_t s0 = lane < rows ? ptr[base + lane] : 0, e = lane < rows ? ptr[base + lane + 1] : 0;
   int longest = (int)(e - s0);
 #pragma unroll
@@ -105,7 +106,7 @@ __global__ void __launch_bounds__(32 * kNkWarps)
   double s = 0.0;
   for (int c = 0; c < longest; c += 32) {
 #pragma unroll 8
-    for (int r = 0; r < 32; ++r) {
+    for (int r = 0; r < R; ++r) {
       const int64_t k = __shfl_sync(0xffffffffu, s0, r) + c + lane;
       if (k < __shfl_sync(0xffffffffu, e, r))
         buf[r * kNkPitch + lane] = make_double2(val[k], x[col[k]]);
@@ -119,6 +120,24 @@ __global__ void __launch_bounds__(32 * kNkWarps)
     __syncwarp();
   }
   if (lane < rows) xn[base + lane] = fma(-omega, s / val[e - 1], x[base + lane]);
+}
+template <int R>
+constexpr int kNkSmem = kNkWarps * R * kNkPitch * (int)sizeof(double2);
+
+// Rows per warp by the number of rows: with few, the launch lasts as long as a
+// warp's loads and chains.  us per sweep with 1, 4, 8 and 32 rows per warp: cloths
+// of 161 rows 6.3, 6.5, 7.8, 13.5, of 2,945 10.7, 10.4, 10.4, 16.5, of 49,408 61.9,
+// 22.6, 16.9, 21.0; beams of 6,125 43.1, 22.9, 24.7, 62.1, of 46,760 262, 96.6, 59.7,
+// 70.6.
+constexpr int kNkFew = 1 << 12, kNkSome = 1 << 16;
+
+template <int R>
+static mgpbd_status nk_sweep(Handle *h, const double *x, double *xn) {
+  const Level &L = h->lev[0];
+  k_nk_sweep<R><<<blocks_covering(h->m, R * kNkWarps), 32 * kNkWarps, kNkSmem<R>, h->stream>>>(
+      h->m, L.ptr, L.col, L.val, h->p.nk_omega, x, xn);
+  MG_LAUNCH("k_nk_sweep");
+  return MGPBD_OK;
 }
 
 // ---------------------------------------------------------------------------
@@ -822,7 +841,6 @@ mgpbd_status level_precision_copies(Handle *h, int l) {
 // first launch there), never per launch: per launch, one thread could lower it
 // between another thread's setting and that thread's launch, which then fails.
 constexpr int kGalerkinSmemMax = 200 * 1024;
-constexpr int kNkSmem = kNkWarps * 32 * kNkPitch * (int)sizeof(double2);
 
 __global__ void k_gal_values_k(int na, int k, const int64_t *mptr, const int32_t *mrow,
                                const int64_t *ptr, const int32_t *col, const double *val,
@@ -837,7 +855,7 @@ static mgpbd_status galerkin_smem_limits() {
   return once(device, []() -> mgpbd_status {
     const cudaFuncAttribute limit = cudaFuncAttributeMaxDynamicSharedMemorySize;
     MG_CUDA(cudaFuncSetAttribute(k_gal_values, limit, kGalerkinSmemMax));
-    MG_CUDA(cudaFuncSetAttribute(k_nk_sweep, limit, kNkSmem));
+    MG_CUDA(cudaFuncSetAttribute(k_nk_sweep<32>, limit, kNkSmem<32>));
     MG_CUDA(cudaFuncSetAttribute(k_gal_values_k, limit, kGalerkinSmemMax));
     return MGPBD_OK;
   });
@@ -1381,9 +1399,9 @@ mgpbd_status amg_setup(Handle *h) {
                                                             amax, xa);
       MG_LAUNCH("k_nk_init");
       for (int s = 0; s < h->p.nk_sweeps; ++s) {
-        k_nk_sweep<<<blocks_covering(h->m, 32 * kNkWarps), 32 * kNkWarps, kNkSmem, h->stream>>>(
-            h->m, L0.ptr, L0.col, L0.val, h->p.nk_omega, xa, xb);
-        MG_LAUNCH("k_nk_sweep");
+        MG_TRY(h->m <= kNkFew ? nk_sweep<4>(h, xa, xb)
+                              : (h->m <= kNkSome ? nk_sweep<8>(h, xa, xb)
+                                                 : nk_sweep<32>(h, xa, xb)));
         MG_CUDA(cudaMemcpyAsync(xa, xb, sizeof(double) * h->m, cudaMemcpyDeviceToDevice,
                                 h->stream));
       }

@@ -120,3 +120,17 @@ def test_setup_bits_on_ragged_sizes(make):
             for a, b in zip(o.level_agg(l)[1:], g.level_agg(l)[1:]):
                 assert np.array_equal(a, b), l
             assert g.level_omega(l) == pytest.approx(o.level_omega(l), rel=1e-10)
+
+
+@pytest.mark.parametrize("rows", [1, 3, 4, 5, 31, 4095, 4096, 4097, 65535, 65536, 65537])
+def test_near_kernel_bits_at_rows_per_warp(rows):
+    """4 rows per warp up to 4,096, 8 up to 65,536, then 32: the near-kernel
+    vector is the oracle's, bit for bit, on every side."""
+    mesh = cut_cloth(rows)
+    p = default_params(coarse_max=400)
+    o, g = Oracle(mesh, p, omp=True), solver(mesh, p)
+    for s in (o, g):
+        s.begin_frame()
+        s.eval_assemble()
+        s.prepare_solve()
+    assert np.array_equal(o.level_agg(0)[4], g.level_agg(0)[4])

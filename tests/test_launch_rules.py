@@ -28,9 +28,9 @@ def launch(kernel, source):
 
 
 def test_near_kernel_sweep_covers_every_row(tmp_path):
-    """One warp takes 32 rows and does not loop: 2^20 blocks of 128 rows would
-    stop at row 134,217,728."""
-    assert launch("k_nk_sweep", "setup.cu").startswith("blocks_covering(h->m, 32 * kNkWarps)")
+    """One warp takes 4 to 32 rows and does not loop: 2^20 blocks of 128 rows
+    would stop at row 134,217,728."""
+    assert launch("k_nk_sweep<R>", "setup.cu").startswith("blocks_covering(h->m, R * kNkWarps)")
     out = run_host(tmp_path, """
   for (long long n : {1LL, 31LL, 128LL, 129LL, (1LL << 27), (1LL << 27) + 1, (1LL << 31) - 1})
     printf("%lld %d\\n", n, blocks_covering(n, 128));""")
