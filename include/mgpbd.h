@@ -313,8 +313,9 @@ mgpbd_status mgpbd_get_lambda(mgpbd_handle_t *h, double *lambda, double *dlambda
 
 /* ---- measurement ----
  * mgpbd_profile(h, enable) with enable a mask: bit 0 (1) records a CUDA event
- * pair around every level-0 smoother sweep (one CSR launch, or the vertex and
- * row passes of the matrix-free sweep) (the dominant kernel of the V-cycle,
+ * pair around every plain level-0 smoother sweep (one CSR launch, or the vertex
+ * and row passes of the matrix-free sweep; not the sweep from zero, nor those
+ * that take the prolongation along or write z) (the dominant kernel of the V-cycle,
  * Sec. 5.2 of the paper: the V-cycle takes most of an iteration and the
  * smoother most of the V-cycle); bit 1 (2) around every A.p of the PCG
  * recurrence (read with mgpbd_profile_read_ap); 0 stops.  Each event pair

@@ -1809,12 +1809,11 @@ static mgpbd_status vcycle_level(Handle *h, int l, const T *b_in, T **res, bool 
   }
   int s = 0;  // post-smoothing sweeps done
   if (jac && nk == 1 && !mf && fuse_prolong<T>(L) && (sweeps > 1 || !top)) {
-    // the first sweep takes the prolongation with it
-    if (l == 0) MG_TRY(prof_begin(h));
+    // the first sweep takes the prolongation with it (more bytes than the timed
+    // sweeps: not one of them, and neither is the last, which writes z)
     DISPATCH_G(G, MG_TRY(rows_launch(h, "k_jacobi_prolong", k_jacobi_prolong<GG, T>, n, GG, n,
                                      L.ptr, L.col, val, dinv, om, b_in, L.agg, Ps<T>(L), xc, x,
                                      x2, sc)));
-    if (l == 0) MG_TRY(prof_end(h));
     std::swap(x, x2);
     s = 1;
   } else if (nk == 1) {
@@ -1836,7 +1835,6 @@ static mgpbd_status vcycle_level(Handle *h, int l, const T *b_in, T **res, bool 
       MG_TRY(mf_level0_final<T>(h, x, b_in, dinv, om, *top));
       break;
     }
-    MG_TRY(prof_begin(h));
     DISPATCH_G(G, DISPATCH_EARLY(early_rows<T>(L), {
       if constexpr (sizeof(T) == 8 && !EE) {
         // z is the sweep's own output here; with the dot product in it the
@@ -1853,7 +1851,6 @@ static mgpbd_status vcycle_level(Handle *h, int l, const T *b_in, T **res, bool 
                             top->c));
       }
     }));
-    MG_TRY(prof_end(h));
   }
   if (z_written) *z_written = zw;
   *res = x;

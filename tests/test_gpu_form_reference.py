@@ -203,3 +203,19 @@ def test_last_iteration_leaves_the_vcycle_out():
     cycle, product, solve = best(lambda: g.vcycle(r)), best(lambda: g.apply(r)), best(lambda: g.solve(r))
     g.close()
     assert solve <= 1.5 * cycle + 2 * product, (solve, cycle, product)
+
+
+@pytest.mark.parametrize("rows,per_cycle", [(9000, 1), (80000, 2)])
+def test_profile_times_plain_sweeps_only(rows, per_cycle):
+    """The sweep channel's bytes per launch are those of a plain CSR sweep, so
+    the sweep that takes the prolongation along (up to 786,432 entries) and the
+    one that writes z are not timed: of the three sweeps behind the one from
+    zero, one and two are."""
+    g = ready(cut_cloth(rows), precision=1, pcg_rtol=1e-300, pcg_maxiter=10)
+    b = torch.ones(rows, dtype=torch.float64, device="cuda")
+    g.profile(True)
+    _, info = g.solve(b)
+    assert info["pcg_iters"] == 10
+    # the cycles before each iteration's end but the last one's
+    assert g.profile_read()["launches"] == 10 * per_cycle
+    g.close()
