@@ -393,9 +393,9 @@ static mgpbd_status create(const mgpbd_mesh_desc *md, const mgpbd_params *p, voi
   CK(alloc_n(h->arena, &h->pp, (size_t)m));
   CK(alloc_n(h->arena, &h->pq, (size_t)m));
   CK(alloc_n(h->arena, &h->sc, 1));
-  CK(alloc_n(h->arena, &h->partials, 4096 + 16));
-  CK(alloc_n(h->arena, &h->part_pq, 4096));
-  CK(alloc_n(h->arena, &h->part_rz, 4096));
+  CK(alloc_n(h->arena, &h->partials, kPartials + 16));
+  CK(alloc_n(h->arena, &h->part_pq, kPartials));
+  CK(alloc_n(h->arena, &h->part_rz, kPartials));
   CK(alloc_n(h->arena, &h->counter, 16));
   CK(alloc_n(h->arena, &h->gbar, 16));
   CK(alloc_n(h->arena, &h->flag, 16));

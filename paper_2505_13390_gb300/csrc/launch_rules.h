@@ -17,6 +17,16 @@ inline int blocks_covering(int64_t rows, int rows_per_block) {
   return (int)(b < 1 ? 1 : b);
 }
 
+// Block partials that each of a handle's reductions has room for, and the blocks
+// of a kernel that leaves one each: at most one resident wave of them, and never
+// more than there is room for, whatever the part's number of SMs.
+constexpr int kPartials = 4096;
+inline int partial_blocks(int64_t blocks, int64_t resident) {
+  int64_t b = blocks < resident ? blocks : resident;
+  if (b > kPartials) b = kPartials;
+  return (int)(b < 1 ? 1 : b);
+}
+
 // A setting that the runtime keeps per device (a kernel's shared-memory limit,
 // for one) and that is made once: `f` runs for each device until it has
 // succeeded there (a status >= 0), one thread at a time.

@@ -54,7 +54,7 @@ constexpr int kVertexThreads = 64;
 // The early forms have one thread per row and one group per vertex, without a
 // loop: the vertices are limited too, and a pass with a dot product, which
 // leaves one partial per block, by the partials the handle holds.
-constexpr int kEarlyDotRows = 4096 * kDotThreads;
+constexpr int kEarlyDotRows = kPartials * kDotThreads;
 template <class T>
 static bool early(const Handle *h, bool dot = false) {
   const int rows = sizeof(T) == 8 ? kEarlyRows64 : kEarlyRows32;
@@ -780,7 +780,7 @@ template <class T, int MODE>
 static int mf_dot_grid(const Handle *h) {
   const int blocks = blocks_for(h->m, kDotThreads);
   if (early<T>(h, true)) return blocks;  // one row per thread, as mf_row_launch has it
-  return std::min(blocks, wave_blocks((const void *)k_mf_row<T, MODE>, kDotThreads));
+  return dot_blocks(blocks, (const void *)k_mf_row<T, MODE>);
 }
 
 template <class T, int MODE>
@@ -1039,9 +1039,7 @@ mgpbd_status mf_apply_pq_form(Handle *h, bool pairs, const double *p, double *q,
                               const DotCtx &c) {
   if (pairs) {
     MG_TRY(mf_vertex(h, (const float2 *)h->p_df));
-    const int grid =
-        std::min((h->m + kDotThreads - 1) / kDotThreads,
-                 wave_blocks((const void *)k_mf_row_df, kDotThreads));
+    const int grid = dot_blocks(blocks_for(h->m, kDotThreads), (const void *)k_mf_row_df);
     h->n_pq = grid;
     MG_TRY(chain_launch(h, "k_mf_row_df(A.p)", k_mf_row_df, grid, kDotThreads, h->E, h->m,
                         h->edge, h->tet,

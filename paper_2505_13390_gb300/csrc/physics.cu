@@ -536,7 +536,7 @@ mgpbd_status launch_update(Handle *h, mgpbd_solve_info *info) {
   }
   MG_CUDA(cudaMemcpyAsync(h->xbak, h->x, sizeof(double) * n3, cudaMemcpyDeviceToDevice,
                           h->stream));
-  double *d_nb = h->partials + 4096 + 4;  // scratch scalar after the dot partials
+  double *d_nb = h->partials + kPartials + 4;  // scratch scalar after the dot partials
   double nb = 0.0;
   for (int t = 0; t <= h->p.backtrack; ++t) {
     k_apply_x<<<blocks_for(n3, 256), 256, 0, h->stream>>>(n3, om, h->dx, h->xbak, h->x);

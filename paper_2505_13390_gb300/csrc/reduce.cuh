@@ -358,6 +358,11 @@ __device__ __forceinline__ void behind_gate(const PcgScalars *sc, F body,
 #define VG_WARPS(vb, vn)                                                          \
   ((int64_t)(vb) * blockDim.x + threadIdx.x) >> 5, ((int64_t)(vn) * blockDim.x) >> 5
 
+// blocks of a kernel of kDotThreads that leaves one partial per block
+inline int dot_blocks(int64_t blocks, const void *kernel) {
+  return partial_blocks(blocks, wave_blocks(kernel, kDotThreads));
+}
+
 // the test on r.r for the launch being made, if one is due
 inline RRTest take_rr_test(Handle *h) {
   RRTest t;

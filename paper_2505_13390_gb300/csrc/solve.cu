@@ -27,11 +27,11 @@
 namespace mg {
 
 // blocks of a dot-product kernel over n entries: two entries per thread up to
-// four blocks per SM, then about eight; at most the 4096 partials the handle holds
-static int dot_grid(int64_t n) {
+// four blocks per SM, then about eight
+static int64_t dot_grid(int64_t n) {
   const int64_t two = (n + 2 * kDotThreads - 1) / (2 * kDotThreads);
   const int64_t more = std::max<int64_t>(4 * num_sms(), (n + 1023) / 1024);
-  return (int)std::min<int64_t>(4096, std::max<int64_t>(1, std::min(two, more)));
+  return std::max<int64_t>(1, std::min(two, more));
 }
 
 static DotCtx make_ctx(Handle *h, int mode, double *out = nullptr) {
@@ -1064,13 +1064,12 @@ static bool fuse_prolong(const Level &L) {
 // grids of the kernels that end in a dot product: one resident wave at most
 template <int G, bool EARLY>
 static int spmv_pq_blocks(int m) {
-  return std::min(row_blocks(m, G, kDotThreads),
-                  wave_blocks((const void *)k_spmv_pq<G, double, double, EARLY>, kDotThreads));
+  return dot_blocks(row_blocks(m, G, kDotThreads),
+                    (const void *)k_spmv_pq<G, double, double, EARLY>);
 }
 template <int G, class T, bool EARLY>
 static int jacobi_final_blocks(int n) {
-  return std::min(row_blocks(n, G, kDotThreads),
-                  wave_blocks((const void *)k_jacobi_final<G, T, EARLY>, kDotThreads));
+  return dot_blocks(row_blocks(n, G, kDotThreads), (const void *)k_jacobi_final<G, T, EARLY>);
 }
 // p update: four entries per thread; on large instances two large blocks per SM,
 // which loop.  With up to sixteen blocks of 128 threads per SM, each adding 1,500
@@ -1085,7 +1084,7 @@ static int p_blocks(int m, int threads) {
 }
 template <class T>
 static int xr_blocks(int m) {
-  return std::min(dot_grid(m), wave_blocks((const void *)k_xr_update<T>, kDotThreads));
+  return dot_blocks(dot_grid(m), (const void *)k_xr_update<T>);
 }
 
 #define DISPATCH_G(G, ...)                  \
@@ -1676,7 +1675,7 @@ static mgpbd_status rows_launch(Handle *h, const char *what, void (*k)(P...), in
 static mgpbd_status launch_dot(Handle *h, const double *x, const double *y, int64_t n, int mode,
                                int check_done, double *out = nullptr) {
   const DotCtx c = mode == DOT_PART ? rz_ctx(h) : make_ctx(h, mode, out);
-  const int blocks = std::min(dot_grid(n), wave_blocks((const void *)k_dot, kDotThreads));
+  const int blocks = dot_blocks(dot_grid(n), (const void *)k_dot);
   if (mode == DOT_PART) h->n_rz = blocks;
   return chain_launch(h, "k_dot", k_dot, blocks, kDotThreads, n, x, y, c, check_done);
 }
@@ -2114,9 +2113,7 @@ mgpbd_status pcg_solve(Handle *h, const double *b, double *x, mgpbd_solve_info *
 mgpbd_status pcg_finish(Handle *h, const double *b, double *x, mgpbd_solve_info *info) {
   const int m = h->m;
   memset(info, 0, sizeof(*info));
-  k_true_resid<<<std::min(row_blocks(m, 4, kDotThreads),
-                          wave_blocks((const void *)k_true_resid, kDotThreads)),
-                 kDotThreads, 0, h->stream>>>(
+  k_true_resid<<<dot_blocks(row_blocks(m, 4, kDotThreads), (const void *)k_true_resid), kDotThreads, 0, h->stream>>>(
       m, h->lev[0].ptr, h->lev[0].col, h->lev[0].val, x, b, make_ctx(h, DOT_TR));
   MG_LAUNCH("k_true_resid");
   MG_CUDA(cudaMemcpyAsync(h->sc_host, h->sc, sizeof(PcgScalars), cudaMemcpyDeviceToHost,
@@ -2164,7 +2161,7 @@ mgpbd_status evict_l2(Handle *h) {
   const int64_t n = std::min<int64_t>(L.nnz / 2, (256ll << 20) / 16);
   if (n <= 0 || !L.val) return MGPBD_OK;
   k_evict<<<std::min<int64_t>(4 * num_sms(), (n + 255) / 256), 256, 0, h->stream>>>(
-      reinterpret_cast<const ulonglong2 *>(L.val), n, reinterpret_cast<int *>(h->partials + 4096 + 15));
+      reinterpret_cast<const ulonglong2 *>(L.val), n, reinterpret_cast<int *>(h->partials + kPartials + 15));
   MG_LAUNCH("k_evict");
   return MGPBD_OK;
 }
@@ -2279,7 +2276,7 @@ mgpbd_status xpbd_step(Handle *h, mgpbd_solve_info *info) {
   memset(info, 0, sizeof(*info));
   if (h->m == 0) return MGPBD_OK;
   const Level &L = h->lev[0];
-  double *d_bn = h->partials + 4096 + 6;
+  double *d_bn = h->partials + kPartials + 6;
   MG_TRY(dot_dd(h, h->b, h->b, h->m, d_bn));
   k_xpbd_step<<<blocks_for(h->m, 256), 256, 0, h->stream>>>(h->m, L.ptr, L.val, h->b, h->dl);
   MG_LAUNCH("k_xpbd_step");
@@ -2342,13 +2339,12 @@ mgpbd_status power_method(Handle *h, int l) {
   const int n = L.n;
   double *y = h->pp, *z = h->pq;
   double *part[2] = {h->part_pq, h->part_rz};
-  int np = std::min(blocks_for(n, kDotThreads), 4 * num_sms());
+  int np = partial_blocks(blocks_for(n, kDotThreads), 4 * num_sms());
   k_pow_init<<<np, kDotThreads, 0, h->stream>>>(n, h->p.seed_pow, l, y, part[0]);
   MG_LAUNCH("k_pow_init");
   // four lanes per row, the fewest FP64 additions in the fold: setup of a 46,760-row
   // beam of long rows takes 3.38 ms, 3.50 with eight
-  const int blocks = std::min(row_blocks(n, 4, kDotThreads),
-                              wave_blocks((const void *)k_pow_step, kDotThreads));
+  const int blocks = dot_blocks(row_blocks(n, 4, kDotThreads), (const void *)k_pow_step);
   for (int it = 0; it < h->p.power_iters; ++it) {
     k_pow_step<<<blocks, kDotThreads, 0, h->stream>>>(n, L.ptr, L.col, L.val, y, part[it & 1], np,
                                                      z, part[(it & 1) ^ 1]);
@@ -2356,7 +2352,7 @@ mgpbd_status power_method(Handle *h, int l) {
     np = blocks;
     std::swap(y, z);
   }
-  double *d_lam = h->partials + 4096 + 2;  // a scalar after the partials
+  double *d_lam = h->partials + kPartials + 2;  // a scalar after the partials
   k_pow_lambda<<<1, kDotThreads, 0, h->stream>>>(part[h->p.power_iters & 1], np, d_lam);
   MG_LAUNCH("k_pow_lambda");
   double lam = 0.0;

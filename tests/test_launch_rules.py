@@ -59,6 +59,24 @@ def test_settings_are_made_on_each_device(tmp_path):
     assert out[0] == "1 1 1 1 1 2"
 
 
+def test_partials_never_exceed_their_room(tmp_path):
+    """The grid of every kernel that leaves one partial per block goes through
+    the rule, which holds on a part of any number of SMs."""
+    out = run_host(tmp_path, """
+  for (long long blocks : {0LL, 1LL, 4095LL, 4096LL, 4097LL, 1LL << 40})
+    for (long long resident : {1LL, 2432LL, 4096LL, 100000LL})
+      printf("%lld %lld %d\\n", blocks, resident, partial_blocks(blocks, resident));
+  printf("%d\\n", kPartials);""")
+    room = int(out[24])
+    for blocks, resident, got in (map(int, line.split()) for line in out[:24]):
+        assert got == max(1, min(blocks, resident, room))
+    for name in ("solve.cu", "mfree.cu"):
+        src = open(os.path.join(CSRC, name)).read()
+        # kernels of kDotThreads are those that leave partials
+        assert not re.search(r"wave_blocks\([^;]*kDotThreads\)", src), name
+    assert "&h->partials, kPartials + 16" in open(os.path.join(CSRC, "api.cu")).read()
+
+
 @pytest.mark.gpu
 def test_near_kernel_beyond_two_to_the_27_rows():
     """A chain of 2^27 + 3,000 rows whose rows are dead (both ends pinned) but
