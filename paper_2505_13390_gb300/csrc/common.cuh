@@ -86,9 +86,7 @@ inline mgpbd_status alloc_n(Arena &a, T **p, size_t n) {
 struct PcgScalars {
   double bnorm2;   // |b|^2
   double rz[2];    // r.z; iteration k's is in rz[k & 1]
-  double pq;       // p.q
   double rr;       // r.r
-  double alpha, beta;
   double tr2;      // |b - A x|^2 (true residual)
   double thr2;     // (rtol |b|)^2: r.r at or below it has converged
   int done;        // 1 once converged or failed

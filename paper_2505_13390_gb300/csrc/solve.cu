@@ -2,13 +2,13 @@
 // weighted-Jacobi smoother, restriction/prolongation through the aggregates,
 // the coarsest dense Cholesky, and the power method for lambda_max(D^-1 A).
 //
-// Scalars of the PCG recurrence (r.z, p.q, alpha, beta, |r|) stay on the
-// device: a dot product leaves one partial per block, and every block of the
-// kernel that needs it (x/r update, p update) folds the partials in one fixed
-// order, so results are deterministic run to run and no host round trip is
-// needed inside an iteration.  Kernels of an iteration return at once when the
-// device flag `done` is set, so the host launches iterations in chunks and
-// reads the flag once per chunk.
+// The PCG recurrence stays on the device (r.z, r.r, the iteration counts and the
+// status in PcgScalars; alpha and beta in the kernels that use them): a dot
+// product leaves one partial per block, and every block of the kernel that needs
+// it (x/r update, p update) folds the partials in one fixed order, so results are
+// deterministic run to run and no host round trip is needed inside an iteration.
+// Kernels of an iteration return at once when the device flag `done` is set, so
+// the host launches iterations in chunks and reads the flag once per chunk.
 //
 // Precision: MGPBD_FP64 runs everything in FP64.  MGPBD_MIXED runs the
 // V-cycle bulk (smoothing, residuals, restriction, prolongation) with FP32
@@ -131,9 +131,7 @@ __device__ __forceinline__ void xr_update_body(int vb, int vn, int64_t n, double
     sh_ok = pq > 0.0;
     sh_al = rz / pq;
     if (vb == 0 && !gate.closed()) {
-      sc->pq = pq;
       if (pq > 0.0) {
-        sc->alpha = sh_al;
         sc->iters = it + 1;
       } else {
         sc->status = MGPBD_E_BREAKDOWN;
@@ -246,7 +244,6 @@ __device__ __forceinline__ void p_update_body(int vb, int vn, int64_t n, double 
       if (n_rr) sc->rr = rr;
       if (go) {
         sc->rz[it & 1] = rz;
-        sc->beta = sh_be;
         sc->p_updates = it;
       } else {
         sc->status = st;
@@ -298,7 +295,7 @@ __global__ void k_pcg_init(PcgScalars *sc, unsigned int *bar) {
   sc->iters = sc->p_updates = 0;
   sc->thr2 = 0.0;
   sc->status = MGPBD_W_NOT_CONVERGED;
-  sc->rz[0] = sc->rz[1] = sc->pq = sc->rr = sc->alpha = sc->beta = sc->tr2 = 0.0;
+  sc->rz[0] = sc->rz[1] = sc->rr = sc->tr2 = 0.0;
 }
 
 template <class D>
