@@ -997,12 +997,12 @@ static mgpbd_status mf_vertex(Handle *h, const float2 *x, int G = 0, bool check_
   return MGPBD_OK;
 }
 
-// Times the vertex pass with 4, 8 and, in FP32, 16 lanes per vertex in each
-// precision the solve uses and keeps the fastest (params.autotune); with
-// ap_split the A.p's lanes are timed on its pair form.  Sixteen FP64 lanes
-// never pay beyond the timing of one pass: they add as often as they multiply
-// (five additions per lane for two incidences of a tet vertex), which takes
-// FP64 issue slots from every kernel beside it.
+// Times the vertex pass with 4, 8 and 16 lanes per vertex in each precision the
+// solve uses and keeps the fastest (params.autotune).  Sixteen FP64 lanes pay on
+// small tet instances (48 FP64 iterations on a beam of 6,125 rows take 2.26 ms,
+// 2.50 with eight and 3.14 with four; on 46,760 rows 6.06, 5.98 and 6.54).  With
+// ap_split the A.p's lanes are timed on its pair form, with four and eight: sixteen
+// gain at most 0.3% there (2.13 and 2.13 ms on 6,125 rows) and lose 8% on 30,506.
 mgpbd_status mf_autotune(Handle *h) {
   if (h->m == 0 || !h->vslot) return MGPBD_OK;
   auto pick = [&](auto *x, int n_cands, int *out) -> mgpbd_status {
@@ -1028,7 +1028,7 @@ mgpbd_status mf_autotune(Handle *h) {
   if (h->p.ap_split)
     MG_TRY(pick((const float2 *)h->p_df, 2, &h->mf_g64));
   else
-    MG_TRY(pick((const double *)h->pr, 2, &h->mf_g64));
+    MG_TRY(pick((const double *)h->pr, 3, &h->mf_g64));
   if (h->p.precision == MGPBD_MIXED) MG_TRY(pick((const float *)h->lev[0].b, 3, &h->mf_g32));
   return MGPBD_OK;
 }

@@ -219,3 +219,13 @@ def test_profile_times_plain_sweeps_only(rows, per_cycle):
     # the cycles before each iteration's end but the last one's
     assert g.profile_read()["launches"] == 10 * per_cycle
     g.close()
+
+
+def test_autotuner_times_sixteen_fp64_lanes():
+    """On a beam of 6,125 rows the FP64 vertex pass is fastest with sixteen
+    lanes per vertex (its lists hold about thirty rows), and so are whole
+    solves: the autotuner has to try them."""
+    mesh = hex_block(5, 10, 10, h=0.01, alpha=1e-8, pin="x0", seed=1)
+    g = ready(mesh, precision=0, level0_op=1, autotune=1)
+    assert g.lanes(0)["vert64"] == 16
+    g.close()
