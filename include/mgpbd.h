@@ -109,7 +109,7 @@ typedef struct {
                            future-work direction, Sec. 6).  Setup and Galerkin
                            products always use the assembled matrix. */
   int use_graphs;       /* 1: capture chunks of 8 PCG iterations into a CUDA graph and
-                           replay it (one launch instead of ~40 per iteration; the
+                           replay it (one launch instead of 9 to 51 per iteration; the
                            graph is re-captured after each setup); 0: plain launches.
                            Needs a stream of the caller's own: on the legacy default
                            stream (NULL) launches stay plain. */

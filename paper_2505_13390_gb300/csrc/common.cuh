@@ -261,7 +261,8 @@ mgpbd_status prof_harvest(Handle *h, int iters);
 // ---------------------------------------------------------------------------
 // launch chains (programmatic dependent launch)
 // ---------------------------------------------------------------------------
-// A PCG iteration is a chain of 15 to 35 dependent kernels, most of them a few
+// A PCG iteration is a chain of 9 (two CSR levels) to 31 (the 1.65M-tet block) and
+// 51 (five levels, Chebyshev) dependent kernels, most of them a few
 // microseconds long.  Launched through chain_launch, a kernel's blocks become
 // resident as soon as its predecessor's have finished, before the
 // predecessor's memory flush and without the launch gap; chain_wait() holds

@@ -45,9 +45,10 @@ constexpr int kUStride = 3, kUStrideDf = 4;
 // on 195,585 rows 5.07 / 5.30, 689,281 12.90 / 13.29, 925,033 13.52 / 13.69,
 // 938,561 16.16 / 16.40, 1,226,241 20.60 / 19.84.
 constexpr int kEarlyRows32 = 1 << 20, kEarlyRows64 = 1 << 17;
-// tet instances of up to this many rows start with eight FP64 lanes per vertex:
-// a beam's frame takes 191 ms, 201 with four lanes and unfused prolongations;
-// on 3.7M rows A.p takes 224 us with eight and 213 with four
+// tet instances of up to this many rows start with eight FP64 lanes per vertex.
+// 48 mixed iterations with eight, and with four: 2.68 / 3.03 ms on 30,506 rows of
+// beam, 4.08 / 4.20 on 93,200; 4.38 / 4.08 on 150,433 rows of block; on 3.7M rows
+// A.p takes 224 us with eight and 213 with four
 constexpr int kShortListRows = 1 << 17;
 // threads of the early vertex passes: small blocks, for more SMs (reduce.cuh)
 constexpr int kVertexThreads = 64;
@@ -770,7 +771,8 @@ mgpbd_status mf_create(Handle *h) {
 // the 3.68M-row block (14,375 blocks of rows) the cap measured 0.7% faster
 // per PCG iteration than 4,096 blocks and 2% faster than one block per 256
 // rows.
-// (the passes that end in a dot product run one resident wave of kDotThreads)
+// (the plain passes that end in a dot product run one resident wave of kDotThreads,
+// the early ones one block per kDotThreads rows)
 static int mf_grid(int64_t rows, int threads) {
   return (int)std::max<int64_t>(1, std::min<int64_t>((rows + threads - 1) / threads, 8192));
 }

@@ -2023,7 +2023,7 @@ mgpbd_status pcg_solve(Handle *h, const double *b, double *x, mgpbd_solve_info *
   const int chunk = 8;
   int launched = 0;
   // Chunks of PCG iterations replay a captured CUDA graph (one launch instead
-  // of ~33 per iteration); the graph is re-captured when the hierarchy, the
+  // of 9 to 51 per iteration); the graph is re-captured when the hierarchy, the
   // output array or the profiling switch changes.  With profiling on, the
   // graph carries event-record nodes around the level-0 sweeps, read back
   // after every replay.
