@@ -1985,9 +1985,10 @@ static mgpbd_status pcg_iteration(Handle *h, double *x) {
                         jac ? (double *)L.x : nullptr));
   h->rr_test = !gs && hosts_rr_test(h);
   const bool due = h->rr_test;
-  MG_TRY(vcycle_top(h, r, z, true, DOT_PART));
+  const mgpbd_status vs = vcycle_top(h, r, z, true, DOT_PART);
   const bool tested = due && !h->rr_test;
   h->rr_test = false;
+  MG_TRY(vs);
   const int th = p_threads(m);
   MG_TRY(chain_launch(h, "k_p_update", th > kDotThreads ? k_p_update<true> : k_p_update<false>,
                       p_blocks(m, th), th, m, p, z, h->sc,
