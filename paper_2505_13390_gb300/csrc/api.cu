@@ -70,8 +70,9 @@ mgpbd_status prof_end(Handle *h, int ch) {
 }
 
 // Whether the timed launch of PCG iteration `it` counts in a solve that took
-// `iters` iterations.  Convergence is tested at an iteration's end, so the last
-// one's V-cycle runs as well, but nothing uses it: its sweeps are left out.
+// `iters` iterations.  Convergence is tested behind the x/r update, so the last
+// iteration's V-cycle runs as a whole or in part, but nothing uses it: its sweeps
+// are left out.
 static bool prof_ran(int ch, int it, int iters) {
   return ch == PROF_AP ? it <= iters - 1 : it <= iters - 2;
 }

@@ -6,8 +6,11 @@
 // device (dot_finalize).  Results are therefore identical run to run.  The dot
 // products of the recurrence leave only their partials (DOT_PART): every block
 // of the kernel that needs them (p.q: the x/r update; r.r and r.z: the p
-// update) folds them itself, in the same order, which costs it less than the
-// fence, counter and re-read of a last block cost the kernel before.
+// update) folds them itself, in the same order.  On small instances that costs it
+// less than the fence, counter and re-read of a last block cost the kernel
+// before; on large ones it is one FP64 addition per partial and block, so the
+// consumer has few blocks (p update) or the fold is done once beside other work
+// (rr_test).
 #pragma once
 
 #include "common.cuh"

@@ -285,8 +285,8 @@ template <bool LARGER>
 __global__ void k_p_update(int64_t n, double *p, const double *z, PcgScalars *sc, int maxiter,
                            const double *part_rr, int n_rr, const double *part_rz, int n_rz,
                            float2 *pdf) {
-  p_update_body<LARGER>(blockIdx.x, gridDim.x, n, p, z, sc, maxiter, part_rr, n_rr, part_rz, n_rz, pdf,
-                ChainGate(sc));
+  p_update_body<LARGER>(blockIdx.x, gridDim.x, n, p, z, sc, maxiter, part_rr, n_rr, part_rz, n_rz,
+                        pdf, ChainGate(sc));
 }
 
 __global__ void k_pcg_init(PcgScalars *sc, unsigned int *bar) {
@@ -2111,7 +2111,8 @@ mgpbd_status pcg_solve(Handle *h, const double *b, double *x, mgpbd_solve_info *
 mgpbd_status pcg_finish(Handle *h, const double *b, double *x, mgpbd_solve_info *info) {
   const int m = h->m;
   memset(info, 0, sizeof(*info));
-  k_true_resid<<<dot_blocks(row_blocks(m, 4, kDotThreads), (const void *)k_true_resid), kDotThreads, 0, h->stream>>>(
+  k_true_resid<<<dot_blocks(row_blocks(m, 4, kDotThreads), (const void *)k_true_resid),
+                 kDotThreads, 0, h->stream>>>(
       m, h->lev[0].ptr, h->lev[0].col, h->lev[0].val, x, b, make_ctx(h, DOT_TR));
   MG_LAUNCH("k_true_resid");
   MG_CUDA(cudaMemcpyAsync(h->sc_host, h->sc, sizeof(PcgScalars), cudaMemcpyDeviceToHost,
@@ -2159,7 +2160,8 @@ mgpbd_status evict_l2(Handle *h) {
   const int64_t n = std::min<int64_t>(L.nnz / 2, (256ll << 20) / 16);
   if (n <= 0 || !L.val) return MGPBD_OK;
   k_evict<<<std::min<int64_t>(4 * num_sms(), (n + 255) / 256), 256, 0, h->stream>>>(
-      reinterpret_cast<const ulonglong2 *>(L.val), n, reinterpret_cast<int *>(h->partials + kPartials + 15));
+      reinterpret_cast<const ulonglong2 *>(L.val), n,
+      reinterpret_cast<int *>(h->partials + kPartials + 15));
   MG_LAUNCH("k_evict");
   return MGPBD_OK;
 }
@@ -2172,8 +2174,9 @@ static mgpbd_status time_resid(Handle *h, const Level &L, int G, const T *val, c
   for (int rep = 0; rep < 5; ++rep) {
     MG_TRY(evict_l2(h));
     MG_CUDA(cudaEventRecord(h->ev0, h->stream));
-    DISPATCH_G(G, DISPATCH_EARLY(early_rows<T>(L), k_resid<GG, T, EE><<<row_blocks(n, GG), 256, 0, h->stream>>>(
-                                            n, L.ptr, L.col, val, b, x, r, nullptr, RRTest())));
+    DISPATCH_G(G, DISPATCH_EARLY(early_rows<T>(L),
+                                 k_resid<GG, T, EE><<<row_blocks(n, GG), 256, 0, h->stream>>>(
+                                     n, L.ptr, L.col, val, b, x, r, nullptr, RRTest())));
     MG_LAUNCH("k_resid(tune)");
     MG_CUDA(cudaEventRecord(h->ev1, h->stream));
     MG_CUDA(cudaEventSynchronize(h->ev1));
